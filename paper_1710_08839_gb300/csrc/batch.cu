@@ -63,20 +63,14 @@ __global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<R>::value)
     const int s = native_index(g, lex_index(g, x0, x1, x2, x3), p);
     const int po = 1 - p;
     const typename Fields<R>::vec* psi = G.in[r];
-    cplx<R> acc[12];
-#pragma unroll
-    for (int i = 0; i < 12; ++i) acc[i] = mk<R>(0, 0);
+    cplx<R> acc[12], v[12];
     // one code path for every charge (qhat = 0 gives the phase 1 exactly)
-    dirac_dir<R, true, 0>(g, f, psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
-    dirac_dir<R, true, 1>(g, f, psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
-    dirac_dir<R, true, 2>(g, f, psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
-    dirac_dir<R, true, 3>(g, f, psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
-    cplx<R> v[12], w[12];
-    load_spinor(psi, g.V, s, v);
-    clover_mul<true>(f.C, g.V, s, v, w);
+    dirac_hops<R, true>(g, f, psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
 #pragma unroll
-    for (int i = 0; i < 12; ++i) w[i] = w[i] - R(0.5) * acc[i];
-    store_spinor(G.out[r], g.V, s, w);
+    for (int i = 0; i < 12; ++i) acc[i] = HopScale<R>::value * acc[i];
+    load_spinor(psi, g.V, s, v);
+    clover_mul<true, true>(f.C, g.V, s, v, acc);
+    store_spinor(G.out[r], g.V, s, acc);
 }
 
 template <typename R>
@@ -87,7 +81,7 @@ Fields<float> op_fields<float>(qxd_lattice* lat) {
 }
 template <>
 Fields<double> op_fields<double>(qxd_lattice* lat) {
-    return Fields<double>{nullptr, nullptr, lat->U64, lat->Zq64, lat->C64};
+    return Fields<double>{nullptr, nullptr, lat->W64, lat->C64};
 }
 
 // device buffer for group tables, grown on demand, one per (device, stream)

@@ -253,10 +253,12 @@ __global__ void __launch_bounds__(128) k_clover_build(Geom g, const double* __re
     store_packed(id, il, blk, Ci64, Ci32, V, s);
 }
 
-// z^qhat per link from z = exp(i A) (binary powering; |z| = 1 so z^-n = conj(z^n))
-__global__ void k_link_phases(int n, const double2* __restrict__ Z, int qhat, double2* __restrict__ Zq) {
+// W = -1/2 z^qhat U per link, the link of the FP64 hops: z^qhat from z =
+// exp(i A) by binary powering (|z| = 1, so z^-n = conj(z^n)). i = mu V + site.
+__global__ void k_hop_links(Geom g, const double2* __restrict__ Z, const double2* __restrict__ U, int qhat,
+                            double2* __restrict__ W) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= 4 * g.V) return;
     C64 b = mk(Z[i].x, Z[i].y), r = mk(1.0, 0.0);
     int m = qhat < 0 ? -qhat : qhat;
     while (m) {
@@ -265,7 +267,14 @@ __global__ void k_link_phases(int n, const double2* __restrict__ Z, int qhat, do
         m >>= 1;
     }
     if (qhat < 0) r = conj(r);
-    Zq[i] = make_double2(r.re, r.im);
+    r = -0.5 * r;
+    const int mu = i / g.V, s = i - mu * g.V;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        const size_t k = ((size_t)mu * 9 + e) * g.V + s;
+        const C64 w = r * mk(U[k].x, U[k].y);
+        W[k] = make_double2(w.re, w.im);
+    }
 }
 
 }  // namespace
@@ -280,8 +289,8 @@ int launch_clover_build(qxd_lattice* lat, int* d_bad) {
                                                     lat->C32, lat->Cinv64, lat->Cinv32, d_bad);
     QXD_LAUNCHED("k_clover_build");
     const int nl = 4 * g.V;
-    k_link_phases<<<(nl + 255) / 256, 256, 0, lat->stream>>>(nl, lat->Z64, lat->qhat, lat->Zq64);
-    QXD_LAUNCHED("k_link_phases");
+    k_hop_links<<<(nl + 255) / 256, 256, 0, lat->stream>>>(g, lat->Z64, lat->U64, lat->qhat, lat->W64);
+    QXD_LAUNCHED("k_hop_links");
     return QXD_OK;
 }
 

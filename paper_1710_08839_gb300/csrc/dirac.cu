@@ -41,16 +41,13 @@ __global__ void __launch_bounds__(DW_THREADS, DW_PP_MIN_BLOCKS)
     const int s = native_index(g, lex_index(g, x0, x1, x2, x3), p);
     int nb[8];
     neighbours8(g, x0, x1, x2, x3, 1 - p, nb);
-    cplx<float> acc[12];
-#pragma unroll
-    for (int i = 0; i < 12; ++i) acc[i] = mk(0.f, 0.f);
+    cplx<float> acc[12], v[12];
     hops_pipelined<QNZ>(f, g.V, s, nb, q, acc);
-    cplx<float> v[12], w[12];
-    load_spinor(f.psi, g.V, s, v);
-    clover_mul<true>(f.C, g.V, s, v, w);
 #pragma unroll
-    for (int i = 0; i < 12; ++i) w[i] = w[i] - 0.5f * acc[i];
-    store_spinor_cs(f.out, g.V, s, w);
+    for (int i = 0; i < 12; ++i) acc[i] = HopScale<float>::value * acc[i];
+    load_spinor(f.psi, g.V, s, v);
+    clover_mul<true, true>(f.C, g.V, s, v, acc);
+    store_spinor_cs(f.out, g.V, s, acc);
 }
 
 template <typename R, bool QNZ>
@@ -63,20 +60,14 @@ __global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<R>::value)
     const int p = (x0 + x1 + x2 + x3) & 1;
     const int s = native_index(g, lex_index(g, x0, x1, x2, x3), p);
     const int po = 1 - p;
-    cplx<R> acc[12];
+    cplx<R> acc[12], v[12];
+    dirac_hops<R, QNZ>(g, f, f.psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
 #pragma unroll
-    for (int i = 0; i < 12; ++i) acc[i] = mk<R>(0, 0);
-    dirac_dir<R, QNZ, 0>(g, f, f.psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
-    dirac_dir<R, QNZ, 1>(g, f, f.psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
-    dirac_dir<R, QNZ, 2>(g, f, f.psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
-    dirac_dir<R, QNZ, 3>(g, f, f.psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
-    cplx<R> v[12], w[12];
+    for (int i = 0; i < 12; ++i) acc[i] = HopScale<R>::value * acc[i];
     load_spinor(f.psi, g.V, s, v);
-    clover_mul<true>(f.C, g.V, s, v, w);
-#pragma unroll
-    for (int i = 0; i < 12; ++i) w[i] = w[i] - R(0.5) * acc[i];
-    if constexpr (sizeof(R) == 4) store_spinor_cs(f.out, g.V, s, w);
-    else store_spinor(f.out, g.V, s, w);
+    clover_mul<true, true>(f.C, g.V, s, v, acc);
+    if constexpr (sizeof(R) == 4) store_spinor_cs(f.out, g.V, s, acc);
+    else store_spinor(f.out, g.V, s, acc);
 }
 
 // lexicographic [site][spin][colour][re,im] <-> native structure of arrays
@@ -133,9 +124,8 @@ int launch_dirac_shape(qxd_lattice* lat, void* out, const void* in, int prec, co
             else k_dirac<float, false><<<blocks, sh.threads, 0, st>>>(g, f, 0.f, x0b, nx0, n);
         }
     } else {
-        Fields<double> f{(const double2*)in, (double2*)out, lat->U64, lat->Zq64, lat->C64};
-        if (qnz) k_dirac<double, true><<<blocks, sh.threads, 0, st>>>(g, f, (double)lat->qhat, x0b, nx0, n);
-        else k_dirac<double, false><<<blocks, sh.threads, 0, st>>>(g, f, 0.0, x0b, nx0, n);
+        Fields<double> f{(const double2*)in, (double2*)out, lat->W64, lat->C64};
+        k_dirac<double, false><<<blocks, sh.threads, 0, st>>>(g, f, 0.0, x0b, nx0, n);  // charge in the links
     }
     QXD_LAUNCHED("k_dirac");
     return QXD_OK;

@@ -41,9 +41,17 @@ struct Fields<double> {
     using cvec = double;
     const double2* __restrict__ psi;
     double2* __restrict__ out;
-    const double2* __restrict__ U;  // [4][9][V]
-    const double2* __restrict__ A;  // [4][V] z = exp(i A) as (cos A, sin A)
+    const double2* __restrict__ U;  // [4][9][V] W = -1/2 z^qhat U
     const double* __restrict__ C;   // [72][V]
+};
+
+// Factor that turns the raw sum of hops into H psi. The FP64 links are
+// compound, W = -1/2 z^qhat U, so a hop needs neither the U(1) phase (24 of
+// its instructions) nor the factor; the FP32 links are the SU(3) link, with
+// the phase from the angle.
+template <typename R>
+struct HopScale {
+    static constexpr R value = sizeof(R) == 4 ? R(-0.5) : R(1);
 };
 
 // ---------------------------------------------------------------------------
@@ -105,13 +113,11 @@ __device__ __forceinline__ void load_link(const double2* __restrict__ U, int V, 
     }
 }
 
-// U(1) factor z(x,mu)^qhat of the hopping term.
-// FP32: from the stored angle, exp(i qhat A). The argument is reduced to
-// [-pi, pi] (|A| <= pi, so only a few periods are removed) and evaluated with
-// the hardware approximation __sincosf, whose absolute error there is ~1e-6,
-// well inside the FP32 tolerance of the operator.
-// FP64: z^qhat stored per operator (built with the clover term from
-// z = (cos A, sin A) by binary powering).
+// U(1) factor z(x,mu)^qhat of the FP32 hopping term, from the stored angle:
+// exp(i qhat A). The argument is reduced to [-pi, pi] (|A| <= pi, so only a
+// few periods are removed) and evaluated with the hardware approximation
+// __sincosf, whose absolute error there is ~1e-6, well inside the FP32
+// tolerance of the operator.
 __device__ __forceinline__ cplx<float> link_phase(const float4* __restrict__ A, int V, int mu, int s, float q) {
     float t = q * reinterpret_cast<const float*>(A + s)[mu];
     const float k = rintf(t * 0.15915494309189535f);
@@ -119,10 +125,6 @@ __device__ __forceinline__ cplx<float> link_phase(const float4* __restrict__ A, 
     float sn, cs;
     __sincosf(t, &sn, &cs);
     return mk(cs, sn);
-}
-__device__ __forceinline__ cplx<double> link_phase(const double2* __restrict__ Zq, int V, int mu, int s, double) {
-    const double2 z = Zq[(size_t)mu * V + s];
-    return mk(z.x, z.y);
 }
 
 template <typename R>
@@ -135,13 +137,13 @@ __device__ __forceinline__ void times3(cplx<R> ph, cplx<R> v[3]) {
 template <typename R>
 __device__ __forceinline__ void su3_mul(const cplx<R> u[3][3], const cplx<R> h[3], cplx<R> g[3]) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) g[a] = u[a][0] * h[0] + u[a][1] * h[1] + u[a][2] * h[2];
+    for (int a = 0; a < 3; ++a) g[a] = mad(u[a][2], h[2], mad(u[a][1], h[1], u[a][0] * h[0]));
 }
 // g = u^+ h
 template <typename R>
 __device__ __forceinline__ void su3_dag_mul(const cplx<R> u[3][3], const cplx<R> h[3], cplx<R> g[3]) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) g[a] = cmul(u[0][a], h[0]) + cmul(u[1][a], h[1]) + cmul(u[2][a], h[2]);
+    for (int a = 0; a < 3; ++a) g[a] = cmad(u[2][a], h[2], cmad(u[1][a], h[1], cmul(u[0][a], h[0])));
 }
 
 // ---------------------------------------------------------------------------
@@ -168,10 +170,18 @@ __device__ __forceinline__ void project(const cplx<R> p[12], cplx<R> h0[3], cplx
     }
 }
 
-template <typename R, int MU, int DIR>
+// FIRST: the first hop of a site, direction 0 forwards, sets acc (the sum
+// starts there, not from zero)
+template <typename R, int MU, int DIR, bool FIRST = false>
 __device__ __forceinline__ void accumulate(cplx<R> acc[12], const cplx<R> g0[3], const cplx<R> g1[3]) {
+    static_assert(!FIRST || (MU == 0 && DIR > 0), "the first hop is direction 0 forwards");
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
+        if (FIRST) {
+            acc[c] = acc[6 + c] = g0[c];
+            acc[3 + c] = acc[9 + c] = g1[c];
+            continue;
+        }
         acc[c] = acc[c] + g0[c];
         acc[3 + c] = acc[3 + c] + g1[c];
         if (MU == 0) {
@@ -194,23 +204,27 @@ __device__ __forceinline__ void accumulate(cplx<R> acc[12], const cplx<R> g0[3],
 // clover blocks: y = M v, two Hermitian 6x6 blocks, packed (6 real diag,
 // 15 complex strictly-lower entries row major)
 // ---------------------------------------------------------------------------
-template <typename R>
+// ADD: y += M v (the sum continues the multiply-add chains), else y = M v.
+// The diagonal, 4 + m0 and by far the largest term, comes last: the chains
+// then round at the size of the small terms (with it first the FP64 D was
+// off by 2.2e-16 instead of 1.5e-16 in norm).
+template <typename R, bool ADD>
 __device__ __forceinline__ void herm6_mul(const R d[6], const cplx<R> L[15], const cplx<R> v[6], cplx<R> y[6]) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) y[i] = d[i] * v[i];
     int k = 0;
 #pragma unroll
     for (int i = 1; i < 6; ++i)
 #pragma unroll
         for (int j = 0; j < i; ++j, ++k) {
-            y[i] = y[i] + L[k] * v[j];
-            y[j] = y[j] + cmul(L[k], v[i]);
+            y[i] = !ADD && j == 0 ? L[k] * v[j] : mad(L[k], v[j], y[i]);
+            y[j] = !ADD && i == 1 ? cmul(L[k], v[i]) : cmad(L[k], v[i], y[j]);
         }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) y[i] = rmad(d[i], v[i], y[i]);
 }
 
 // STREAM: evict-first loads, for kernels that read each clover block once per
 // launch (not the Schwarz block solves, which re-read it every MR step)
-template <bool STREAM = false>
+template <bool STREAM = false, bool ADD = false>
 __device__ __forceinline__ void clover_mul(const float4* __restrict__ C, int V, int s, const cplx<float> v[12],
                                            cplx<float> w[12]) {
 #pragma unroll
@@ -230,11 +244,11 @@ __device__ __forceinline__ void clover_mul(const float4* __restrict__ C, int V, 
         for (int i = 0; i < 6; ++i) d[i] = r[i];
 #pragma unroll
         for (int k = 0; k < 15; ++k) L[k] = mk(r[6 + 2 * k], r[7 + 2 * k]);
-        herm6_mul(d, L, v + 6 * blk, w + 6 * blk);
+        herm6_mul<float, ADD>(d, L, v + 6 * blk, w + 6 * blk);
     }
 }
 
-template <bool STREAM = false>
+template <bool STREAM = false, bool ADD = false>
 __device__ __forceinline__ void clover_mul(const double* __restrict__ C, int V, int s, const cplx<double> v[12],
                                            cplx<double> w[12]) {
 #pragma unroll
@@ -246,14 +260,15 @@ __device__ __forceinline__ void clover_mul(const double* __restrict__ C, int V, 
 #pragma unroll
         for (int k = 0; k < 15; ++k)
             L[k] = mk(C[(size_t)(36 * blk + 6 + 2 * k) * V + s], C[(size_t)(36 * blk + 7 + 2 * k) * V + s]);
-        herm6_mul(d, L, v + 6 * blk, w + 6 * blk);
+        herm6_mul<double, ADD>(d, L, v + 6 * blk, w + 6 * blk);
     }
 }
 
 // The two hops of direction MU at site x (native index s, parity 1 - po),
-// raw sum (without the factor -1/2) added to acc. The neighbour spinors are
-// read from psi at index (native index - poff) with stride pstride, so the
-// same code serves full-lattice and half-lattice fields.
+// raw sum (H psi is HopScale times it) added to acc; direction 0 comes first
+// and sets acc. The neighbour spinors are read from psi at index (native index
+// - poff) with stride pstride, so the same code serves full-lattice and
+// half-lattice fields. QNZ: FP32 only (U(1) phase from the angles).
 template <typename R, bool QNZ, int MU>
 __device__ __forceinline__ void dirac_dir(const Geom& g, const Fields<R>& f,
                                           const typename Fields<R>::vec* __restrict__ psi, int pstride,
@@ -268,12 +283,12 @@ __device__ __forceinline__ void dirac_dir(const Geom& g, const Fields<R>& f,
         load_link(f.U, g.V, MU, s, u);
         su3_mul(u, h0, g0);
         su3_mul(u, h1, g1);
-        if (QNZ) {
+        if constexpr (QNZ && sizeof(R) == 4) {
             cplx<R> ph = link_phase(f.A, g.V, MU, s, q);
             times3(ph, g0);
             times3(ph, g1);
         }
-        accumulate<R, MU, +1>(acc, g0, g1);
+        accumulate<R, MU, +1, MU == 0>(acc, g0, g1);
     }
     // backward hop: (1 + g_mu) U(x-mu,mu)^+ z(x-mu,mu)^-q psi(x-mu)
     {
@@ -283,13 +298,24 @@ __device__ __forceinline__ void dirac_dir(const Geom& g, const Fields<R>& f,
         load_link(f.U, g.V, MU, sb, u);
         su3_dag_mul(u, h0, g0);
         su3_dag_mul(u, h1, g1);
-        if (QNZ) {
+        if constexpr (QNZ && sizeof(R) == 4) {
             cplx<R> ph = conj(link_phase(f.A, g.V, MU, sb, q));
             times3(ph, g0);
             times3(ph, g1);
         }
         accumulate<R, MU, -1>(acc, g0, g1);
     }
+}
+
+// raw sum of the eight hops at site x (see dirac_dir)
+template <typename R, bool QNZ>
+__device__ __forceinline__ void dirac_hops(const Geom& g, const Fields<R>& f,
+                                           const typename Fields<R>::vec* __restrict__ psi, int pstride, int poff, R q,
+                                           int x0, int x1, int x2, int x3, int s, int po, cplx<R> acc[12]) {
+    dirac_dir<R, QNZ, 0>(g, f, psi, pstride, poff, q, x0, x1, x2, x3, s, po, acc);
+    dirac_dir<R, QNZ, 1>(g, f, psi, pstride, poff, q, x0, x1, x2, x3, s, po, acc);
+    dirac_dir<R, QNZ, 2>(g, f, psi, pstride, poff, q, x0, x1, x2, x3, s, po, acc);
+    dirac_dir<R, QNZ, 3>(g, f, psi, pstride, poff, q, x0, x1, x2, x3, s, po, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -338,7 +364,7 @@ __device__ __forceinline__ void hop_load(const Fields<float>& f, int V, int k, i
 
 // raw hop (without the factor -1/2) added to acc: (1 - DIR g_mu) W psi(x + DIR mu)
 // with W = U z^qhat forwards and its adjoint backwards
-template <bool QNZ, int MU, int DIR>
+template <bool QNZ, int MU, int DIR, bool FIRST = false>
 __device__ __forceinline__ void hop_compute(const HopData& d, float q, cplx<float> acc[12]) {
     cplx<float> v[12], h0[3], h1[3], g0[3], g1[3], u[3][3];
 #pragma unroll
@@ -374,10 +400,10 @@ __device__ __forceinline__ void hop_compute(const HopData& d, float q, cplx<floa
         times3(ph, g0);
         times3(ph, g1);
     }
-    accumulate<float, MU, DIR>(acc, g0, g1);
+    accumulate<float, MU, DIR, FIRST>(acc, g0, g1);
 }
 
-// acc += raw sum of the eight hops at site s with neighbours nb
+// acc = raw sum of the eight hops at site s with neighbours nb
 template <bool QNZ>
 __device__ __forceinline__ void hops_pipelined(const Fields<float>& f, int V, int s, const int nb[8], float q,
                                                cplx<float> acc[12]) {
@@ -385,7 +411,7 @@ __device__ __forceinline__ void hops_pipelined(const Fields<float>& f, int V, in
     HopData d[2];
     hop_load(f, V, 0, s, nb[0], a_own, d[0]);
     hop_load(f, V, 1, s, nb[1], a_own, d[1]);
-    hop_compute<QNZ, 0, +1>(d[0], q, acc);
+    hop_compute<QNZ, 0, +1, true>(d[0], q, acc);
     hop_load(f, V, 2, s, nb[2], a_own, d[0]);
     hop_compute<QNZ, 0, -1>(d[1], q, acc);
     hop_load(f, V, 3, s, nb[3], a_own, d[1]);

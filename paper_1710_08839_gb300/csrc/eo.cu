@@ -33,42 +33,37 @@ __global__ void __launch_bounds__(DW_THREADS, DwMinBlocksEo<R>::value)
     sweep_coords_parity(g, p, tau, x0, x1, x2, x3);
     const int s = native_index(g, lex_index(g, x0, x1, x2, x3), p);
     const int po = 1 - p;
-    cplx<R> acc[12];
-#pragma unroll
-    for (int i = 0; i < 12; ++i) acc[i] = mk<R>(0, 0);
-    dirac_dir<R, QNZ, 0>(g, f, in.p, in.stride, in.off, q, x0, x1, x2, x3, s, po, acc);
-    dirac_dir<R, QNZ, 1>(g, f, in.p, in.stride, in.off, q, x0, x1, x2, x3, s, po, acc);
-    dirac_dir<R, QNZ, 2>(g, f, in.p, in.stride, in.off, q, x0, x1, x2, x3, s, po, acc);
-    dirac_dir<R, QNZ, 3>(g, f, in.p, in.stride, in.off, q, x0, x1, x2, x3, s, po, acc);
-    cplx<R> w[12];
+    cplx<R> acc[12], w[12];
+    dirac_hops<R, QNZ>(g, f, in.p, in.stride, in.off, q, x0, x1, x2, x3, s, po, acc);
+    constexpr R HS = HopScale<R>::value;  // H psi = HS acc
     if (MODE == EO_HOP) {
 #pragma unroll
-        for (int i = 0; i < 12; ++i) w[i] = R(-0.5) * acc[i];
+        for (int i = 0; i < 12; ++i) w[i] = HS * acc[i];
     } else if (MODE == EO_INV_HOP) {
         cplx<R> t[12];
 #pragma unroll
-        for (int i = 0; i < 12; ++i) t[i] = R(-0.5) * acc[i];
+        for (int i = 0; i < 12; ++i) t[i] = HS * acc[i];
         clover_mul<true>(Cl, g.V, s, t, w);
     } else if (MODE == EO_CLOVER_AUX_MHOP || MODE == EO_G5_CLOVER_AUX_MHOP) {
         cplx<R> a[12];
         load_spinor(aux.p, aux.stride, s - aux.off, a);
-        clover_mul<true>(Cl, g.V, s, a, w);
 #pragma unroll
-        for (int i = 0; i < 12; ++i) w[i] = w[i] + R(0.5) * acc[i];
+        for (int i = 0; i < 12; ++i) w[i] = (-HS) * acc[i];
+        clover_mul<true, true>(Cl, g.V, s, a, w);
         if (MODE == EO_G5_CLOVER_AUX_MHOP) {
             // gamma5 = diag(1, 1, -1, -1): spins 2 and 3 change sign
 #pragma unroll
-            for (int i = 6; i < 12; ++i) w[i] = R(-1) * w[i];
+            for (int i = 6; i < 12; ++i) w[i] = -w[i];
         }
     } else if (MODE == EO_AUX_MHOP) {
         load_spinor(aux.p, aux.stride, s - aux.off, w);
 #pragma unroll
-        for (int i = 0; i < 12; ++i) w[i] = w[i] + R(0.5) * acc[i];
+        for (int i = 0; i < 12; ++i) w[i] = rmad(-HS, acc[i], w[i]);
     } else {  // EO_INV_AUX_MHOP
         cplx<R> a[12];
         load_spinor(aux.p, aux.stride, s - aux.off, a);
 #pragma unroll
-        for (int i = 0; i < 12; ++i) a[i] = a[i] + R(0.5) * acc[i];
+        for (int i = 0; i < 12; ++i) a[i] = rmad(-HS, acc[i], a[i]);
         clover_mul<true>(Cl, g.V, s, a, w);
     }
     store_spinor(out.p, out.stride, s - out.off, w);
@@ -112,7 +107,9 @@ int launch_eo(qxd_lattice* lat, int mode, int p, SpRef<R> in, SpRef<R> aux, SpRe
               cudaStream_t st) {
     Fields<R> f = fields_of<R>(lat);
     const typename Fields<R>::cvec* Cl = clover_of<R>(lat, inverse);
-    if (lat->qhat != 0) return launch_mode<R, true>(lat, mode, p, f, in, aux, out, Cl, st);
+    if constexpr (sizeof(R) == 4) {  // FP64: the charge is in the links
+        if (lat->qhat != 0) return launch_mode<R, true>(lat, mode, p, f, in, aux, out, Cl, st);
+    }
     return launch_mode<R, false>(lat, mode, p, f, in, aux, out, Cl, st);
 }
 

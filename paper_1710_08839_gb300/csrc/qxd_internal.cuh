@@ -167,8 +167,9 @@ __host__ __device__ __forceinline__ int neighbour_lex(const Geom& g, int x0, int
 // links  FP64 : double2 U[4][9][V]  full 3x3, row major
 // angle  FP32 : float4  A[V]        A(x, mu), mu = 0..3
 // angle  FP64 : double  A[4][V]
-// phase  FP64 : double2 Z[4][V]    z = exp(i A) as (cos A, sin A); per operator
-//                                   also Zq[4][V] = z^qhat (built with the clover)
+// phase  FP64 : double2 Z[4][V]    z = exp(i A) as (cos A, sin A)
+// hop link FP64: double2 W[4][9][V] W(x,mu) = -1/2 z(x,mu)^qhat U(x,mu), full
+//                                   3x3, per operator (built with the clover)
 // clover FP32 : float4  C[18][V]    two Hermitian 6x6 blocks (spins {0,1},
 //                                   then {2,3}), 36 floats each: 6 real
 //                                   diagonals, then the 15 complex entries
@@ -220,6 +221,25 @@ template <typename R>
 __host__ __device__ __forceinline__ cplx<R> cmul(cplx<R> a, cplx<R> b) {
     return {a.re * b.re + a.im * b.im, a.re * b.im - a.im * b.re};
 }
+// acc + a * b and acc + conj(a) * b as chains of fused multiply-adds: four
+// instructions. acc + a * b written with the operators above takes six (the
+// compiler may not move the sum into the product), which is what bounded the
+// FP64 kernels: GB300 issues two FP64 lanes per clock and SM.
+__host__ __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__host__ __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+template <typename R>
+__host__ __device__ __forceinline__ cplx<R> mad(cplx<R> a, cplx<R> b, cplx<R> acc) {
+    return {fma_(-a.im, b.im, fma_(a.re, b.re, acc.re)), fma_(a.im, b.re, fma_(a.re, b.im, acc.im))};
+}
+template <typename R>
+__host__ __device__ __forceinline__ cplx<R> cmad(cplx<R> a, cplx<R> b, cplx<R> acc) {
+    return {fma_(a.im, b.im, fma_(a.re, b.re, acc.re)), fma_(-a.im, b.re, fma_(a.re, b.im, acc.im))};
+}
+// acc + s * a, s real
+template <typename R>
+__host__ __device__ __forceinline__ cplx<R> rmad(R s, cplx<R> a, cplx<R> acc) {
+    return {fma_(s, a.re, acc.re), fma_(s, a.im, acc.im)};
+}
 // i * a, -i * a
 template <typename R>
 __host__ __device__ __forceinline__ cplx<R> times_i(cplx<R> a) { return {-a.im, a.re}; }
@@ -255,7 +275,7 @@ struct qxd_lattice {
     double m0 = 0, csw = 0, cswqed = 0;
     int qhat = 0;
     bool has_params = false;
-    double2* Zq64 = nullptr;   // [4][V] z^qhat for this operator's qhat (FP64 kernels)
+    double2* W64 = nullptr;    // [4][9][V] -1/2 z^qhat U for this operator's qhat (FP64 kernels)
     double* C64 = nullptr;     // [72][V]
     float4* C32 = nullptr;     // [18][V]
     double* Cinv64 = nullptr;  // [72][V]

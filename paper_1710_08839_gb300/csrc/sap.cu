@@ -60,23 +60,6 @@ struct SmemField {
     }
 };
 
-// Links of the block for the one-thread-per-pair form (FP64): read from the
-// global field.
-template <typename R>
-struct BlockLinks;
-
-template <>
-struct BlockLinks<double> {
-    __device__ __forceinline__ void link(const Fields<double>& f, const Geom& g, int mu, int, int s,
-                                         cplx<double> u[3][3]) const {
-        load_link(f.U, g.V, mu, s, u);
-    }
-    __device__ __forceinline__ cplx<double> phase(const Fields<double>& f, const Geom& g, int mu, int, int s,
-                                                  double q) const {
-        return link_phase(f.A, g.V, mu, s, q);
-    }
-};
-
 struct Site {
     int l[4];   // coordinates inside the block
     int x[4];   // global coordinates
@@ -107,78 +90,56 @@ __device__ __forceinline__ int back_native(const Geom& g, const Site& t) {
 }
 
 // hops of direction MU that stay inside the block (Dirichlet block boundary);
-// the neighbour spinor comes from shared memory (field of the other parity)
-template <typename R, bool QNZ, int MU>
-__device__ __forceinline__ void block_dir(const Geom& g, const Fields<R>& f, const BlockLinks<R>& bl,
-                                          const SmemField<R>& src, R q, const Site& t, cplx<R> acc[12]) {
+// the neighbour spinor comes from shared memory (field of the other parity).
+// FP64 only: the links are compound (the charge and the factor -1/2 are in).
+template <typename R, int MU>
+__device__ __forceinline__ void block_dir(const Geom& g, const Fields<R>& f, const SmemField<R>& src, const Site& t,
+                                          cplx<R> acc[12]) {
     constexpr int stride = MU == 0 ? 64 : MU == 1 ? 16 : MU == 2 ? 4 : 1;
     cplx<R> v[12], h0[3], h1[3], g0[3], g1[3], u[3][3];
     if (t.l[MU] < SAP_BS - 1) {
         src.load((t.lidx + stride) >> 1, v);
         project<R, MU, +1>(v, h0, h1);
-        bl.link(f, g, MU, t.lidx, t.s, u);
+        load_link(f.U, g.V, MU, t.s, u);
         su3_mul(u, h0, g0);
         su3_mul(u, h1, g1);
-        if (QNZ) {
-            cplx<R> ph = bl.phase(f, g, MU, t.lidx, t.s, q);
-            times3(ph, g0);
-            times3(ph, g1);
-        }
         accumulate<R, MU, +1>(acc, g0, g1);
     }
     if (t.l[MU] > 0) {
         src.load((t.lidx - stride) >> 1, v);
         project<R, MU, -1>(v, h0, h1);
-        const int sb = back_native<MU>(g, t);
-        bl.link(f, g, MU, t.lidx - stride, sb, u);
+        load_link(f.U, g.V, MU, back_native<MU>(g, t), u);
         su3_dag_mul(u, h0, g0);
         su3_dag_mul(u, h1, g1);
-        if (QNZ) {
-            cplx<R> ph = conj(bl.phase(f, g, MU, t.lidx - stride, sb, q));
-            times3(ph, g0);
-            times3(ph, g1);
-        }
         accumulate<R, MU, -1>(acc, g0, g1);
     }
 }
 
-template <typename R, bool QNZ>
-__device__ __forceinline__ void block_hops(const Geom& g, const Fields<R>& f, const BlockLinks<R>& bl,
-                                        const SmemField<R> src, R q, const Site& t, cplx<R> acc[12]) {
+template <typename R>
+__device__ __forceinline__ void block_hops(const Geom& g, const Fields<R>& f, const SmemField<R> src, const Site& t,
+                                           cplx<R> acc[12]) {
 #pragma unroll
     for (int i = 0; i < 12; ++i) acc[i] = mk<R>(0, 0);
-    block_dir<R, QNZ, 0>(g, f, bl, src, q, t, acc);
-    block_dir<R, QNZ, 1>(g, f, bl, src, q, t, acc);
-    block_dir<R, QNZ, 2>(g, f, bl, src, q, t, acc);
-    block_dir<R, QNZ, 3>(g, f, bl, src, q, t, acc);
+    block_dir<R, 0>(g, f, src, t, acc);
+    block_dir<R, 1>(g, f, src, t, acc);
+    block_dir<R, 2>(g, f, src, t, acc);
+    block_dir<R, 3>(g, f, src, t, acc);
 }
 
-// r = eta - (D psi)(x), D over the whole lattice, at one site
-template <typename R, bool QNZ>
-__device__ __forceinline__ void residual_body(const Geom& g, const Fields<R>& f, const typename Fields<R>::vec* eta,
-                                              R q, const Site& t, bool psi_zero, cplx<R> r[12]) {
+// r = eta - (D psi)(x), D over the whole lattice, at one site; out of line,
+// for the one-thread-per-pair kernel, which calls it twice
+template <typename R>
+__device__ __noinline__ void residual_at(const Geom& g, const Fields<R>& f, const typename Fields<R>::vec* eta,
+                                         const Site& t, bool psi_zero, cplx<R> r[12]) {
     load_spinor(eta, g.V, t.s, r);
     if (psi_zero) return;
     const int po = 1 - ((t.x[0] + t.x[1] + t.x[2] + t.x[3]) & 1);
-    cplx<R> acc[12];
-#pragma unroll
-    for (int i = 0; i < 12; ++i) acc[i] = mk<R>(0, 0);
-    dirac_dir<R, QNZ, 0>(g, f, f.psi, g.V, 0, q, t.x[0], t.x[1], t.x[2], t.x[3], t.s, po, acc);
-    dirac_dir<R, QNZ, 1>(g, f, f.psi, g.V, 0, q, t.x[0], t.x[1], t.x[2], t.x[3], t.s, po, acc);
-    dirac_dir<R, QNZ, 2>(g, f, f.psi, g.V, 0, q, t.x[0], t.x[1], t.x[2], t.x[3], t.s, po, acc);
-    dirac_dir<R, QNZ, 3>(g, f, f.psi, g.V, 0, q, t.x[0], t.x[1], t.x[2], t.x[3], t.s, po, acc);
-    cplx<R> v[12], w[12];
+    cplx<R> acc[12], v[12];
+    dirac_hops<R, false>(g, f, f.psi, g.V, 0, R(0), t.x[0], t.x[1], t.x[2], t.x[3], t.s, po, acc);
     load_spinor(f.psi, g.V, t.s, v);
-    clover_mul(f.C, g.V, t.s, v, w);
+    clover_mul<false, true>(f.C, g.V, t.s, v, acc);
 #pragma unroll
-    for (int i = 0; i < 12; ++i) r[i] = r[i] - (w[i] - R(0.5) * acc[i]);
-}
-
-// out-of-line form for the one-thread-per-pair kernel, which calls it twice
-template <typename R, bool QNZ>
-__device__ __noinline__ void residual_at(const Geom& g, const Fields<R>& f, const typename Fields<R>::vec* eta,
-                                         R q, const Site& t, bool psi_zero, cplx<R> r[12]) {
-    residual_body<R, QNZ>(g, f, eta, q, t, psi_zero, r);
+    for (int i = 0; i < 12; ++i) r[i] = r[i] - acc[i];
 }
 
 // sum over the NT threads of the block, result in every thread. TAIL_SYNC
@@ -218,12 +179,12 @@ __device__ __forceinline__ void block_sum3(R a, R b, R c, R* red, R out[3]) {
 //                      omega = <w,rho>/<w,w>, delta_e += omega rho,
 //                      rho -= omega w (even)             for k < nmr
 //   last step:         delta_o = M_oo^-1 (r_o - H_oe delta_e)     (odd)
-template <typename R, bool QNZ>
+template <typename R>
 __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg, int bidx, int colour, int psi_zero,
                                                const Fields<R>& f, const typename Fields<R>::cvec* __restrict__ Cinv,
-                                               const typename Fields<R>::vec* __restrict__ eta, int nmr, R q) {
+                                               const typename Fields<R>::vec* __restrict__ eta, int nmr) {
+    static_assert(sizeof(R) == 8, "FP64 block solve (compound links)");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    BlockLinks<R> bl;
     R* sm = reinterpret_cast<R*>(smem_raw);
     const SmemField<R> s_ro{sm};                    // r on the odd sites
     const SmemField<R> s_rho{sm + 24 * SAP_HALF};   // MR residual (even)
@@ -256,7 +217,7 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
     cplx<R> re[12], v[12], w[12], acc[12];
 #pragma unroll 1
     for (int k = 0; k < 2; ++k) {
-        residual_at<R, QNZ>(g, f, eta, q, k ? so : se, psi_zero, k ? v : re);
+        residual_at<R>(g, f, eta, k ? so : se, psi_zero, k ? v : re);
     }
     s_ro.store(t, v);
     clover_mul(Cinv, g.V, so.s, v, w);  // t_o = M_oo^-1 r_o
@@ -272,25 +233,24 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
         const bool odd = (step & 1) != 0;   // steps 1, 3, ..., 2 nmr + 1 work on the odd sites
         const bool last = step == nsteps - 1;
         // odd steps read rho (or delta_e on the last step), even steps read t_o
-        block_hops<R, QNZ>(g, f, bl, odd ? (last ? s_t : s_rho) : s_t, q, odd ? so : se, acc);
+        block_hops<R>(g, f, odd ? (last ? s_t : s_rho) : s_t, odd ? so : se, acc);
+        // acc = H psi on the sites of this step's parity
         if (step == 0) {
 #pragma unroll
-            for (int i = 0; i < 12; ++i) rho[i] = re[i] + R(0.5) * acc[i];
+            for (int i = 0; i < 12; ++i) rho[i] = re[i] - acc[i];
             s_rho.store(t, rho);
         } else if (last) {
             s_ro.load(t, v);
 #pragma unroll
-            for (int i = 0; i < 12; ++i) v[i] = v[i] + R(0.5) * acc[i];
+            for (int i = 0; i < 12; ++i) v[i] = v[i] - acc[i];
             clover_mul(Cinv, g.V, so.s, v, w);  // delta_o
         } else if (odd) {
-#pragma unroll
-            for (int i = 0; i < 12; ++i) v[i] = R(-0.5) * acc[i];
-            clover_mul(Cinv, g.V, so.s, v, w);
+            clover_mul(Cinv, g.V, so.s, acc, w);
             s_t.store(t, w);
         } else {
-            clover_mul(f.C, g.V, se.s, rho, w);
 #pragma unroll
-            for (int i = 0; i < 12; ++i) w[i] = w[i] + R(0.5) * acc[i];
+            for (int i = 0; i < 12; ++i) w[i] = -acc[i];
+            clover_mul<false, true>(f.C, g.V, se.s, rho, w);
             R a_re = 0, a_im = 0, b = 0;
 #pragma unroll
             for (int i = 0; i < 12; ++i) {
@@ -304,8 +264,8 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
                 const cplx<R> om = mk(sums[0] / sums[2], sums[1] / sums[2]);
 #pragma unroll
                 for (int i = 0; i < 12; ++i) {
-                    de[i] = de[i] + om * rho[i];
-                    rho[i] = rho[i] - om * w[i];
+                    de[i] = mad(om, rho[i], de[i]);
+                    rho[i] = mad(-om, w[i], rho[i]);
                 }
             }
             if (step == nsteps - 2) s_t.store(t, de);  // delta_e for the last step
@@ -330,12 +290,11 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
     }
 }
 
-template <typename R, bool QNZ>
+template <typename R>
 __global__ void __launch_bounds__(SAP_THREADS, 2) k_sap_block(Geom g, SapGeom sg, int colour, int psi_zero,
                                                               Fields<R> f, const typename Fields<R>::cvec* __restrict__ Cinv,
-                                                              const typename Fields<R>::vec* __restrict__ eta, int nmr,
-                                                              R q) {
-    sap_block_body<R, QNZ>(g, sg, blockIdx.x, colour, psi_zero, f, Cinv, eta, nmr, q);
+                                                              const typename Fields<R>::vec* __restrict__ eta, int nmr) {
+    sap_block_body<R>(g, sg, blockIdx.x, colour, psi_zero, f, Cinv, eta, nmr);
 }
 
 // ---------------------------------------------------------------------------
@@ -556,19 +515,21 @@ __device__ __forceinline__ void clover_half(const float4* __restrict__ C, int V,
         const cplx<float>* w = v + 3 * blk;
         const cplx<float>* pp = p + 3 * blk;
         cplx<float> z[3];
-        z[0] = d0 * w[0] + cmul(l10, w[1]) + cmul(l20, w[2]);
-        z[1] = l10 * w[0] + d1 * w[1] + cmul(l21, w[2]);
-        z[2] = l20 * w[0] + l21 * w[1] + d2 * w[2];
+        // the diagonal, the largest term, comes last
+        z[0] = cmad(l20, w[2], cmul(l10, w[1]));
+        z[1] = cmad(l21, w[2], l10 * w[0]);
+        z[2] = mad(l21, w[1], l20 * w[0]);
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
             for (int b = 0; b < 3; ++b) {
                 // E[a][b] = sg ? B[a][b] : conj(B[b][a])
                 const cplx<float> e = mk(sg ? B[a][b].re : B[b][a].re, sg ? B[a][b].im : -B[b][a].im);
-                z[a] = z[a] + e * pp[b];
+                z[a] = mad(e, pp[b], z[a]);
             }
-#pragma unroll
-        for (int a = 0; a < 3; ++a) y[3 * blk + a] = z[a];
+        y[3 * blk] = rmad(d0, w[0], z[0]);
+        y[3 * blk + 1] = rmad(d1, w[1], z[1]);
+        y[3 * blk + 2] = rmad(d2, w[2], z[2]);
     }
     (void)sgn;
 }
@@ -782,8 +743,8 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
                     const cplx<float> om = mk(sums[0] / sums[2], sums[1] / sums[2]);
 #pragma unroll
                     for (int i = 0; i < 6; ++i) {
-                        de[i] = de[i] + om * rho[i];
-                        rho[i] = rho[i] - om * w[i];
+                        de[i] = mad(om, rho[i], de[i]);
+                        rho[i] = mad(-om, w[i], rho[i]);
                     }
                 }
                 if (step == nsteps - 2) {
@@ -883,14 +844,12 @@ int split_flags(int cy, int colour, int ncy) {
 }
 
 // FP64 visit `cy` of colour `colour` out of ncy cycles
-template <bool QNZ>
 int launch_sap_block64(qxd_lattice* lat, const SapGeom& sg, int cy, int colour, Fields<double> f,
                        const double* Cinv, const double2* eta, int nmr, cudaStream_t st) {
     const size_t smem = sap_smem_bytes<double>();
     const int psi_zero = (cy == 0 && colour == 0) ? 1 : 0;
-    QXD_CUDA(cudaFuncSetAttribute(k_sap_block<double, QNZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_sap_block<double, QNZ><<<sg.nhalf, SAP_THREADS, smem, st>>>(lat->g, sg, colour, psi_zero, f, Cinv, eta, nmr,
-                                                                   (double)lat->qhat);
+    QXD_CUDA(cudaFuncSetAttribute(k_sap_block<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_sap_block<double><<<sg.nhalf, SAP_THREADS, smem, st>>>(lat->g, sg, colour, psi_zero, f, Cinv, eta, nmr);
     QXD_LAUNCHED("k_sap_block");
     return QXD_OK;
 }
@@ -974,14 +933,10 @@ int sap_apply(qxd_lattice* lat, SapWork& w, void* out, const void* in, int ncy, 
         // psi starts at zero; the first half-cycle writes the blocks of colour 0
         // without reading psi, and the blocks of colour 1 must read zeros there
         QXD_CUDA(cudaMemsetAsync(out, 0, (size_t)g.V * 24 * sizeof(R), st));
-        const Fields<double> f{(const double2*)out, nullptr, lat->U64, lat->Zq64, lat->C64};
+        const Fields<double> f{(const double2*)out, nullptr, lat->W64, lat->C64};
         for (int cy = 0; cy < ncy; ++cy)
             for (int colour = 0; colour < 2; ++colour) {
-                const int rc = lat->qhat != 0
-                                   ? launch_sap_block64<true>(lat, w.sg, cy, colour, f, lat->Cinv64,
-                                                              (const double2*)in, nmr, st)
-                                   : launch_sap_block64<false>(lat, w.sg, cy, colour, f, lat->Cinv64,
-                                                               (const double2*)in, nmr, st);
+                const int rc = launch_sap_block64(lat, w.sg, cy, colour, f, lat->Cinv64, (const double2*)in, nmr, st);
                 if (rc) return rc;
             }
         return QXD_OK;
