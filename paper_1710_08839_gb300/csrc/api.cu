@@ -311,6 +311,7 @@ int qxd_Dw(qxd_lattice* lat, void* out, const void* in, int flags, void* stream)
     cudaStream_t st = stream ? (cudaStream_t)stream : lat->stream;
     if (out == in) return fail(QXD_ERR_ARG, "qxd_Dw: in and out must not overlap");
     if (native) return launch_dirac(lat, out, in, prec, st);
+    if (!host && dirac_takes_lex(out, in, prec)) return launch_dirac_lex(lat, out, in, prec, st);
     int rc = ensure_scratch(lat);
     if (rc) return rc;
     size_t bytes = qxd_spinor_bytes(lat, prec);

@@ -3,9 +3,10 @@
 //                                  + (1 + g_mu) W(x-mu,mu)^+ psi(x-mu) ],
 //   W(x,mu) = U(x,mu) z(x,mu)^qhat,  M(x) = (4 + m0) + dDsw(x),
 // which is Eqs. (18)-(20) expanded (the diagonal 4 of Dw moved into M).
-// One thread per site; spin projection to half spinors before the colour
+// FP32: one thread per site; spin projection to half spinors before the colour
 // multiplication (the projectors commute with W). FP32: links as two rows
-// plus the U(1) angle, hops software-pipelined (k_dirac32); FP64: full links.
+// plus the U(1) angle, hops software-pipelined (k_dirac32); FP64: compound
+// links, a site's work split over threads (dirac64.cu).
 // Both parities in one sweep, in the tiled order of sweep_coords so
 // neighbour data is reused from L2.
 //
@@ -20,6 +21,7 @@
 #include <tuple>
 #include <vector>
 
+#include "dirac64.cuh"
 #include "dirac_common.cuh"
 #include "tune.cuh"
 
@@ -50,24 +52,23 @@ __global__ void __launch_bounds__(DW_THREADS, DW_PP_MIN_BLOCKS)
     store_spinor_cs(f.out, g.V, s, acc);
 }
 
-template <typename R, bool QNZ>
-__global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<R>::value)
-    k_dirac(Geom g, Fields<R> f, R q, int x0b, int nx0, int nsites) {
+// FP32, the plain hop order (80 registers, 6 blocks per SM)
+template <bool QNZ>
+__global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<float>::value)
+    k_dirac(Geom g, Fields<float> f, float q, int x0b, int nx0, int nsites) {
     const int tau = blockIdx.x * blockDim.x + threadIdx.x;
     if (tau >= nsites) return;
     int x0, x1, x2, x3;
     sweep_coords_slab(g, x0b, nx0, tau, x0, x1, x2, x3);
     const int p = (x0 + x1 + x2 + x3) & 1;
     const int s = native_index(g, lex_index(g, x0, x1, x2, x3), p);
-    const int po = 1 - p;
-    cplx<R> acc[12], v[12];
-    dirac_hops<R, QNZ>(g, f, f.psi, g.V, 0, q, x0, x1, x2, x3, s, po, acc);
+    cplx<float> acc[12], v[12];
+    dirac_hops<float, QNZ>(g, f, f.psi, g.V, 0, q, x0, x1, x2, x3, s, 1 - p, acc);
 #pragma unroll
-    for (int i = 0; i < 12; ++i) acc[i] = HopScale<R>::value * acc[i];
+    for (int i = 0; i < 12; ++i) acc[i] = HopScale<float>::value * acc[i];
     load_spinor(f.psi, g.V, s, v);
     clover_mul<true, true>(f.C, g.V, s, v, acc);
-    if constexpr (sizeof(R) == 4) store_spinor_cs(f.out, g.V, s, acc);
-    else store_spinor(f.out, g.V, s, acc);
+    store_spinor_cs(f.out, g.V, s, acc);
 }
 
 // lexicographic [site][spin][colour][re,im] <-> native structure of arrays
@@ -105,9 +106,9 @@ __global__ void k_unpack(Geom g, const typename Fields<R>::vec* __restrict__ nat
 namespace {
 
 // D with launch shape sh (hop order, threads per block, sweep window) on the
-// x0 planes [x0b, x0b + nx0)
+// x0 planes [x0b, x0b + nx0); lex (FP64 only): lexicographic fields
 int launch_dirac_shape(qxd_lattice* lat, void* out, const void* in, int prec, const DwShape& sh, cudaStream_t st,
-                       int x0b = 0, int nx0 = -1) {
+                       int x0b = 0, int nx0 = -1, bool lex = false) {
     Geom g = lat->g;
     g.R = sh.rows;
     if (nx0 < 0) nx0 = g.N0;
@@ -120,12 +121,12 @@ int launch_dirac_shape(qxd_lattice* lat, void* out, const void* in, int prec, co
             if (qnz) k_dirac32<true><<<blocks, sh.threads, 0, st>>>(g, f, (float)lat->qhat, x0b, nx0, n);
             else k_dirac32<false><<<blocks, sh.threads, 0, st>>>(g, f, 0.f, x0b, nx0, n);
         } else {
-            if (qnz) k_dirac<float, true><<<blocks, sh.threads, 0, st>>>(g, f, (float)lat->qhat, x0b, nx0, n);
-            else k_dirac<float, false><<<blocks, sh.threads, 0, st>>>(g, f, 0.f, x0b, nx0, n);
+            if (qnz) k_dirac<true><<<blocks, sh.threads, 0, st>>>(g, f, (float)lat->qhat, x0b, nx0, n);
+            else k_dirac<false><<<blocks, sh.threads, 0, st>>>(g, f, 0.f, x0b, nx0, n);
         }
     } else {
-        Fields<double> f{(const double2*)in, (double2*)out, lat->W64, lat->C64};
-        k_dirac<double, false><<<blocks, sh.threads, 0, st>>>(g, f, 0.0, x0b, nx0, n);  // charge in the links
+        return launch_dirac64(lat, lex ? lex_out<double>(out) : full_out<double>(out, g.V),
+                              lex ? lex_ref<double>(in) : full_ref<double>(in, g.V), sh.threads, sh.rows, x0b, nx0, st);
     }
     QXD_LAUNCHED("k_dirac");
     return QXD_OK;
@@ -151,7 +152,7 @@ std::vector<int> window_candidates(const Geom& g) {
 
 // time every candidate shape on this call's input (3 launches each after
 // one untimed launch) and return the fastest
-int tune_dirac(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st, DwShape* best) {
+int tune_dirac(qxd_lattice* lat, void* out, const void* in, int prec, bool lex, cudaStream_t st, DwShape* best) {
     std::vector<DwShape> cand;
     const std::vector<int> rows = window_candidates(lat->g);
     for (int pl = (prec == QXD_FP32 ? 1 : 0); pl >= 0; --pl)
@@ -166,9 +167,9 @@ int tune_dirac(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream
     int rc = QXD_OK;
     best->ms = 0.f;
     for (DwShape& c : cand) {
-        if ((rc = launch_dirac_shape(lat, out, in, prec, c, st))) break;
+        if ((rc = launch_dirac_shape(lat, out, in, prec, c, st, 0, -1, lex))) break;
         cudaEventRecord(e0, st);
-        for (int rep = 0; rep < 3 && !rc; ++rep) rc = launch_dirac_shape(lat, out, in, prec, c, st);
+        for (int rep = 0; rep < 3 && !rc; ++rep) rc = launch_dirac_shape(lat, out, in, prec, c, st, 0, -1, lex);
         if (rc) break;
         cudaEventRecord(e1, st);
         const cudaError_t e = cudaEventSynchronize(e1);
@@ -188,19 +189,35 @@ int tune_dirac(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream
 
 }  // namespace
 
-int launch_dirac(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st) {
+namespace {
+
+int dirac_full(qxd_lattice* lat, void* out, const void* in, int prec, bool lex, cudaStream_t st) {
     const DwKey key = dw_key(lat, prec);
     DwShape sh;
     if (!dw_shape_get(key, &sh)) {
         if (autotune_enabled()) {
-            int rc = tune_dirac(lat, out, in, prec, st, &sh);
+            int rc = tune_dirac(lat, out, in, prec, lex, st, &sh);
             if (rc) return rc;
         } else {
             sh = dw_default_shape(lat, prec);
         }
         dw_shape_put(key, sh, autotune_enabled() ? "tuned" : "default");
     }
-    return launch_dirac_shape(lat, out, in, prec, sh, st);
+    return launch_dirac_shape(lat, out, in, prec, sh, st, 0, -1, lex);
+}
+
+}  // namespace
+
+int launch_dirac(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st) {
+    return dirac_full(lat, out, in, prec, false, st);
+}
+
+bool dirac_takes_lex(const void* out, const void* in, int prec) {
+    return prec == QXD_FP64 && aligned16(out) && aligned16(in);
+}
+
+int launch_dirac_lex(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st) {
+    return dirac_full(lat, out, in, prec, true, st);
 }
 
 int launch_dirac_planes(qxd_lattice* lat, void* out, const void* in, int prec, int x0b, int nx0, cudaStream_t st) {

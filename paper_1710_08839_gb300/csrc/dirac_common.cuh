@@ -21,6 +21,8 @@ struct DwMinBlocks {
     static constexpr int value = sizeof(R) == 4 ? 6 : 4;
 };
 
+constexpr int NUM_SMS = 152;
+
 template <typename R>
 struct Fields;
 

@@ -4,48 +4,46 @@
 //   D_ee = M_ee, D_oo = M_oo, D_eo = H_eo, D_oe = H_oe,
 //   D_hat = M_ee - H_eo M_oo^-1 H_oe   (on the even sites).
 // The kernels below evaluate, for all sites x of one parity p,
-//   HOP              out = H psi
 //   INV_HOP          out = M^-1 (H psi)
 //   CLOVER_AUX_MHOP  out = M aux - H psi
 //   AUX_MHOP         out = aux - H psi
 //   INV_AUX_MHOP     out = M^-1 (aux - H psi)
 //   G5_CLOVER_AUX_MHOP  out = gamma5 (M aux - H psi)
-// where psi lives on the other parity. Each field is addressed as
+// where psi lives on the other parity; in FP32 here, one thread per site, in
+// FP64 in dirac64.cu. Each field is addressed as
 // (pointer, stride, offset): element k of the site with native index s is at
 // p[k * stride + s - offset], so full-lattice arrays (stride V, offset 0)
 // and half-lattice arrays (stride V/2, offset parity * V/2) both work.
 #include <string>
 
 #include "dirac_common.cuh"
+#include "dirac64.cuh"
 #include "eo.cuh"
 
 namespace qxd {
 
 namespace {
 
-template <typename R, bool QNZ, int MODE>
-__global__ void __launch_bounds__(DW_THREADS, DwMinBlocksEo<R>::value)
-    k_dslash_half(Geom g, int p, Fields<R> f, SpRef<R> in, SpRef<R> aux, SpRefOut<R> out,
-                  const typename Fields<R>::cvec* __restrict__ Cl, R q) {
+template <bool QNZ, int MODE>
+__global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<float>::value)
+    k_dslash_half(Geom g, int p, Fields<float> f, SpRef<float> in, SpRef<float> aux, SpRefOut<float> out,
+                  const float4* __restrict__ Cl, float q) {
     const int tau = blockIdx.x * blockDim.x + threadIdx.x;
     if (tau >= g.Vh) return;
     int x0, x1, x2, x3;
     sweep_coords_parity(g, p, tau, x0, x1, x2, x3);
     const int s = native_index(g, lex_index(g, x0, x1, x2, x3), p);
     const int po = 1 - p;
-    cplx<R> acc[12], w[12];
-    dirac_hops<R, QNZ>(g, f, in.p, in.stride, in.off, q, x0, x1, x2, x3, s, po, acc);
-    constexpr R HS = HopScale<R>::value;  // H psi = HS acc
-    if (MODE == EO_HOP) {
-#pragma unroll
-        for (int i = 0; i < 12; ++i) w[i] = HS * acc[i];
-    } else if (MODE == EO_INV_HOP) {
-        cplx<R> t[12];
+    cplx<float> acc[12], w[12];
+    dirac_hops<float, QNZ>(g, f, in.p, in.stride, in.off, q, x0, x1, x2, x3, s, po, acc);
+    constexpr float HS = HopScale<float>::value;  // H psi = HS acc
+    if (MODE == EO_INV_HOP) {
+        cplx<float> t[12];
 #pragma unroll
         for (int i = 0; i < 12; ++i) t[i] = HS * acc[i];
         clover_mul<true>(Cl, g.V, s, t, w);
     } else if (MODE == EO_CLOVER_AUX_MHOP || MODE == EO_G5_CLOVER_AUX_MHOP) {
-        cplx<R> a[12];
+        cplx<float> a[12];
         load_spinor(aux.p, aux.stride, s - aux.off, a);
 #pragma unroll
         for (int i = 0; i < 12; ++i) w[i] = (-HS) * acc[i];
@@ -60,13 +58,18 @@ __global__ void __launch_bounds__(DW_THREADS, DwMinBlocksEo<R>::value)
 #pragma unroll
         for (int i = 0; i < 12; ++i) w[i] = rmad(-HS, acc[i], w[i]);
     } else {  // EO_INV_AUX_MHOP
-        cplx<R> a[12];
+        cplx<float> a[12];
         load_spinor(aux.p, aux.stride, s - aux.off, a);
 #pragma unroll
         for (int i = 0; i < 12; ++i) a[i] = rmad(-HS, acc[i], a[i]);
         clover_mul<true>(Cl, g.V, s, a, w);
     }
     store_spinor(out.p, out.stride, s - out.off, w);
+    if (out.zero_other) {
+#pragma unroll
+        for (int i = 0; i < 12; ++i) w[i] = mk(0.f, 0.f);
+        store_spinor(out.p, out.stride, (p ? s - g.Vh : s + g.Vh) - out.off, w);
+    }
 }
 
 // out = M in (or M^-1 in) on the sites of parity p
@@ -76,25 +79,30 @@ __global__ void k_clover_half(Geom g, int p, SpRef<R> in, SpRefOut<R> out,
     const int h = blockIdx.x * blockDim.x + threadIdx.x;
     if (h >= g.Vh) return;
     const int s = p * g.Vh + h;
+    int lex = 0;
+    if (in.lex || out.lex) {
+        int x0, x1, x2, x3;
+        native_coords(g, s, x0, x1, x2, x3);
+        lex = lex_index(g, x0, x1, x2, x3);
+    }
     cplx<R> a[12], w[12];
-    load_spinor(in.p, in.stride, s - in.off, a);
+    load_spinor(in.p + in.at(lex, s), in.stride, 0, a);
     clover_mul<true>(Cl, g.V, s, a, w);
-    store_spinor(out.p, out.stride, s - out.off, w);
+    store_spinor(out.p + out.at(lex, s), out.stride, 0, w);
 }
 
-template <typename R, bool QNZ>
-int launch_mode(qxd_lattice* lat, int mode, int p, const Fields<R>& f, SpRef<R> in, SpRef<R> aux,
-                SpRefOut<R> out, const typename Fields<R>::cvec* Cl, cudaStream_t st) {
+template <bool QNZ>
+int launch_mode(qxd_lattice* lat, int mode, int p, const Fields<float>& f, SpRef<float> in, SpRef<float> aux,
+                SpRefOut<float> out, const float4* Cl, cudaStream_t st) {
     const Geom& g = lat->g;
     const int blocks = (g.Vh + DW_THREADS - 1) / DW_THREADS;
-    const R q = (R)lat->qhat;
+    const float q = (float)lat->qhat;
     switch (mode) {
-        case EO_HOP: k_dslash_half<R, QNZ, EO_HOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
-        case EO_INV_HOP: k_dslash_half<R, QNZ, EO_INV_HOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
-        case EO_CLOVER_AUX_MHOP: k_dslash_half<R, QNZ, EO_CLOVER_AUX_MHOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
-        case EO_AUX_MHOP: k_dslash_half<R, QNZ, EO_AUX_MHOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
-        case EO_G5_CLOVER_AUX_MHOP: k_dslash_half<R, QNZ, EO_G5_CLOVER_AUX_MHOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
-        default: k_dslash_half<R, QNZ, EO_INV_AUX_MHOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
+        case EO_INV_HOP: k_dslash_half<QNZ, EO_INV_HOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
+        case EO_CLOVER_AUX_MHOP: k_dslash_half<QNZ, EO_CLOVER_AUX_MHOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
+        case EO_AUX_MHOP: k_dslash_half<QNZ, EO_AUX_MHOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
+        case EO_G5_CLOVER_AUX_MHOP: k_dslash_half<QNZ, EO_G5_CLOVER_AUX_MHOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
+        default: k_dslash_half<QNZ, EO_INV_AUX_MHOP><<<blocks, DW_THREADS, 0, st>>>(g, p, f, in, aux, out, Cl, q); break;
     }
     QXD_LAUNCHED("k_dslash_half");
     return QXD_OK;
@@ -102,15 +110,18 @@ int launch_mode(qxd_lattice* lat, int mode, int p, const Fields<R>& f, SpRef<R> 
 
 }  // namespace
 
-template <typename R>
-int launch_eo(qxd_lattice* lat, int mode, int p, SpRef<R> in, SpRef<R> aux, SpRefOut<R> out, bool inverse,
-              cudaStream_t st) {
-    Fields<R> f = fields_of<R>(lat);
-    const typename Fields<R>::cvec* Cl = clover_of<R>(lat, inverse);
-    if constexpr (sizeof(R) == 4) {  // FP64: the charge is in the links
-        if (lat->qhat != 0) return launch_mode<R, true>(lat, mode, p, f, in, aux, out, Cl, st);
-    }
-    return launch_mode<R, false>(lat, mode, p, f, in, aux, out, Cl, st);
+template <>
+int launch_eo<float>(qxd_lattice* lat, int mode, int p, SpRef<float> in, SpRef<float> aux, SpRefOut<float> out,
+                     bool inverse, cudaStream_t st) {
+    const Fields<float> f = fields_of<float>(lat);
+    const float4* Cl = clover_of<float>(lat, inverse);
+    if (lat->qhat != 0) return launch_mode<true>(lat, mode, p, f, in, aux, out, Cl, st);
+    return launch_mode<false>(lat, mode, p, f, in, aux, out, Cl, st);
+}
+template <>
+int launch_eo<double>(qxd_lattice* lat, int mode, int p, SpRef<double> in, SpRef<double> aux, SpRefOut<double> out,
+                      bool inverse, cudaStream_t st) {
+    return launch_eo64(lat, mode, p, in, aux, out, inverse, st);
 }
 
 template <typename R>
@@ -122,8 +133,6 @@ int launch_clover_half(qxd_lattice* lat, int p, SpRef<R> in, SpRefOut<R> out, bo
     return QXD_OK;
 }
 
-template int launch_eo<float>(qxd_lattice*, int, int, SpRef<float>, SpRef<float>, SpRefOut<float>, bool, cudaStream_t);
-template int launch_eo<double>(qxd_lattice*, int, int, SpRef<double>, SpRef<double>, SpRefOut<double>, bool, cudaStream_t);
 template int launch_clover_half<float>(qxd_lattice*, int, SpRef<float>, SpRefOut<float>, bool, cudaStream_t);
 template int launch_clover_half<double>(qxd_lattice*, int, SpRef<double>, SpRefOut<double>, bool, cudaStream_t);
 
@@ -150,31 +159,23 @@ namespace {
 
 enum { EOAPI_DHAT, EOAPI_PREPARE, EOAPI_RECONSTRUCT };
 
-// in/out are full-lattice native arrays
+// in/out are full-lattice arrays, tmp a native one
 template <typename R>
-int eo_native(qxd_lattice* lat, int what, void* out, const void* in, void* tmp, cudaStream_t st) {
+int eo_parts(qxd_lattice* lat, int what, SpRefOut<R> out, SpRef<R> in, void* tmp, cudaStream_t st) {
     const int V = lat->g.V;
     int rc;
-    if (what == EOAPI_DHAT) {
-        // tmp (odd half of a full array) holds M_oo^-1 H_oe in_e
-        if ((rc = apply_dhat<R>(lat, full_out<R>(out, V), full_ref<R>(in, V), full_out<R>(tmp, V), st))) return rc;
-    } else if (what == EOAPI_PREPARE) {
-        if ((rc = launch_clover_half<R>(lat, 1, full_ref<R>(in, V), full_out<R>(tmp, V), true, st))) return rc;
-        if ((rc = launch_eo<R>(lat, EO_AUX_MHOP, 0, full_ref<R>(tmp, V), full_ref<R>(in, V), full_out<R>(out, V),
-                               false, st)))
-            return rc;
-    } else {
-        // out holds x (even part read); in holds b
-        return launch_eo<R>(lat, EO_INV_AUX_MHOP, 1, full_ref<R>(out, V), full_ref<R>(in, V), full_out<R>(out, V),
-                            true, st);
-    }
-    // zero the odd sites of out: native layout keeps each component's odd
-    // sites in one contiguous range
-    const size_t comp = sizeof(R) == 4 ? 6 : 12;
-    const size_t vb = sizeof(typename Fields<R>::vec);
-    for (size_t k = 0; k < comp; ++k)
-        QXD_CUDA(cudaMemsetAsync((char*)out + (k * V + lat->g.Vh) * vb, 0, (size_t)lat->g.Vh * vb, st));
-    return QXD_OK;
+    if (what == EOAPI_RECONSTRUCT)  // out holds x (even part read); in holds b
+        return launch_eo<R>(lat, EO_INV_AUX_MHOP, 1, as_in(out), in, out, true, st);
+    out.zero_other = 1;  // the odd sites of out
+    // tmp (odd half of a full array) holds M_oo^-1 H_oe in_e
+    if (what == EOAPI_DHAT) return apply_dhat<R>(lat, out, in, full_out<R>(tmp, V), st);
+    if ((rc = launch_clover_half<R>(lat, 1, in, full_out<R>(tmp, V), true, st))) return rc;
+    return launch_eo<R>(lat, EO_AUX_MHOP, 0, full_ref<R>(tmp, V), in, out, false, st);
+}
+
+template <typename R>
+int eo_native(qxd_lattice* lat, int what, void* out, const void* in, void* tmp, cudaStream_t st) {
+    return eo_parts<R>(lat, what, full_out<R>(out, lat->g.V), full_ref<R>(in, lat->g.V), tmp, st);
 }
 
 int eo_api(qxd_lattice* lat, int what, void* out, const void* in, int flags, void* stream, const char* name) {
@@ -190,6 +191,9 @@ int eo_api(qxd_lattice* lat, int what, void* out, const void* in, int flags, voi
     if (flags & QXD_LAYOUT_NATIVE)
         return prec == QXD_FP32 ? eo_native<float>(lat, what, out, in, lat->scratch_lex, st)
                                 : eo_native<double>(lat, what, out, in, lat->scratch_lex, st);
+    // FP64: the kernels, bound by arithmetic, read and write the caller's layout
+    if (prec == QXD_FP64 && aligned16(in) && aligned16(out))
+        return eo_parts<double>(lat, what, lex_out<double>(out), lex_ref<double>(in), lat->scratch_lex, st);
     if ((rc = launch_pack(lat, lat->scratch_in, in, prec, st))) return rc;
     if (what == EOAPI_RECONSTRUCT && (rc = launch_pack(lat, lat->scratch_out, out, prec, st))) return rc;
     rc = prec == QXD_FP32 ? eo_native<float>(lat, what, lat->scratch_out, lat->scratch_in, lat->scratch_lex, st)

@@ -5,28 +5,34 @@
 
 namespace qxd {
 
-enum { EO_HOP = 0, EO_INV_HOP = 1, EO_CLOVER_AUX_MHOP = 2, EO_AUX_MHOP = 3, EO_INV_AUX_MHOP = 4,
+enum { EO_INV_HOP = 1, EO_CLOVER_AUX_MHOP = 2, EO_AUX_MHOP = 3, EO_INV_AUX_MHOP = 4,
        EO_G5_CLOVER_AUX_MHOP = 5 };
 
-template <typename R>
-using DwMinBlocksEo = DwMinBlocks<R>;
-
-// spinor field reference: element k of native site s at p[k * stride + s - off]
+// spinor field reference: element k of a site at p[at(lexicographic index,
+// native index) + k * stride]: native fields at p[k * stride + s - off],
+// lexicographic ones (lex = elements per site, stride 1) at p[l * lex + k]
 template <typename R>
 struct SpRef {
     const typename Fields<R>::vec* p = nullptr;
     int stride = 0;
     int off = 0;
+    int lex = 0;
+    __device__ __forceinline__ size_t at(int l, int s) const { return lex ? (size_t)l * lex : (size_t)(s - off); }
 };
+// zero_other: the even-odd kernels also set the other site of each pair
+// (lexicographic indices 2h and 2h + 1: one of each parity) to zero
 template <typename R>
 struct SpRefOut {
     typename Fields<R>::vec* p = nullptr;
     int stride = 0;
     int off = 0;
+    int lex = 0;
+    int zero_other = 0;
+    __device__ __forceinline__ size_t at(int l, int s) const { return lex ? (size_t)l * lex : (size_t)(s - off); }
 };
 template <typename R>
 inline SpRef<R> as_in(SpRefOut<R> o) {
-    return SpRef<R>{o.p, o.stride, o.off};
+    return SpRef<R>{o.p, o.stride, o.off, o.lex};
 }
 // full-lattice native array
 template <typename R>
@@ -37,6 +43,17 @@ template <typename R>
 inline SpRefOut<R> full_out(void* p, int V) {
     return SpRefOut<R>{(typename Fields<R>::vec*)p, V, 0};
 }
+// full-lattice lexicographic array
+template <typename R>
+inline SpRef<R> lex_ref(const void* p) {
+    return SpRef<R>{(const typename Fields<R>::vec*)p, 1, 0, sizeof(R) == 4 ? SPINOR_F4 : SPINOR_D2};
+}
+template <typename R>
+inline SpRefOut<R> lex_out(void* p) {
+    return SpRefOut<R>{(typename Fields<R>::vec*)p, 1, 0, sizeof(R) == 4 ? SPINOR_F4 : SPINOR_D2};
+}
+// the vector loads and stores of lexicographic fields need 16-byte alignment
+inline bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 // half-lattice native array holding the sites of parity par
 template <typename R>
 inline SpRef<R> half_ref(const void* p, int Vh, int par) {

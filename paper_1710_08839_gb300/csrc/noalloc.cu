@@ -59,6 +59,7 @@ int dw_noalloc(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream
     unsigned char* base = nullptr;
     int rc = noalloc_scratch(lat->device, &base);
     if (rc) return rc;
+    if (dirac_takes_lex(out, in, prec)) return launch_dirac_lex(lat, out, in, prec, st);
     unsigned char* nat_in = base;
     unsigned char* nat_out = base + kNoAllocFieldBytes;
     // pack writes every entry of nat_in and the operator every entry of

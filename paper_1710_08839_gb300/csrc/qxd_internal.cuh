@@ -312,6 +312,10 @@ int launch_gauge_ingest(qxd_lattice* lat, const double* su3, const double* ang, 
 int launch_field_tensor(qxd_lattice* lat);
 int launch_clover_build(qxd_lattice* lat, int* d_bad);
 int launch_dirac(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st);
+// D on lexicographic device fields without a change of layout, where the
+// kernel is bound by arithmetic (FP64) and the vector loads are aligned
+bool dirac_takes_lex(const void* out, const void* in, int prec);
+int launch_dirac_lex(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st);
 int launch_pack(qxd_lattice* lat, void* nat, const void* lex, int prec, cudaStream_t st);
 int launch_unpack(qxd_lattice* lat, void* lex, const void* nat, int prec, cudaStream_t st);
 // page-locked host buffers: device address of p (false for pageable memory)
