@@ -329,14 +329,14 @@ int qxd_Dw(qxd_lattice* lat, void* out, const void* in, int flags, void* stream)
             return QXD_OK;
         }
         if (in_pl) {
-            if ((rc = launch_pack_from_host(lat, lat->scratch_in, in_dev, prec, st))) return rc;
+            if ((rc = launch_pack(lat, lat->scratch_in, in_dev, prec, st))) return rc;
         } else {
             QXD_CUDA(cudaMemcpyAsync(lat->scratch_lex, in, bytes, cudaMemcpyHostToDevice, st));
             if ((rc = launch_pack(lat, lat->scratch_in, lat->scratch_lex, prec, st))) return rc;
         }
         if ((rc = launch_dirac(lat, lat->scratch_out, lat->scratch_in, prec, st))) return rc;
         if (out_pl) {
-            if ((rc = launch_unpack_to_host(lat, out_dev, lat->scratch_out, prec, st))) return rc;
+            if ((rc = launch_unpack(lat, out_dev, lat->scratch_out, prec, st))) return rc;
         } else {
             if ((rc = launch_unpack(lat, lat->scratch_lex, lat->scratch_out, prec, st))) return rc;
             QXD_CUDA(cudaMemcpyAsync(out, lat->scratch_lex, bytes, cudaMemcpyDeviceToHost, st));

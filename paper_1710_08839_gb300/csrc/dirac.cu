@@ -71,40 +71,6 @@ __global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<float>::value)
     store_spinor_cs(f.out, g.V, s, acc);
 }
 
-// lexicographic [site][spin][colour][re,im] <-> native structure of arrays
-template <typename R>
-__global__ void k_pack(Geom g, const R* __restrict__ lex, typename Fields<R>::vec* __restrict__ nat) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.V) return;
-    int x0, x1, x2, x3;
-    native_coords(g, s, x0, x1, x2, x3);
-    const size_t l = (size_t)lex_index(g, x0, x1, x2, x3);
-    cplx<R> v[12];
-#pragma unroll
-    for (int i = 0; i < 12; ++i) v[i] = mk(lex[l * 24 + 2 * i], lex[l * 24 + 2 * i + 1]);
-    store_spinor(nat, g.V, s, v);
-}
-
-template <typename R>
-__global__ void k_unpack(Geom g, const typename Fields<R>::vec* __restrict__ nat, R* __restrict__ lex) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.V) return;
-    int x0, x1, x2, x3;
-    native_coords(g, s, x0, x1, x2, x3);
-    const size_t l = (size_t)lex_index(g, x0, x1, x2, x3);
-    cplx<R> v[12];
-    load_spinor(nat, g.V, s, v);
-#pragma unroll
-    for (int i = 0; i < 12; ++i) {
-        lex[l * 24 + 2 * i] = v[i].re;
-        lex[l * 24 + 2 * i + 1] = v[i].im;
-    }
-}
-
-}  // namespace
-
-namespace {
-
 // D with launch shape sh (hop order, threads per block, sweep window) on the
 // x0 planes [x0b, x0b + nx0); lex (FP64 only): lexicographic fields
 int launch_dirac_shape(qxd_lattice* lat, void* out, const void* in, int prec, const DwShape& sh, cudaStream_t st,
@@ -224,24 +190,6 @@ int launch_dirac_planes(qxd_lattice* lat, void* out, const void* in, int prec, i
     DwShape sh;
     if (!dw_shape_get(dw_key(lat, prec), &sh)) sh = dw_default_shape(lat, prec);
     return launch_dirac_shape(lat, out, in, prec, sh, st, x0b, nx0);
-}
-
-int launch_pack(qxd_lattice* lat, void* nat, const void* lex, int prec, cudaStream_t st) {
-    const Geom& g = lat->g;
-    const int blocks = (g.V + 255) / 256;
-    if (prec == QXD_FP32) k_pack<float><<<blocks, 256, 0, st>>>(g, (const float*)lex, (float4*)nat);
-    else k_pack<double><<<blocks, 256, 0, st>>>(g, (const double*)lex, (double2*)nat);
-    QXD_LAUNCHED("k_pack");
-    return QXD_OK;
-}
-
-int launch_unpack(qxd_lattice* lat, void* lex, const void* nat, int prec, cudaStream_t st) {
-    const Geom& g = lat->g;
-    const int blocks = (g.V + 255) / 256;
-    if (prec == QXD_FP32) k_unpack<float><<<blocks, 256, 0, st>>>(g, (const float4*)nat, (float*)lex);
-    else k_unpack<double><<<blocks, 256, 0, st>>>(g, (const double2*)nat, (double*)lex);
-    QXD_LAUNCHED("k_unpack");
-    return QXD_OK;
 }
 
 }  // namespace qxd

@@ -1,10 +1,5 @@
 // Spinor transfer between page-locked host memory and the native device
-// layout without a staging copy: the GPU reads (writes) the caller's
-// lexicographic host buffer directly over the CPU-GPU link while packing
-// (unpacking). One thread per 16-byte element in lexicographic order, so the
-// host side is read and written contiguously; the scattered side is device
-// memory. Used by qxd_Dw when the host buffers are page-locked (registered
-// with or allocated by CUDA); pageable buffers keep the copy path.
+// layout.
 //
 // qxd_Dw with page-locked buffers is pipelined over slabs of x0 planes: a
 // slab is a contiguous range of the lexicographic host buffer. One stream
@@ -25,42 +20,8 @@ namespace qxd {
 
 namespace {
 
-// element i of the lexicographic field: site l = i / C, element k = i % C;
-// native element k of site s is at k * V + s (C = 6 float4 or 12 double2)
-// (elements [i0, i1) of the field)
-template <typename T, int C>
-__global__ void k_pack_from_host(Geom g, const T* __restrict__ lex, T* __restrict__ nat, size_t i0, size_t i1) {
-    for (size_t i = i0 + (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < i1; i += (size_t)gridDim.x * blockDim.x) {
-        const int l = (int)(i / C), k = (int)(i - (size_t)l * C);
-        int r = l;
-        const int x3 = r % g.N3;
-        r /= g.N3;
-        const int x2 = r % g.N2;
-        r /= g.N2;
-        const int x1 = r % g.N1;
-        const int x0 = r / g.N1;
-        const int s = native_index(g, l, (x0 + x1 + x2 + x3) & 1);
-        nat[(size_t)k * g.V + s] = lex[i];
-    }
-}
-
-template <typename T, int C>
-__global__ void k_unpack_to_host(Geom g, const T* __restrict__ nat, T* __restrict__ lex, size_t i0, size_t i1) {
-    for (size_t i = i0 + (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < i1; i += (size_t)gridDim.x * blockDim.x) {
-        const int l = (int)(i / C), k = (int)(i - (size_t)l * C);
-        int r = l;
-        const int x3 = r % g.N3;
-        r /= g.N3;
-        const int x2 = r % g.N2;
-        r /= g.N2;
-        const int x1 = r % g.N1;
-        const int x0 = r / g.N1;
-        const int s = native_index(g, l, (x0 + x1 + x2 + x3) & 1);
-        lex[i] = nat[(size_t)k * g.V + s];
-    }
-}
-
-constexpr unsigned kGrid = 152 * 16;  // 16 blocks of 256 threads per SM
+// blocks of one layout conversion of the pipeline: it takes part of the GPU
+constexpr unsigned kGrid = 152 * 4;
 
 }  // namespace
 
@@ -73,39 +34,6 @@ bool host_device_view(const void* p, void** dev) {
     if (a.type != cudaMemoryTypeHost || !a.devicePointer) return false;
     *dev = a.devicePointer;
     return true;
-}
-
-// sites [s0, s0 + ns) of the lexicographic order (a slab of x0 planes)
-int pack_from_host_sites(qxd_lattice* lat, void* nat, const void* lex_dev, int prec, size_t s0, size_t ns,
-                         unsigned grid, cudaStream_t st) {
-    const Geom& g = lat->g;
-    if (prec == QXD_FP32)
-        k_pack_from_host<float4, 6><<<grid, 256, 0, st>>>(g, (const float4*)lex_dev, (float4*)nat, 6 * s0, 6 * (s0 + ns));
-    else
-        k_pack_from_host<double2, 12><<<grid, 256, 0, st>>>(g, (const double2*)lex_dev, (double2*)nat, 12 * s0,
-                                                             12 * (s0 + ns));
-    QXD_LAUNCHED("k_pack_from_host");
-    return QXD_OK;
-}
-
-int unpack_to_host_sites(qxd_lattice* lat, void* lex_dev, const void* nat, int prec, size_t s0, size_t ns,
-                         unsigned grid, cudaStream_t st) {
-    const Geom& g = lat->g;
-    if (prec == QXD_FP32)
-        k_unpack_to_host<float4, 6><<<grid, 256, 0, st>>>(g, (const float4*)nat, (float4*)lex_dev, 6 * s0, 6 * (s0 + ns));
-    else
-        k_unpack_to_host<double2, 12><<<grid, 256, 0, st>>>(g, (const double2*)nat, (double2*)lex_dev, 12 * s0,
-                                                             12 * (s0 + ns));
-    QXD_LAUNCHED("k_unpack_to_host");
-    return QXD_OK;
-}
-
-int launch_pack_from_host(qxd_lattice* lat, void* nat, const void* lex_dev, int prec, cudaStream_t st) {
-    return pack_from_host_sites(lat, nat, lex_dev, prec, 0, (size_t)lat->g.V, kGrid, st);
-}
-
-int launch_unpack_to_host(qxd_lattice* lat, void* lex_dev, const void* nat, int prec, cudaStream_t st) {
-    return unpack_to_host_sites(lat, lex_dev, nat, prec, 0, (size_t)lat->g.V, kGrid, st);
 }
 
 // streams (host reads, host writes) and events of the pipeline
@@ -166,7 +94,6 @@ int dw_host_pipelined(qxd_lattice* lat, void* out_dev, const void* in_dev, int p
     HostPipe& h = *lat->hostpipe;
     const int planes = g.N0 / S;
     const size_t slab = (size_t)planes * g.N1 * g.N2 * g.N3;
-    const unsigned grid = kGrid / 4;  // each transfer kernel takes part of the GPU
     // the pipeline starts after the work already queued on st
     QXD_CUDA(cudaEventRecord(h.start, st));
     QXD_CUDA(cudaStreamWaitEvent(h.rd, h.start, 0));
@@ -176,7 +103,7 @@ int dw_host_pipelined(qxd_lattice* lat, void* out_dev, const void* in_dev, int p
     for (int k = 0; k < S; ++k) {
         QXD_CUDA(cudaMemcpyAsync((char*)lat->scratch_lex + k * slab * esz, (const char*)in_dev + k * slab * esz,
                                  slab * esz, cudaMemcpyDefault, h.rd));
-        if ((rc = pack_from_host_sites(lat, lat->scratch_in, lat->scratch_lex, prec, k * slab, slab, grid, h.rd)))
+        if ((rc = launch_pack_sites(lat, lat->scratch_in, lat->scratch_lex, prec, k * slab, slab, kGrid, h.rd)))
             return rc;
         QXD_CUDA(cudaEventRecord(h.in[k], h.rd));
     }
@@ -190,8 +117,8 @@ int dw_host_pipelined(qxd_lattice* lat, void* out_dev, const void* in_dev, int p
         if (r) return r;
         QXD_CUDA(cudaEventRecord(h.out[ev], st));
         QXD_CUDA(cudaStreamWaitEvent(h.wr, h.out[ev], 0));
-        if ((r = unpack_to_host_sites(lat, h.stage_out, lat->scratch_out, prec, lo * plane, (hi - lo) * plane, grid,
-                                      h.wr)))
+        if ((r = launch_unpack_sites(lat, h.stage_out, lat->scratch_out, prec, lo * plane, (hi - lo) * plane, kGrid,
+                                     h.wr)))
             return r;
         QXD_CUDA(cudaMemcpyAsync((char*)out_dev + lo * plane * esz, (const char*)h.stage_out + lo * plane * esz,
                                  (hi - lo) * plane * esz, cudaMemcpyDefault, h.wr));

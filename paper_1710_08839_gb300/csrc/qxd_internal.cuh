@@ -318,10 +318,14 @@ bool dirac_takes_lex(const void* out, const void* in, int prec);
 int launch_dirac_lex(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st);
 int launch_pack(qxd_lattice* lat, void* nat, const void* lex, int prec, cudaStream_t st);
 int launch_unpack(qxd_lattice* lat, void* lex, const void* nat, int prec, cudaStream_t st);
+// the same for the lexicographic sites [s0, s0 + ns) (both even) with at most
+// max_blocks thread blocks; lex may be the device address of page-locked host memory
+int launch_pack_sites(qxd_lattice* lat, void* nat, const void* lex, int prec, size_t s0, size_t ns, unsigned max_blocks,
+                      cudaStream_t st);
+int launch_unpack_sites(qxd_lattice* lat, void* lex, const void* nat, int prec, size_t s0, size_t ns,
+                        unsigned max_blocks, cudaStream_t st);
 // page-locked host buffers: device address of p (false for pageable memory)
 bool host_device_view(const void* p, void** dev);
-int launch_pack_from_host(qxd_lattice* lat, void* nat, const void* lex_dev, int prec, cudaStream_t st);
-int launch_unpack_to_host(qxd_lattice* lat, void* lex_dev, const void* nat, int prec, cudaStream_t st);
 // out = D in on the x0 planes [x0b, x0b + nx0) only (native fields; the
 // launch shape of the full-lattice D)
 int launch_dirac_planes(qxd_lattice* lat, void* out, const void* in, int prec, int x0b, int nx0, cudaStream_t st);
