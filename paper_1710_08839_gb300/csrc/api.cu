@@ -311,11 +311,9 @@ int qxd_Dw(qxd_lattice* lat, void* out, const void* in, int flags, void* stream)
     cudaStream_t st = stream ? (cudaStream_t)stream : lat->stream;
     if (out == in) return fail(QXD_ERR_ARG, "qxd_Dw: in and out must not overlap");
     if (native) return launch_dirac(lat, out, in, prec, st);
-    if (!host && dirac_takes_lex(out, in, prec)) return launch_dirac_lex(lat, out, in, prec, st);
-    int rc = ensure_scratch(lat);
-    if (rc) return rc;
+    int rc;
+    if ((host || dirac_lex_needs_scratch(out, in, prec)) && (rc = ensure_scratch(lat))) return rc;
     size_t bytes = qxd_spinor_bytes(lat, prec);
-    const void* lex_in = in;
     if (host) {
         // page-locked buffers are read and written by the kernels directly,
         // pipelined over slabs of x0 planes when both are page-locked;
@@ -344,9 +342,7 @@ int qxd_Dw(qxd_lattice* lat, void* out, const void* in, int flags, void* stream)
         QXD_CUDA(cudaStreamSynchronize(st));
         return QXD_OK;
     }
-    if ((rc = launch_pack(lat, lat->scratch_in, lex_in, prec, st))) return rc;
-    if ((rc = launch_dirac(lat, lat->scratch_out, lat->scratch_in, prec, st))) return rc;
-    return launch_unpack(lat, out, lat->scratch_out, prec, st);
+    return launch_dirac_lex(lat, out, in, lat->scratch_in, lat->scratch_out, prec, st);
 }
 
 }  // extern "C"

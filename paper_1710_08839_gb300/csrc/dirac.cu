@@ -34,45 +34,47 @@ namespace {
 // FP32: the pipelined hop order of hops_pipelined (128 registers)
 template <bool QNZ>
 __global__ void __launch_bounds__(DW_THREADS, DW_PP_MIN_BLOCKS)
-    k_dirac32(Geom g, Fields<float> f, float q, int x0b, int nx0, int nsites) {
+    k_dirac32(Geom g, Fields<float> f, SpRefOut<float> out, float q, int x0b, int nx0, int nsites) {
     const int tau = blockIdx.x * blockDim.x + threadIdx.x;
     if (tau >= nsites) return;
     int x0, x1, x2, x3;
     sweep_coords_slab(g, x0b, nx0, tau, x0, x1, x2, x3);
     const int p = (x0 + x1 + x2 + x3) & 1;
-    const int s = native_index(g, lex_index(g, x0, x1, x2, x3), p);
+    const int lex = lex_index(g, x0, x1, x2, x3);
+    const int s = native_index(g, lex, p);
     int nb[8];
     neighbours8(g, x0, x1, x2, x3, 1 - p, nb);
     cplx<float> acc[12], v[12];
-    hops_pipelined<QNZ>(f, g.V, s, nb, q, acc);
+    hops_pipelined<QNZ>(f, f.psi, g.V, 0, g.V, s, nb, q, acc);
 #pragma unroll
     for (int i = 0; i < 12; ++i) acc[i] = HopScale<float>::value * acc[i];
     load_spinor(f.psi, g.V, s, v);
     clover_mul<true, true>(f.C, g.V, s, v, acc);
-    store_spinor_cs(f.out, g.V, s, acc);
+    store_spinor_cs(out.p + out.at(lex, s), out.stride, 0, acc);
 }
 
 // FP32, the plain hop order (80 registers, 6 blocks per SM)
 template <bool QNZ>
 __global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<float>::value)
-    k_dirac(Geom g, Fields<float> f, float q, int x0b, int nx0, int nsites) {
+    k_dirac(Geom g, Fields<float> f, SpRefOut<float> out, float q, int x0b, int nx0, int nsites) {
     const int tau = blockIdx.x * blockDim.x + threadIdx.x;
     if (tau >= nsites) return;
     int x0, x1, x2, x3;
     sweep_coords_slab(g, x0b, nx0, tau, x0, x1, x2, x3);
     const int p = (x0 + x1 + x2 + x3) & 1;
-    const int s = native_index(g, lex_index(g, x0, x1, x2, x3), p);
+    const int lex = lex_index(g, x0, x1, x2, x3);
+    const int s = native_index(g, lex, p);
     cplx<float> acc[12], v[12];
     dirac_hops<float, QNZ>(g, f, f.psi, g.V, 0, q, x0, x1, x2, x3, s, 1 - p, acc);
 #pragma unroll
     for (int i = 0; i < 12; ++i) acc[i] = HopScale<float>::value * acc[i];
     load_spinor(f.psi, g.V, s, v);
     clover_mul<true, true>(f.C, g.V, s, v, acc);
-    store_spinor_cs(f.out, g.V, s, acc);
+    store_spinor_cs(out.p + out.at(lex, s), out.stride, 0, acc);
 }
 
 // D with launch shape sh (hop order, threads per block, sweep window) on the
-// x0 planes [x0b, x0b + nx0); lex (FP64 only): lexicographic fields
+// x0 planes [x0b, x0b + nx0); lex: lexicographic output, and in FP64 input
 int launch_dirac_shape(qxd_lattice* lat, void* out, const void* in, int prec, const DwShape& sh, cudaStream_t st,
                        int x0b = 0, int nx0 = -1, bool lex = false) {
     Geom g = lat->g;
@@ -82,13 +84,14 @@ int launch_dirac_shape(qxd_lattice* lat, void* out, const void* in, int prec, co
     const int blocks = (n + sh.threads - 1) / sh.threads;
     const bool qnz = lat->qhat != 0;
     if (prec == QXD_FP32) {
-        Fields<float> f{(const float4*)in, (float4*)out, lat->U32, lat->A32, lat->C32};
+        const Fields<float> f{(const float4*)in, nullptr, lat->U32, lat->A32, lat->C32};
+        const SpRefOut<float> o = lex ? lex_out<float>(out) : full_out<float>(out, g.V);
         if (sh.pipelined) {
-            if (qnz) k_dirac32<true><<<blocks, sh.threads, 0, st>>>(g, f, (float)lat->qhat, x0b, nx0, n);
-            else k_dirac32<false><<<blocks, sh.threads, 0, st>>>(g, f, 0.f, x0b, nx0, n);
+            if (qnz) k_dirac32<true><<<blocks, sh.threads, 0, st>>>(g, f, o, (float)lat->qhat, x0b, nx0, n);
+            else k_dirac32<false><<<blocks, sh.threads, 0, st>>>(g, f, o, 0.f, x0b, nx0, n);
         } else {
-            if (qnz) k_dirac<true><<<blocks, sh.threads, 0, st>>>(g, f, (float)lat->qhat, x0b, nx0, n);
-            else k_dirac<false><<<blocks, sh.threads, 0, st>>>(g, f, 0.f, x0b, nx0, n);
+            if (qnz) k_dirac<true><<<blocks, sh.threads, 0, st>>>(g, f, o, (float)lat->qhat, x0b, nx0, n);
+            else k_dirac<false><<<blocks, sh.threads, 0, st>>>(g, f, o, 0.f, x0b, nx0, n);
         }
     } else {
         return launch_dirac64(lat, lex ? lex_out<double>(out) : full_out<double>(out, g.V),
@@ -178,12 +181,21 @@ int launch_dirac(qxd_lattice* lat, void* out, const void* in, int prec, cudaStre
     return dirac_full(lat, out, in, prec, false, st);
 }
 
-bool dirac_takes_lex(const void* out, const void* in, int prec) {
-    return prec == QXD_FP64 && aligned16(out) && aligned16(in);
+// FP64, bound by arithmetic, reads and writes the caller's layout. FP32 gathers
+// each site nine times, which wants the native layout, but writes it once: the
+// input is packed (39 us for 1.3M sites), the output stored in place.
+int launch_dirac_lex(qxd_lattice* lat, void* out, const void* in, void* nat_in, void* nat_out, int prec,
+                     cudaStream_t st) {
+    if (prec == QXD_FP64 && aligned16(out) && aligned16(in)) return dirac_full(lat, out, in, prec, true, st);
+    int rc = launch_pack(lat, nat_in, in, prec, st);
+    if (rc) return rc;
+    if (prec == QXD_FP32 && aligned16(out)) return dirac_full(lat, out, nat_in, prec, true, st);
+    if ((rc = dirac_full(lat, nat_out, nat_in, prec, false, st))) return rc;
+    return launch_unpack(lat, out, nat_out, prec, st);
 }
 
-int launch_dirac_lex(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st) {
-    return dirac_full(lat, out, in, prec, true, st);
+bool dirac_lex_needs_scratch(const void* out, const void* in, int prec) {
+    return !(prec == QXD_FP64 && aligned16(out) && aligned16(in));
 }
 
 int launch_dirac_planes(qxd_lattice* lat, void* out, const void* in, int prec, int x0b, int nx0, cudaStream_t st) {

@@ -350,14 +350,15 @@ __device__ __forceinline__ void neighbours8(const Geom& g, int x0, int x1, int x
 }
 
 // loads of hop k at site s (forward: link and angle of s; backward: of the
-// neighbour sn); a_own = the four angles of s
-__device__ __forceinline__ void hop_load(const Fields<float>& f, int V, int k, int s, int sn, const float4& a_own,
-                                         HopData& d) {
+// neighbour sn); a_own = the four angles of s; psi, pst, poff: the spinors, as
+// in dirac_dir
+__device__ __forceinline__ void hop_load(const Fields<float>& f, const float4* __restrict__ psi, int pst, int poff, int V,
+                                         int k, int s, int sn, const float4& a_own, HopData& d) {
     const int mu = k >> 1;
     const bool fwd = (k & 1) == 0;
     const int sl = fwd ? s : sn;
 #pragma unroll
-    for (int c = 0; c < 6; ++c) d.sp[c] = f.psi[(size_t)c * V + sn];
+    for (int c = 0; c < 6; ++c) d.sp[c] = psi[(size_t)c * pst + (sn - poff)];
 #pragma unroll
     for (int j = 0; j < 3; ++j) d.lk[j] = f.U[((size_t)mu * 3 + j) * V + sl];
     if (fwd) d.ang = mu == 0 ? a_own.x : mu == 1 ? a_own.y : mu == 2 ? a_own.z : a_own.w;
@@ -407,24 +408,24 @@ __device__ __forceinline__ void hop_compute(const HopData& d, float q, cplx<floa
 
 // acc = raw sum of the eight hops at site s with neighbours nb
 template <bool QNZ>
-__device__ __forceinline__ void hops_pipelined(const Fields<float>& f, int V, int s, const int nb[8], float q,
-                                               cplx<float> acc[12]) {
+__device__ __forceinline__ void hops_pipelined(const Fields<float>& f, const float4* __restrict__ psi, int pst,
+                                               int poff, int V, int s, const int nb[8], float q, cplx<float> acc[12]) {
     const float4 a_own = QNZ ? f.A[s] : make_float4(0.f, 0.f, 0.f, 0.f);
     HopData d[2];
-    hop_load(f, V, 0, s, nb[0], a_own, d[0]);
-    hop_load(f, V, 1, s, nb[1], a_own, d[1]);
+    hop_load(f, psi, pst, poff, V, 0, s, nb[0], a_own, d[0]);
+    hop_load(f, psi, pst, poff, V, 1, s, nb[1], a_own, d[1]);
     hop_compute<QNZ, 0, +1, true>(d[0], q, acc);
-    hop_load(f, V, 2, s, nb[2], a_own, d[0]);
+    hop_load(f, psi, pst, poff, V, 2, s, nb[2], a_own, d[0]);
     hop_compute<QNZ, 0, -1>(d[1], q, acc);
-    hop_load(f, V, 3, s, nb[3], a_own, d[1]);
+    hop_load(f, psi, pst, poff, V, 3, s, nb[3], a_own, d[1]);
     hop_compute<QNZ, 1, +1>(d[0], q, acc);
-    hop_load(f, V, 4, s, nb[4], a_own, d[0]);
+    hop_load(f, psi, pst, poff, V, 4, s, nb[4], a_own, d[0]);
     hop_compute<QNZ, 1, -1>(d[1], q, acc);
-    hop_load(f, V, 5, s, nb[5], a_own, d[1]);
+    hop_load(f, psi, pst, poff, V, 5, s, nb[5], a_own, d[1]);
     hop_compute<QNZ, 2, +1>(d[0], q, acc);
-    hop_load(f, V, 6, s, nb[6], a_own, d[0]);
+    hop_load(f, psi, pst, poff, V, 6, s, nb[6], a_own, d[0]);
     hop_compute<QNZ, 2, -1>(d[1], q, acc);
-    hop_load(f, V, 7, s, nb[7], a_own, d[1]);
+    hop_load(f, psi, pst, poff, V, 7, s, nb[7], a_own, d[1]);
     hop_compute<QNZ, 3, +1>(d[0], q, acc);
     hop_compute<QNZ, 3, -1>(d[1], q, acc);
 }

@@ -25,17 +25,19 @@ namespace qxd {
 namespace {
 
 template <bool QNZ, int MODE>
-__global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<float>::value)
+__global__ void __launch_bounds__(DW_THREADS, DW_PP_MIN_BLOCKS)
     k_dslash_half(Geom g, int p, Fields<float> f, SpRef<float> in, SpRef<float> aux, SpRefOut<float> out,
                   const float4* __restrict__ Cl, float q) {
     const int tau = blockIdx.x * blockDim.x + threadIdx.x;
     if (tau >= g.Vh) return;
     int x0, x1, x2, x3;
     sweep_coords_parity(g, p, tau, x0, x1, x2, x3);
-    const int s = native_index(g, lex_index(g, x0, x1, x2, x3), p);
-    const int po = 1 - p;
+    const int lex = lex_index(g, x0, x1, x2, x3);
+    const int s = native_index(g, lex, p);
+    int nb[8];
+    neighbours8(g, x0, x1, x2, x3, 1 - p, nb);
     cplx<float> acc[12], w[12];
-    dirac_hops<float, QNZ>(g, f, in.p, in.stride, in.off, q, x0, x1, x2, x3, s, po, acc);
+    hops_pipelined<QNZ>(f, in.p, in.stride, in.off, g.V, s, nb, q, acc);
     constexpr float HS = HopScale<float>::value;  // H psi = HS acc
     if (MODE == EO_INV_HOP) {
         cplx<float> t[12];
@@ -44,7 +46,7 @@ __global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<float>::value)
         clover_mul<true>(Cl, g.V, s, t, w);
     } else if (MODE == EO_CLOVER_AUX_MHOP || MODE == EO_G5_CLOVER_AUX_MHOP) {
         cplx<float> a[12];
-        load_spinor(aux.p, aux.stride, s - aux.off, a);
+        load_spinor(aux.p + aux.at(lex, s), aux.stride, 0, a);
 #pragma unroll
         for (int i = 0; i < 12; ++i) w[i] = (-HS) * acc[i];
         clover_mul<true, true>(Cl, g.V, s, a, w);
@@ -54,21 +56,21 @@ __global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<float>::value)
             for (int i = 6; i < 12; ++i) w[i] = -w[i];
         }
     } else if (MODE == EO_AUX_MHOP) {
-        load_spinor(aux.p, aux.stride, s - aux.off, w);
+        load_spinor(aux.p + aux.at(lex, s), aux.stride, 0, w);
 #pragma unroll
         for (int i = 0; i < 12; ++i) w[i] = rmad(-HS, acc[i], w[i]);
     } else {  // EO_INV_AUX_MHOP
         cplx<float> a[12];
-        load_spinor(aux.p, aux.stride, s - aux.off, a);
+        load_spinor(aux.p + aux.at(lex, s), aux.stride, 0, a);
 #pragma unroll
         for (int i = 0; i < 12; ++i) a[i] = rmad(-HS, acc[i], a[i]);
         clover_mul<true>(Cl, g.V, s, a, w);
     }
-    store_spinor(out.p, out.stride, s - out.off, w);
+    store_spinor(out.p + out.at(lex, s), out.stride, 0, w);
     if (out.zero_other) {
 #pragma unroll
         for (int i = 0; i < 12; ++i) w[i] = mk(0.f, 0.f);
-        store_spinor(out.p, out.stride, (p ? s - g.Vh : s + g.Vh) - out.off, w);
+        store_spinor(out.p + out.at(lex ^ 1, p ? s - g.Vh : s + g.Vh), out.stride, 0, w);
     }
 }
 
@@ -159,23 +161,45 @@ namespace {
 
 enum { EOAPI_DHAT, EOAPI_PREPARE, EOAPI_RECONSTRUCT };
 
-// in/out are full-lattice arrays, tmp a native one
+// in/out are full-lattice arrays, tmp a native one. gin: the field whose even
+// sites the hops gather (in for D_hat, x for the reconstruction).
 template <typename R>
-int eo_parts(qxd_lattice* lat, int what, SpRefOut<R> out, SpRef<R> in, void* tmp, cudaStream_t st) {
+int eo_parts(qxd_lattice* lat, int what, SpRefOut<R> out, SpRef<R> in, SpRef<R> gin, void* tmp, cudaStream_t st) {
     const int V = lat->g.V;
     int rc;
     if (what == EOAPI_RECONSTRUCT)  // out holds x (even part read); in holds b
-        return launch_eo<R>(lat, EO_INV_AUX_MHOP, 1, as_in(out), in, out, true, st);
+        return launch_eo<R>(lat, EO_INV_AUX_MHOP, 1, gin, in, out, true, st);
     out.zero_other = 1;  // the odd sites of out
-    // tmp (odd half of a full array) holds M_oo^-1 H_oe in_e
-    if (what == EOAPI_DHAT) return apply_dhat<R>(lat, out, in, full_out<R>(tmp, V), st);
+    if (what == EOAPI_DHAT) {  // tmp (odd half of a full array) holds M_oo^-1 H_oe in_e
+        const SpRefOut<R> t = full_out<R>(tmp, V);
+        if ((rc = launch_eo<R>(lat, EO_INV_HOP, 1, gin, SpRef<R>{}, t, true, st))) return rc;
+        return launch_eo<R>(lat, EO_CLOVER_AUX_MHOP, 0, as_in(t), in, out, false, st);
+    }
     if ((rc = launch_clover_half<R>(lat, 1, in, full_out<R>(tmp, V), true, st))) return rc;
     return launch_eo<R>(lat, EO_AUX_MHOP, 0, full_ref<R>(tmp, V), in, out, false, st);
 }
 
 template <typename R>
 int eo_native(qxd_lattice* lat, int what, void* out, const void* in, void* tmp, cudaStream_t st) {
-    return eo_parts<R>(lat, what, full_out<R>(out, lat->g.V), full_ref<R>(in, lat->g.V), tmp, st);
+    const SpRefOut<R> o = full_out<R>(out, lat->g.V);
+    const SpRef<R> i = full_ref<R>(in, lat->g.V);
+    return eo_parts<R>(lat, what, o, i, what == EOAPI_RECONSTRUCT ? as_in(o) : i, tmp, st);
+}
+
+// caller's lexicographic layout read and written in place. FP32: the field
+// that the hops gather is packed first (its even sites), each site of which is
+// read eight times; everything else is read or written once.
+template <typename R>
+int eo_lex(qxd_lattice* lat, int what, void* out, const void* in, cudaStream_t st) {
+    const SpRefOut<R> o = lex_out<R>(out);
+    const SpRef<R> i = lex_ref<R>(in);
+    SpRef<R> gin = what == EOAPI_RECONSTRUCT ? as_in(o) : i;
+    if (sizeof(R) == 4 && what != EOAPI_PREPARE) {
+        const int rc = launch_pack_even(lat, lat->scratch_in, gin.p, QXD_FP32, st);
+        if (rc) return rc;
+        gin = full_ref<R>(lat->scratch_in, lat->g.V);
+    }
+    return eo_parts<R>(lat, what, o, i, gin, lat->scratch_lex, st);
 }
 
 int eo_api(qxd_lattice* lat, int what, void* out, const void* in, int flags, void* stream, const char* name) {
@@ -191,9 +215,8 @@ int eo_api(qxd_lattice* lat, int what, void* out, const void* in, int flags, voi
     if (flags & QXD_LAYOUT_NATIVE)
         return prec == QXD_FP32 ? eo_native<float>(lat, what, out, in, lat->scratch_lex, st)
                                 : eo_native<double>(lat, what, out, in, lat->scratch_lex, st);
-    // FP64: the kernels, bound by arithmetic, read and write the caller's layout
-    if (prec == QXD_FP64 && aligned16(in) && aligned16(out))
-        return eo_parts<double>(lat, what, lex_out<double>(out), lex_ref<double>(in), lat->scratch_lex, st);
+    if (aligned16(in) && aligned16(out))
+        return prec == QXD_FP32 ? eo_lex<float>(lat, what, out, in, st) : eo_lex<double>(lat, what, out, in, st);
     if ((rc = launch_pack(lat, lat->scratch_in, in, prec, st))) return rc;
     if (what == EOAPI_RECONSTRUCT && (rc = launch_pack(lat, lat->scratch_out, out, prec, st))) return rc;
     rc = prec == QXD_FP32 ? eo_native<float>(lat, what, lat->scratch_out, lat->scratch_in, lat->scratch_lex, st)

@@ -59,14 +59,9 @@ int dw_noalloc(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream
     unsigned char* base = nullptr;
     int rc = noalloc_scratch(lat->device, &base);
     if (rc) return rc;
-    if (dirac_takes_lex(out, in, prec)) return launch_dirac_lex(lat, out, in, prec, st);
-    unsigned char* nat_in = base;
-    unsigned char* nat_out = base + kNoAllocFieldBytes;
-    // pack writes every entry of nat_in and the operator every entry of
-    // nat_out, so nothing left by an earlier call is read
-    if ((rc = launch_pack(lat, nat_in, in, prec, st))) return rc;
-    if ((rc = launch_dirac(lat, nat_out, nat_in, prec, st))) return rc;
-    return launch_unpack(lat, out, nat_out, prec, st);
+    // pack writes every entry of the native input and the operator every entry
+    // of its output, so nothing left by an earlier call is read
+    return launch_dirac_lex(lat, out, in, base, base + kNoAllocFieldBytes, prec, st);
 }
 
 }  // namespace

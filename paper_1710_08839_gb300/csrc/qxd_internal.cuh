@@ -312,12 +312,16 @@ int launch_gauge_ingest(qxd_lattice* lat, const double* su3, const double* ang, 
 int launch_field_tensor(qxd_lattice* lat);
 int launch_clover_build(qxd_lattice* lat, int* d_bad);
 int launch_dirac(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st);
-// D on lexicographic device fields without a change of layout, where the
-// kernel is bound by arithmetic (FP64) and the vector loads are aligned
-bool dirac_takes_lex(const void* out, const void* in, int prec);
-int launch_dirac_lex(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st);
+// D on lexicographic device fields; nat_in, nat_out: native scratch fields,
+// used unless the kernels can read and write the caller's layout
+bool dirac_lex_needs_scratch(const void* out, const void* in, int prec);
+int launch_dirac_lex(qxd_lattice* lat, void* out, const void* in, void* nat_in, void* nat_out, int prec,
+                     cudaStream_t st);
 int launch_pack(qxd_lattice* lat, void* nat, const void* lex, int prec, cudaStream_t st);
 int launch_unpack(qxd_lattice* lat, void* lex, const void* nat, int prec, cudaStream_t st);
+// the even sites only (the odd sites of nat are left as they are if lex is
+// 16-byte aligned)
+int launch_pack_even(qxd_lattice* lat, void* nat, const void* lex, int prec, cudaStream_t st);
 // the same for the lexicographic sites [s0, s0 + ns) (both even) with at most
 // max_blocks thread blocks; lex may be the device address of page-locked host memory
 int launch_pack_sites(qxd_lattice* lat, void* nat, const void* lex, int prec, size_t s0, size_t ns, unsigned max_blocks,
