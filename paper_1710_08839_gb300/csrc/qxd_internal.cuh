@@ -270,6 +270,7 @@ struct qxd_lattice {
     float4* A32 = nullptr;   // [V]
     double* ftens = nullptr; // [60][V]
     bool has_gauge = false;
+    bool mirror_built = false;  // mirror half built from the physical one (exact conjugate), not given
 
     // parameters and clover term
     double m0 = 0, csw = 0, cswqed = 0;

@@ -32,6 +32,7 @@
 
 #include "blas.cuh"
 #include "eo.cuh"
+#include "herm6.cuh"
 #include "rhmc.cuh"
 
 namespace qxd {
@@ -103,7 +104,15 @@ __global__ void __launch_bounds__(RED_THREADS) k_sw_logdet(int V, int first, int
 #pragma unroll
         for (int q = 0; q < 15; ++q)
             l[q] = mk(C[(size_t)(36 * blk + 6 + 2 * q) * V + s], C[(size_t)(36 * blk + 7 + 2 * q) * V + s]);
-        const double v = ln_abs_det6(d, l);
+        // well-conditioned blocks: |det| = prod |D_j| without pivoting (the sizes
+        // keep the product in range); others by pivoted elimination
+        double D[6], iD[6], v;
+        C64 L[15];
+        const double nrm = herm6_bound(d, l);
+        if (nrm < 1e40 && nrm > 1e-40 && ldl6(d, l, 0.05 * nrm, D, iD, L))
+            v = log(fabs(D[0] * D[1] * D[2] * D[3] * D[4] * D[5]));
+        else
+            v = ln_abs_det6(d, l);
         if (isfinite(v)) acc[0] += v;
         else acc[1] += 1.0;
     }
