@@ -140,7 +140,11 @@ int qxd_set_params(qxd_lattice* lat, double m0, double csw, double cswqed, int q
  * SAP paths; Sec. 2.4, Doo^-1). Needs qxd_set_gauge and qxd_set_params
  * (else QXD_ERR_STATE). Returns QXD_ERR_SW_SINGULAR if any block is
  * singular to working precision or non-finite (inverse pivots below
- * 1e-12 of the block norm). Synchronises the lattice stream.
+ * 1e-12 of the block norm). On lattices that admit the Schwarz blocks of
+ * qxd_sap it also lays the FP32 operator out block by block for it (504 bytes
+ * per site, allocated by the first build and kept with the lattice; if there
+ * is no memory for it, the first FP32 Schwarz application tries again).
+ * Synchronises the lattice stream.
  */
 int qxd_sw_build(qxd_lattice* lat);
 

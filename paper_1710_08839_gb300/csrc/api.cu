@@ -47,7 +47,7 @@ static int dalloc(T** p, size_t n, const char* what) {
 static void free_all(qxd_lattice* L) {
     release_hostio(L);
     void* own[] = {L->W64, L->C64, L->C32, L->Cinv64, L->Cinv32, L->d_status, L->scratch_in, L->scratch_out,
-                   L->scratch_lex, L->sap_r, L->sap_multi};
+                   L->scratch_lex, L->sap_r, L->sap_multi, L->sap_plan};
     for (void* p : own)
         if (p) cudaFree(p);
     if (L->parent) return;  // the gauge field belongs to the parent
@@ -269,6 +269,12 @@ int qxd_sw_build(qxd_lattice* lat) {
     lat->has_clover = false;
     int rc = launch_clover_build(lat, lat->d_status);
     if (rc) return rc;
+    bool plan = sap_admissible(lat);
+    if (plan && (rc = launch_sap_plan(lat, lat->stream))) {
+        if (rc != QXD_ERR_OOM) return rc;
+        cudaGetLastError();  // the first SAP application tries again
+        plan = false;
+    }
     int st[4];
     cudaError_t e = cudaMemcpyAsync(st, lat->d_status, sizeof(st), cudaMemcpyDeviceToHost, lat->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(lat->stream);
@@ -278,6 +284,7 @@ int qxd_sw_build(qxd_lattice* lat) {
     lat->has_clover = true;
     lat->built_gauge_version = gauge_owner(lat)->gauge_version;
     ++lat->op_version;
+    if (plan) lat->sap_plan_version = lat->op_version;
     return QXD_OK;
 }
 

@@ -92,10 +92,9 @@ __device__ __forceinline__ void store_spinor(double2* __restrict__ p, int V, int
 // ---------------------------------------------------------------------------
 // links
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void load_link(const float4* __restrict__ U, int V, int mu, int s, cplx<float> u[3][3]) {
-    const float4 a = U[((size_t)mu * 3 + 0) * V + s];
-    const float4 b = U[((size_t)mu * 3 + 1) * V + s];
-    const float4 c = U[((size_t)mu * 3 + 2) * V + s];
+// the 3x3 link from its stored rows 0 and 1
+__device__ __forceinline__ void link_rows(const float4 r[3], cplx<float> u[3][3]) {
+    const float4 a = r[0], b = r[1], c = r[2];
     u[0][0] = mk(a.x, a.y);
     u[0][1] = mk(a.z, a.w);
     u[0][2] = mk(b.x, b.y);
@@ -106,6 +105,12 @@ __device__ __forceinline__ void load_link(const float4* __restrict__ U, int V, i
     u[2][0] = conj(u[0][1] * u[1][2] - u[0][2] * u[1][1]);
     u[2][1] = conj(u[0][2] * u[1][0] - u[0][0] * u[1][2]);
     u[2][2] = conj(u[0][0] * u[1][1] - u[0][1] * u[1][0]);
+}
+__device__ __forceinline__ void load_link(const float4* __restrict__ U, int V, int mu, int s, cplx<float> u[3][3]) {
+    float4 r[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r[k] = U[((size_t)mu * 3 + k) * V + s];
+    link_rows(r, u);
 }
 __device__ __forceinline__ void load_link(const double2* __restrict__ U, int V, int mu, int s, cplx<double> u[3][3]) {
 #pragma unroll
@@ -120,13 +125,16 @@ __device__ __forceinline__ void load_link(const double2* __restrict__ U, int V, 
 // few periods are removed) and evaluated with the hardware approximation
 // __sincosf, whose absolute error there is ~1e-6, well inside the FP32
 // tolerance of the operator.
-__device__ __forceinline__ cplx<float> link_phase(const float4* __restrict__ A, int V, int mu, int s, float q) {
-    float t = q * reinterpret_cast<const float*>(A + s)[mu];
+__device__ __forceinline__ cplx<float> angle_phase(float a, float q) {
+    float t = q * a;
     const float k = rintf(t * 0.15915494309189535f);
     t = fmaf(-k, 6.2831853071795865f, t);
     float sn, cs;
     __sincosf(t, &sn, &cs);
     return mk(cs, sn);
+}
+__device__ __forceinline__ cplx<float> link_phase(const float4* __restrict__ A, int V, int mu, int s, float q) {
+    return angle_phase(reinterpret_cast<const float*>(A + s)[mu], q);
 }
 
 template <typename R>
@@ -376,15 +384,7 @@ __device__ __forceinline__ void hop_compute(const HopData& d, float q, cplx<floa
         v[2 * c + 1] = mk(d.sp[c].z, d.sp[c].w);
     }
     project<float, MU, DIR>(v, h0, h1);
-    u[0][0] = mk(d.lk[0].x, d.lk[0].y);
-    u[0][1] = mk(d.lk[0].z, d.lk[0].w);
-    u[0][2] = mk(d.lk[1].x, d.lk[1].y);
-    u[1][0] = mk(d.lk[1].z, d.lk[1].w);
-    u[1][1] = mk(d.lk[2].x, d.lk[2].y);
-    u[1][2] = mk(d.lk[2].z, d.lk[2].w);
-    u[2][0] = conj(u[0][1] * u[1][2] - u[0][2] * u[1][1]);
-    u[2][1] = conj(u[0][2] * u[1][0] - u[0][0] * u[1][2]);
-    u[2][2] = conj(u[0][0] * u[1][1] - u[0][1] * u[1][0]);
+    link_rows(d.lk, u);
     if (DIR > 0) {
         su3_mul(u, h0, g0);
         su3_mul(u, h1, g1);
@@ -393,13 +393,8 @@ __device__ __forceinline__ void hop_compute(const HopData& d, float q, cplx<floa
         su3_dag_mul(u, h1, g1);
     }
     if (QNZ) {
-        // exp(i qhat A), argument reduced to [-pi, pi] as in link_phase
-        float t = q * d.ang;
-        const float kk = rintf(t * 0.15915494309189535f);
-        t = fmaf(-kk, 6.2831853071795865f, t);
-        float sn, cs;
-        __sincosf(t, &sn, &cs);
-        const cplx<float> ph = mk(cs, DIR > 0 ? sn : -sn);
+        cplx<float> ph = angle_phase(d.ang, q);
+        if (DIR < 0) ph = conj(ph);
         times3(ph, g0);
         times3(ph, g1);
     }

@@ -14,7 +14,8 @@
 // Starting from psi = 0, ncy cycles give psi = SAP(eta).
 // FP32, single lattice (k_sap_split): two threads per site pair, the block's
 // interior compound links W' = -1/2 z^qhat U (all three rows) and two block
-// fields in shared memory, the clover blocks read through L1. The residual
+// fields in shared memory, the clover blocks read through L1, both from a
+// block-by-block copy of the operator. The residual
 // of a block is not recomputed from eta - D psi: the even-odd block solve
 // leaves the block residual r_B - D_B delta equal to the MR residual rho on
 // the even sites and to zero on the odd sites (delta_o = M_oo^-1 (r_o - H_oe
@@ -80,6 +81,33 @@ __device__ __forceinline__ Site make_site(const Geom& g, const int org[4], int l
     t.s = native_index(g, lex_index(g, t.x[0], t.x[1], t.x[2], t.x[3]), p);
     return t;
 }
+
+// Block number bidx of the blocks of this colour: blocks (b0, b1, b2, b3e) and
+// (.., b3e + 1), b3e even, are one of each colour. Sets its origin, returns its
+// number among all blocks (lexicographic in block coordinates).
+__device__ __forceinline__ int block_origin(const SapGeom& sg, int bidx, int colour, int org[4]) {
+    const int bi2 = 2 * bidx;
+    const int b3e = bi2 % sg.nb3;
+    int rest = bi2 / sg.nb3;
+    const int b2 = rest % sg.nb2;
+    rest /= sg.nb2;
+    const int b1 = rest % sg.nb1;
+    const int b0 = rest / sg.nb1;
+    const int b3 = b3e + ((b0 + b1 + b2 + b3e + colour) & 1);
+    org[0] = SAP_BS * b0;
+    org[1] = SAP_BS * b1;
+    org[2] = SAP_BS * b2;
+    org[3] = SAP_BS * b3;
+    return bi2 - b3e + b3;
+}
+
+// asynchronous copy of 16 bytes from global to shared memory (past L1), and the
+// wait for this thread's copies
+__device__ __forceinline__ void copy_async16(void* smem, const void* gmem) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // native index of the in-block site one step back in direction MU
 template <int MU>
@@ -191,22 +219,8 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
     const SmemField<R> s_t{sm + 48 * SAP_HALF};     // odd temporary / delta_e at the end
     R* red = sm + 72 * SAP_HALF;                    // 3 * warps reduction slots
 
-    // block of this colour handled by this thread block
     int org[4];
-    {
-        const int bi2 = 2 * bidx;
-        const int b3e = bi2 % sg.nb3;
-        int rest = bi2 / sg.nb3;
-        const int b2 = rest % sg.nb2;
-        rest /= sg.nb2;
-        const int b1 = rest % sg.nb1;
-        const int b0 = rest / sg.nb1;
-        const int b3 = b3e + ((b0 + b1 + b2 + b3e + colour) & 1);
-        org[0] = SAP_BS * b0;
-        org[1] = SAP_BS * b1;
-        org[2] = SAP_BS * b2;
-        org[3] = SAP_BS * b3;
-    }
+    block_origin(sg, bidx, colour, org);
     const int t = threadIdx.x;
     const int base = 2 * t;
     const int par0 = ((base >> 6) + ((base >> 4) & 3) + ((base >> 2) & 3) + (base & 3)) & 1;
@@ -313,6 +327,23 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) k_sap_block(Geom g, SapGeom sg
 // The block's compound links W' = -1/2 z^qhat U are staged once per launch
 // with all three rows, so a hop is a projection, one 3x3 complex product and
 // the accumulation: no third-row rebuild, no U(1) phase, no factor -1/2.
+//
+// What belongs to the operator is laid out block by block when the operator is
+// built (k_sap_plan): the compound interior links as they go into shared
+// memory, and the clover blocks that the block solve uses, M_oo^-1 and M_ee, as
+// float4 [2][18][128] with the block's pairs in order. In the native layout a
+// block's sites come in runs of 32 bytes whose other halves belong to blocks of
+// the other colour: half of every DRAM access and three quarters of every
+// cache line were of no use (64x64x32x32 sites, 5 cycles, 5 MR steps: 16.1 ms
+// without, 14.7 with it; DRAM bytes of a launch on 48x48x24x24 1.15 -> 0.82 GB).
+// The bodies of the block hops and of the crossing hops start with
+// __syncwarp(): left to itself the compiler lets the lanes that skipped a body
+// run ahead through the next ones, and warps took them twice (28 % more
+// shared-memory loads; 14.3 -> 13.1 ms). Measured and not kept: M_oo^-1 resident
+// in shared memory (17 of 18 float4 beside the links: 16.8 ms, the loads move to
+// the shared-memory pipe and L1 shrinks), L1 hints on the clover loads (14.5 and
+// 15.0), L2 prefetch of the own or the next block's data (14.5, 14.7), clover
+// loads before the hops (12.9, within the spread elsewhere).
 // ---------------------------------------------------------------------------
 constexpr int SPLIT_THREADS = 256;
 constexpr unsigned FULL_MASK = 0xffffffffu;
@@ -403,6 +434,8 @@ struct SplitLinks {
     }
 };
 
+constexpr int PLAN_LINK_F4 = 16 * SPLIT_LINKS + 2 * SPLIT_LINKS;  // float4 of one block's links
+constexpr int PLAN_CLOVER_F4 = 2 * CLOVER_F4 * SAP_HALF;          // of its clover blocks
 constexpr size_t split_link_bytes() { return 16 * SPLIT_LINKS * sizeof(float4) + 4 * SPLIT_LINKS * sizeof(float2); }
 
 // Hops of direction MU inside the block for thread sg (sgn = +1 for sg = 0,
@@ -417,6 +450,7 @@ __device__ __forceinline__ void split_dir(const SplitLinks& bl, const float2* sr
     constexpr int stride = MU == 0 ? 64 : MU == 1 ? 16 : MU == 2 ? 4 : 1;
     const int lspin = (MU == 0 || MU == 3) ? 2 + sg : 3 - sg;
     cplx<float> a[3], b[3], h[3], gv[3], u[3][3];
+    __syncwarp();  // one copy of each body per warp
     if (t.l[MU] < SAP_BS - 1) {
         const int slot = (t.lidx + stride) >> 1;
         ld_spin(src, sg, slot, a);
@@ -440,6 +474,7 @@ __device__ __forceinline__ void split_dir(const SplitLinks& bl, const float2* sr
             else al[c] = al[c] - sgn * times_i(gv[c]);
         }
     }
+    __syncwarp();
     if (t.l[MU] > 0) {
         const int slot = (t.lidx - stride) >> 1;
         ld_spin(src, sg, slot, a);
@@ -487,23 +522,24 @@ __device__ __forceinline__ void split_hops(const SplitLinks& bl, const float2* s
     }
 }
 
-// Own rows (3 sg + a, a = 0..2) of both packed Hermitian 6x6 blocks of C at
-// site s times v; v and y are own halves, the partner's half is shuffled in.
+// Own rows (3 sg + a, a = 0..2) of both packed Hermitian 6x6 blocks of a site
+// times v; v and y are own halves, the partner's half is shuffled in. C: the
+// site's first float4 of its block's SAP_HALF-strided matrices.
 // In block order the rows of thread sg see a Hermitian 3x3 diagonal block
 // (entries d[3 sg + a] and L(3 sg + a, 3 sg + b)) and the off-diagonal
 // 3x3 block B[a][b] = L(3 + a, b) for sg = 1, B^+ for sg = 0. Every thread
 // of the warp must call it.
-__device__ __forceinline__ void clover_half(const float4* __restrict__ C, int V, int s, int sg, float sgn,
-                                            const cplx<float> v[6], cplx<float> y[6]) {
+__device__ __forceinline__ void clover_half(const float4* __restrict__ C, int sg, const cplx<float> v[6],
+                                            cplx<float> y[6]) {
     cplx<float> p[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) p[k] = mk(__shfl_xor_sync(FULL_MASK, v[k].re, 1), __shfl_xor_sync(FULL_MASK, v[k].im, 1));
 #pragma unroll
     for (int blk = 0; blk < 2; ++blk) {
-        const float4* Cb = C + (size_t)(9 * blk) * V + s;
-        const float4 q0 = Cb[0], q1 = Cb[(size_t)V], q3 = Cb[(size_t)3 * V], q4 = Cb[(size_t)4 * V];
-        const float4 q5 = Cb[(size_t)5 * V], q6 = Cb[(size_t)6 * V], q7 = Cb[(size_t)7 * V];
-        const float4 X = Cb[(size_t)(sg ? 8 : 2) * V];
+        const float4* Cb = C + 9 * blk * SAP_HALF;
+        const float4 q0 = Cb[0], q1 = Cb[SAP_HALF], q3 = Cb[3 * SAP_HALF], q4 = Cb[4 * SAP_HALF];
+        const float4 q5 = Cb[5 * SAP_HALF], q6 = Cb[6 * SAP_HALF], q7 = Cb[7 * SAP_HALF];
+        const float4 X = Cb[(sg ? 8 : 2) * SAP_HALF];
         // packed floats: d_i at i, L_k at (6 + 2k, 7 + 2k); float4 n holds 4n..4n+3
         const float d0 = sg ? q0.w : q0.x, d1 = sg ? q1.x : q0.y, d2 = sg ? q1.y : q0.z;
         const cplx<float> l10 = sg ? mk(q6.x, q6.y) : mk(q1.z, q1.w);  // L(4,3) : L(1,0)
@@ -531,43 +567,98 @@ __device__ __forceinline__ void clover_half(const float4* __restrict__ C, int V,
         y[3 * blk + 1] = rmad(d1, w[1], z[1]);
         y[3 * blk + 2] = rmad(d2, w[2], z[2]);
     }
-    (void)sgn;
 }
 
-// Hop of D from x to its neighbour x + DIR mu across the face of x's block,
-// applied to the field d (raw: without the factor -1/2), added to acc
-template <bool QNZ, int MU, int DIR>
-__device__ __forceinline__ void crossing_hop(const Geom& g, const Fields<float>& f, const float4* __restrict__ d,
-                                             float q, const Site& t, int po, cplx<float> acc[12]) {
-    cplx<float> v[12], h0[3], h1[3], g0[3], g1[3], u[3][3];
-    const int sn = native_index(g, neighbour_lex<MU, DIR>(g, t.x[0], t.x[1], t.x[2], t.x[3]), po);
-    load_spinor(d, g.V, sn, v);
-    project<float, MU, DIR>(v, h0, h1);
-    const int sl = DIR > 0 ? t.s : sn;  // the link of x forwards, of the neighbour backwards
-    load_link(f.U, g.V, MU, sl, u);
-    if (DIR > 0) {
-        su3_mul(u, h0, g0);
-        su3_mul(u, h1, g1);
-    } else {
-        su3_dag_mul(u, h0, g0);
-        su3_dag_mul(u, h1, g1);
+// The hop of D in direction MU that leaves the block at a site t on one of its
+// two faces in that direction: forwards from the upper face, backwards from the
+// lower one. Both cases run as one body with the sign as a factor and the link
+// transposed where needed, so a warp whose lanes sit on both faces takes 4 hops
+// instead of 8 half-empty ones.
+template <bool QNZ, int MU>
+__device__ __forceinline__ void crossing_load(const Geom& g, const Fields<float>& f, const float4* __restrict__ d,
+                                              const Site& t, int po, HopData& h) {
+    const bool fwd = t.l[MU] == SAP_BS - 1;
+    const int lf = neighbour_lex<MU, +1>(g, t.x[0], t.x[1], t.x[2], t.x[3]);
+    const int lb = neighbour_lex<MU, -1>(g, t.x[0], t.x[1], t.x[2], t.x[3]);
+    const int sn = native_index(g, fwd ? lf : lb, po);
+    const int sl = fwd ? t.s : sn;  // the link of x forwards, of the neighbour backwards
+#pragma unroll
+    for (int c = 0; c < 6; ++c) h.sp[c] = d[(size_t)c * g.V + sn];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) h.lk[k] = f.U[((size_t)MU * 3 + k) * g.V + sl];
+    if (QNZ) h.ang = reinterpret_cast<const float*>(f.A + sl)[MU];
+}
+
+// acc += raw crossing hop (without the factor -1/2) from the loads h
+template <bool QNZ, int MU>
+__device__ __forceinline__ void crossing_add(const HopData& h, float q, const Site& t, cplx<float> acc[12]) {
+    const bool fwd = t.l[MU] == SAP_BS - 1;
+    const float D = fwd ? 1.f : -1.f;
+    cplx<float> v[12], h0[3], h1[3], g0[3], g1[3], u[3][3], w[3][3];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        v[2 * c] = mk(h.sp[c].x, h.sp[c].y);
+        v[2 * c + 1] = mk(h.sp[c].z, h.sp[c].w);
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {  // project<MU, DIR> with DIR = D
+        const cplx<float> a0 = v[c], a1 = v[3 + c], a2 = v[6 + c], a3 = v[9 + c];
+        if (MU == 0) h0[c] = rmad(D, a2, a0), h1[c] = rmad(D, a3, a1);
+        else if (MU == 1) h0[c] = rmad(D, times_i(a3), a0), h1[c] = rmad(D, times_i(a2), a1);
+        else if (MU == 2) h0[c] = rmad(D, a3, a0), h1[c] = rmad(-D, a2, a1);
+        else h0[c] = rmad(D, times_i(a2), a0), h1[c] = rmad(-D, times_i(a3), a1);
+    }
+    link_rows(h.lk, u);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) w[a][b] = mk(fwd ? u[a][b].re : u[b][a].re, fwd ? u[a][b].im : -u[b][a].im);
+    su3_mul(w, h0, g0);
+    su3_mul(w, h1, g1);
     if (QNZ) {
-        const cplx<float> ph0 = link_phase(f.A, g.V, MU, sl, q);
-        const cplx<float> ph = DIR > 0 ? ph0 : conj(ph0);
+        cplx<float> ph = angle_phase(h.ang, q);
+        ph.im *= D;
         times3(ph, g0);
         times3(ph, g1);
     }
-    accumulate<float, MU, DIR>(acc, g0, g1);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {  // accumulate<MU, DIR>
+        acc[c] = acc[c] + g0[c];
+        acc[3 + c] = acc[3 + c] + g1[c];
+        if (MU == 0) acc[6 + c] = rmad(D, g0[c], acc[6 + c]), acc[9 + c] = rmad(D, g1[c], acc[9 + c]);
+        else if (MU == 1) acc[6 + c] = rmad(D, times_mi(g1[c]), acc[6 + c]), acc[9 + c] = rmad(D, times_mi(g0[c]), acc[9 + c]);
+        else if (MU == 2) acc[6 + c] = rmad(-D, g1[c], acc[6 + c]), acc[9 + c] = rmad(D, g0[c], acc[9 + c]);
+        else acc[6 + c] = rmad(D, times_mi(g0[c]), acc[6 + c]), acc[9 + c] = rmad(D, times_i(g1[c]), acc[9 + c]);
+    }
 }
 
-// acc += raw sum of the hops of D at site t that leave its block (t on the
-// upper face in mu: forward hop; on the lower face: backward hop)
-template <bool QNZ, int MU>
-__device__ __forceinline__ void crossing_dir(const Geom& g, const Fields<float>& f, const float4* __restrict__ d,
-                                             float q, const Site& t, int po, cplx<float> acc[12]) {
-    if (t.l[MU] == SAP_BS - 1) crossing_hop<QNZ, MU, +1>(g, f, d, q, t, po, acc);
-    if (t.l[MU] == 0) crossing_hop<QNZ, MU, -1>(g, f, d, q, t, po, acc);
+// raw sum of the hops of D at site t that leave its block
+template <bool QNZ>
+__device__ __forceinline__ void crossing_hops(const Geom& g, const Fields<float>& f, const float4* __restrict__ d,
+                                              float q, const Site& t, int po, cplx<float> acc[12]) {
+    HopData h;
+#pragma unroll
+    for (int i = 0; i < 12; ++i) acc[i] = mk(0.f, 0.f);
+    __syncwarp();
+    if (t.l[0] == SAP_BS - 1 || t.l[0] == 0) {
+        crossing_load<QNZ, 0>(g, f, d, t, po, h);
+        crossing_add<QNZ, 0>(h, q, t, acc);
+    }
+    __syncwarp();
+    if (t.l[1] == SAP_BS - 1 || t.l[1] == 0) {
+        crossing_load<QNZ, 1>(g, f, d, t, po, h);
+        crossing_add<QNZ, 1>(h, q, t, acc);
+    }
+    __syncwarp();
+    if (t.l[2] == SAP_BS - 1 || t.l[2] == 0) {
+        crossing_load<QNZ, 2>(g, f, d, t, po, h);
+        crossing_add<QNZ, 2>(h, q, t, acc);
+    }
+    __syncwarp();
+    if (t.l[3] == SAP_BS - 1 || t.l[3] == 0) {
+        crossing_load<QNZ, 3>(g, f, d, t, po, h);
+        crossing_add<QNZ, 3>(h, q, t, acc);
+    }
 }
 
 // How k_sap_split forms the residual of its blocks and what it keeps
@@ -603,7 +694,7 @@ struct SplitRhsList {
 // the crossing hops of the kept delta.
 template <bool QNZ>
 __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm, int bidx, int colour,
-                                               const Fields<float>& f, const float4* __restrict__ Cinv,
+                                               const Fields<float>& f, const SapPlan& plan,
                                                const SplitWork* rhs, int nrhs, int flags, int nmr, float q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4* sW4 = reinterpret_cast<float4*>(smem_raw);
@@ -614,22 +705,8 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     float2* s_t = sm + 12 * SAP_HALF;   // r on the odd sites, the odd temporary, delta_e at the end
     float* red = reinterpret_cast<float*>(sm + 24 * SAP_HALF);  // 3 * warps reduction slots
 
-    // blocks (b0, b1, b2, b3e) and (.., b3e + 1), b3e even: one of each colour
     int org[4];
-    {
-        const int bi2 = 2 * bidx;
-        const int b3e = bi2 % sgm.nb3;
-        int rest = bi2 / sgm.nb3;
-        const int b2 = rest % sgm.nb2;
-        rest /= sgm.nb2;
-        const int b1 = rest % sgm.nb1;
-        const int b0 = rest / sgm.nb1;
-        const int b3 = b3e + ((b0 + b1 + b2 + b3e + colour) & 1);
-        org[0] = SAP_BS * b0;
-        org[1] = SAP_BS * b1;
-        org[2] = SAP_BS * b2;
-        org[3] = SAP_BS * b3;
-    }
+    const int blk = block_origin(sgm, bidx, colour, org);
     const int t = threadIdx.x >> 1;
     const int sg = threadIdx.x & 1;
     const float sgn = sg ? -1.f : 1.f;
@@ -639,29 +716,13 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     const Site so = make_site(g, org, base + 1 - par0);
     const Site& me = sg ? so : se;  // the site this thread stages, and whose residual it computes
 
-    // compound links W' = -1/2 z^qhat U of this thread's site that stay
-    // inside the block (se has parity 0, so parity sg)
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-        if (me.l[mu] == SAP_BS - 1) continue;
-        const int e = mu == 0   ? link_entry<0>(sg, me.lidx)
-                      : mu == 1 ? link_entry<1>(sg, me.lidx)
-                      : mu == 2 ? link_entry<2>(sg, me.lidx)
-                                : link_entry<3>(sg, me.lidx);
-        cplx<float> u[3][3];
-        load_link(f.U, g.V, mu, me.s, u);
-        cplx<float> z = QNZ ? link_phase(f.A, g.V, mu, me.s, q) : mk(1.f, 0.f);
-        z = -0.5f * z;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) u[a][b] = z * u[a][b];
-        sW4[(mu * 4 + 0) * SPLIT_LINKS + e] = make_float4(u[0][0].re, u[0][0].im, u[0][1].re, u[0][1].im);
-        sW4[(mu * 4 + 1) * SPLIT_LINKS + e] = make_float4(u[0][2].re, u[0][2].im, u[1][0].re, u[1][0].im);
-        sW4[(mu * 4 + 2) * SPLIT_LINKS + e] = make_float4(u[1][1].re, u[1][1].im, u[1][2].re, u[1][2].im);
-        sW4[(mu * 4 + 3) * SPLIT_LINKS + e] = make_float4(u[2][0].re, u[2][0].im, u[2][1].re, u[2][1].im);
-        sW2[mu * SPLIT_LINKS + e] = make_float2(u[2][2].re, u[2][2].im);
+    // the block's links, copied while the residual is formed
+    {
+        const float4* src = plan.links + (size_t)blk * PLAN_LINK_F4;
+        for (int k = threadIdx.x; k < PLAN_LINK_F4; k += SPLIT_THREADS) copy_async16(sW4 + k, src + k);
     }
+    const float4* Moi = plan.clover + (size_t)blk * PLAN_CLOVER_F4 + t;  // M_oo^-1, M_ee of this pair
+    const float4* Mee = Moi + CLOVER_F4 * SAP_HALF;
 
 #pragma unroll 1
     for (int ir = 0; ir < nrhs; ++ir) {
@@ -678,25 +739,21 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
             }
             if (flags & SF_CROSS) {  // r -= D_cross delta = r + 1/2 (crossing hops of delta)
                 cplx<float> acc[12];
-#pragma unroll
-                for (int i = 0; i < 12; ++i) acc[i] = mk(0.f, 0.f);
-                const int po = 1 - sg;  // parity of the neighbours
-                crossing_dir<QNZ, 0>(g, f, wk.delta, q, me, po, acc);
-                crossing_dir<QNZ, 1>(g, f, wk.delta, q, me, po, acc);
-                crossing_dir<QNZ, 2>(g, f, wk.delta, q, me, po, acc);
-                crossing_dir<QNZ, 3>(g, f, wk.delta, q, me, po, acc);
+                crossing_hops<QNZ>(g, f, wk.delta, q, me, 1 - sg, acc);  // neighbours of the other parity
 #pragma unroll
                 for (int i = 0; i < 12; ++i) r[i] = r[i] + 0.5f * acc[i];
             }
             st_full(sg ? s_t : s_rho, t, r);
         }
+        __syncwarp();
+        copy_async_wait();
         __syncthreads();
 
         // r_o (this thread's half) stays in registers until the last step; the
         // pair overwrites its own halves of s_t with t_o = M_oo^-1 r_o
         cplx<float> ro[6], v[6], w[6], acc[6], rho[6];
         ld_half(s_t, sg, t, ro);
-        clover_half(Cinv, g.V, so.s, sg, sgn, ro, w);
+        clover_half(Moi, sg, ro, w);
         st_half(s_t, sg, t, w);
         __syncthreads();
 
@@ -719,14 +776,14 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
             } else if (last) {
 #pragma unroll
                 for (int i = 0; i < 6; ++i) v[i] = ro[i] - acc[i];
-                clover_half(Cinv, g.V, so.s, sg, sgn, v, w);  // delta_o (s_rho is no longer read)
+                clover_half(Moi, sg, v, w);  // delta_o (s_rho is no longer read)
                 st_half(s_rho, sg, t, w);
             } else if (odd) {
-                clover_half(Cinv, g.V, so.s, sg, sgn, acc, w);
+                clover_half(Moi, sg, acc, w);
                 st_half(s_t, sg, t, w);
             } else {
                 ld_half(s_rho, sg, t, rho);
-                clover_half(f.C, g.V, se.s, sg, sgn, rho, w);
+                clover_half(Mee, sg, rho, w);
 #pragma unroll
                 for (int i = 0; i < 6; ++i) w[i] = w[i] - acc[i];
                 float a_re = 0.f, a_im = 0.f, b = 0.f;
@@ -787,10 +844,53 @@ template <bool QNZ, bool MULTI>
 __global__ void __launch_bounds__(SPLIT_THREADS, 2) k_sap_split(const __grid_constant__ Geom g,
                                                                 const __grid_constant__ SapGeom sgm, int colour,
                                                                 const __grid_constant__ Fields<float> f,
-                                                                const float4* __restrict__ Cinv,
+                                                                const __grid_constant__ SapPlan plan,
                                                                 const __grid_constant__ SplitRhsList rl, int flags,
                                                                 int nmr, float q) {
-    sap_split_body<QNZ>(g, sgm, blockIdx.x, colour, f, Cinv, rl.r, MULTI ? rl.n : 1, flags, nmr, q);
+    sap_split_body<QNZ>(g, sgm, blockIdx.x, colour, f, plan, rl.r, MULTI ? rl.n : 1, flags, nmr, q);
+}
+
+// The block-by-block copy of the operator for the split kernel: one thread
+// block per lattice block, thread 2t + sg takes the site of parity sg of pair
+// t (parity 0: links and M_ee, parity 1: links and M_oo^-1).
+template <bool QNZ>
+__global__ void __launch_bounds__(SPLIT_THREADS) k_sap_plan(Geom g, SapGeom sgm, Fields<float> f,
+                                                            const float4* __restrict__ Cinv, float4* __restrict__ links,
+                                                            float4* __restrict__ clover, float q) {
+    int org[4];
+    const int blk = block_origin(sgm, blockIdx.x >> 1, blockIdx.x & 1, org);
+    float4* W4 = links + (size_t)blk * PLAN_LINK_F4;
+    float2* W2 = reinterpret_cast<float2*>(W4 + 16 * SPLIT_LINKS);
+    const int t = threadIdx.x >> 1;
+    const int sg = threadIdx.x & 1;
+    const int base = 2 * t;
+    const int par0 = ((base >> 6) + ((base >> 4) & 3) + ((base >> 2) & 3) + (base & 3)) & 1;
+    const Site me = make_site(g, org, base + (sg ? 1 - par0 : par0));
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        if (me.l[mu] == SAP_BS - 1) continue;
+        const int e = mu == 0   ? link_entry<0>(sg, me.lidx)
+                      : mu == 1 ? link_entry<1>(sg, me.lidx)
+                      : mu == 2 ? link_entry<2>(sg, me.lidx)
+                                : link_entry<3>(sg, me.lidx);
+        cplx<float> u[3][3];
+        load_link(f.U, g.V, mu, me.s, u);
+        cplx<float> z = QNZ ? link_phase(f.A, g.V, mu, me.s, q) : mk(1.f, 0.f);
+        z = -0.5f * z;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) u[a][b] = z * u[a][b];
+        W4[(mu * 4 + 0) * SPLIT_LINKS + e] = make_float4(u[0][0].re, u[0][0].im, u[0][1].re, u[0][1].im);
+        W4[(mu * 4 + 1) * SPLIT_LINKS + e] = make_float4(u[0][2].re, u[0][2].im, u[1][0].re, u[1][0].im);
+        W4[(mu * 4 + 2) * SPLIT_LINKS + e] = make_float4(u[1][1].re, u[1][1].im, u[1][2].re, u[1][2].im);
+        W4[(mu * 4 + 3) * SPLIT_LINKS + e] = make_float4(u[2][0].re, u[2][0].im, u[2][1].re, u[2][1].im);
+        W2[mu * SPLIT_LINKS + e] = make_float2(u[2][2].re, u[2][2].im);
+    }
+    float4* C = clover + (size_t)blk * PLAN_CLOVER_F4 + (sg ? 0 : CLOVER_F4 * SAP_HALF) + t;
+    const float4* src = sg ? Cinv : f.C;
+#pragma unroll
+    for (int n = 0; n < CLOVER_F4; ++n) C[n * SAP_HALF] = src[(size_t)n * g.V + me.s];
 }
 
 // batched form: thread block b works on block (b - cta_begin) of the job
@@ -806,7 +906,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 2) k_sap_block_batch(const SapJ
     }
     const SapJob& J = jobs[lo];
     const SplitWork wk{J.eta, const_cast<float4*>(J.f.psi), J.delta, J.rho};
-    sap_split_body<true>(J.g, J.sg, b - J.cta_begin, colour, J.f, J.Cinv, &wk, 1, flags, nmr, J.q);
+    sap_split_body<true>(J.g, J.sg, b - J.cta_begin, colour, J.f, J.plan, &wk, 1, flags, nmr, J.q);
 }
 
 template <typename R>
@@ -860,10 +960,12 @@ int split_cycles(qxd_lattice* lat, const SapGeom& sg, const SplitRhsList& rl, in
     const size_t smem = sap_smem_bytes<float>();
     int rc = split_attrs(k_sap_split<QNZ, MULTI>, smem);
     if (rc) return rc;
-    const Fields<float> f{nullptr, nullptr, lat->U32, lat->A32, lat->C32};
+    SapPlan plan;
+    if ((rc = sap_plan(lat, st, &plan))) return rc;
+    const Fields<float> f{nullptr, nullptr, lat->U32, lat->A32, nullptr};
     for (int cy = 0; cy < ncy; ++cy)
         for (int colour = 0; colour < 2; ++colour) {
-            k_sap_split<QNZ, MULTI><<<sg.nhalf, SPLIT_THREADS, smem, st>>>(lat->g, sg, colour, f, lat->Cinv32, rl,
+            k_sap_split<QNZ, MULTI><<<sg.nhalf, SPLIT_THREADS, smem, st>>>(lat->g, sg, colour, f, plan, rl,
                                                                            split_flags(cy, colour, ncy), nmr,
                                                                            (float)lat->qhat);
             QXD_LAUNCHED("k_sap_split");
@@ -873,21 +975,65 @@ int split_cycles(qxd_lattice* lat, const SapGeom& sg, const SplitRhsList& rl, in
 
 }  // namespace
 
-int sap_check(qxd_lattice* lat) {
-    const Geom& g = lat->g;
+namespace {
+
+// why the lattice does not admit the block colouring (nullptr: it does)
+const char* sap_refusal(const Geom& g) {
     const int N[4] = {g.N0, g.N1, g.N2, g.N3};
     for (int m = 0; m < 4; ++m)
         if (N[m] % SAP_BS || (N[m] / SAP_BS) % 2)
-            return fail(QXD_ERR_ARG, "SAP: every simulated extent must be a multiple of 8 "
-                                     "(4^4 blocks, even number of blocks per direction)");
+            return "SAP: every simulated extent must be a multiple of 8 "
+                   "(4^4 blocks, even number of blocks per direction)";
     if (g.cs2 || g.cs3) {
-        if (g.L1 % SAP_BS)
-            return fail(QXD_ERR_ARG, "SAP: with C* boundaries L1 must be a multiple of 4");
+        if (g.L1 % SAP_BS) return "SAP: with C* boundaries L1 must be a multiple of 4";
         const int sh = g.L1 / SAP_BS;
         if ((g.cs2 && (N[2] / SAP_BS + sh) % 2) || (g.cs3 && (N[3] / SAP_BS + sh) % 2))
-            return fail(QXD_ERR_ARG, "SAP: the block colouring is not consistent across the shifted "
-                                     "C* boundary (L_k/4 + L1/4 must be even)");
+            return "SAP: the block colouring is not consistent across the shifted "
+                   "C* boundary (L_k/4 + L1/4 must be even)";
     }
+    return nullptr;
+}
+
+}  // namespace
+
+int sap_check(qxd_lattice* lat) {
+    const char* why = sap_refusal(lat->g);
+    return why ? fail(QXD_ERR_ARG, why) : QXD_OK;
+}
+
+int launch_sap_plan(qxd_lattice* lat, cudaStream_t st) {
+    const SapGeom sg = sap_geom(lat->g);
+    if (!lat->sap_plan) {
+        const cudaError_t e =
+            cudaMalloc(&lat->sap_plan, (size_t)sg.nblk * (PLAN_LINK_F4 + PLAN_CLOVER_F4) * sizeof(float4));
+        if (e != cudaSuccess) {
+            lat->sap_plan = nullptr;
+            return cuda_fail(e, "SAP: cudaMalloc(operator by blocks)");
+        }
+    }
+    const Fields<float> f{nullptr, nullptr, lat->U32, lat->A32, lat->C32};
+    float4* clover = lat->sap_plan + (size_t)sg.nblk * PLAN_LINK_F4;
+    if (lat->qhat != 0)
+        k_sap_plan<true><<<sg.nblk, SPLIT_THREADS, 0, st>>>(lat->g, sg, f, lat->Cinv32, lat->sap_plan, clover,
+                                                            (float)lat->qhat);
+    else
+        k_sap_plan<false><<<sg.nblk, SPLIT_THREADS, 0, st>>>(lat->g, sg, f, lat->Cinv32, lat->sap_plan, clover, 0.f);
+    QXD_LAUNCHED("k_sap_plan");
+    return QXD_OK;
+}
+
+// Built with the operator (qxd_sw_build), so that requests on several streams
+// may share it; if there was no memory for it then, by the first application.
+bool sap_admissible(const qxd_lattice* lat) { return !sap_refusal(lat->g); }
+
+int sap_plan(qxd_lattice* lat, cudaStream_t st, SapPlan* plan) {
+    if (!lat->sap_plan || lat->sap_plan_version != lat->op_version) {
+        const int rc = launch_sap_plan(lat, st);
+        if (rc) return rc;
+        lat->sap_plan_version = lat->op_version;
+    }
+    const SapGeom sg = sap_geom(lat->g);
+    *plan = SapPlan{lat->sap_plan, lat->sap_plan + (size_t)sg.nblk * PLAN_LINK_F4};
     return QXD_OK;
 }
 

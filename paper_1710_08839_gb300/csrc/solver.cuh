@@ -21,13 +21,22 @@ struct SapWork {
     SapGeom sg{};
 };
 
+// the operator block by block, for the FP32 block solve (sap.cu): the compound
+// interior links and the clover blocks M_oo^-1, M_ee of every block
+struct SapPlan {
+    const float4* links;
+    const float4* clover;
+};
+// lat's plan, built on st if sw_build had no memory for it
+int sap_plan(qxd_lattice* lat, cudaStream_t st, SapPlan* plan);
+
 // one job of a batched SAP application (FP32): out = SAP(eta) on the job's
 // operator; f.psi is the output field
 struct SapJob {
     Geom g;
     SapGeom sg;
     Fields<float> f;
-    const float4* Cinv;
+    SapPlan plan;
     const float4* eta;
     float4* delta;  // work fields: last block corrections (V sites) and
     float4* rho;    // block residuals of the even sites (Vh), 6 float4 each
