@@ -199,10 +199,9 @@ int qxd_eo_reconstruct(qxd_lattice* lat, void* x, const void* b, int flags, void
 int qxd_sap(qxd_lattice* lat, void* out, const void* in, int ncy, int nmr, int flags, void* stream);
 
 /* out[i] = SAP(in[i]), i < nrhs: the FP32 Schwarz method of qxd_sap for
- * nrhs right-hand sides of the same operator, solved together: each thread
- * block stages the links of its block once and solves the block for each
- * right-hand side in turn (the operator's links and clover blocks are read
- * from DRAM once for all of them). Each out[i] is bit for bit the result of
+ * nrhs right-hand sides of the same operator, solved together: one launch
+ * works on all of them, those of one block side by side, so that the operator's
+ * links and clover blocks are shared in L2. Each out[i] is bit for bit the result of
  * qxd_sap(lat, out[i], in[i], ncy, nmr, QXD_FP32 | QXD_LAYOUT_NATIVE).
  * out and in: host arrays of nrhs device pointers to FP32 fields in the
  * native layout (qxd_spinor_pack); every out[i] distinct and different from

@@ -60,9 +60,9 @@ Deal deal(int n, int threads) {
     const int warps = threads / 32;
     d.full = (n / 16) / SCHEDULERS * SCHEDULERS / warps;
     const int left = n - d.full * warps * 16;
-    // 6 threads per site: one round of 232 instructions, or two when nothing else
-    // runs (two next to full blocks were slower than one round of 552)
-    d.fine = left <= SCHEDULERS * (d.full ? 4 : 8);
+    // 6 threads per site: two rounds of 232 instructions at most, against one of
+    // 552 (next to full blocks too: 41472 sites 97 -> 91 us)
+    d.fine = left <= SCHEDULERS * 8;
     const int chunks = d.fine ? (left + 3) / 4 : (left + 15) / 16;
     d.rest = chunks <= NUM_SMS ? chunks : (chunks + SCHEDULERS - 1) / SCHEDULERS * (SCHEDULERS / warps);
     return d;

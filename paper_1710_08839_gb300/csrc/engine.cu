@@ -326,7 +326,7 @@ struct Engine {
             }
         }
         // phi_k = P(rin); large lattices of one operator (and ncy, nmr) solved
-        // together, each thread block staging its links once for all of them
+        // together
         std::vector<SapJob> sj;
         std::map<std::tuple<qxd_lattice*, int, int>, std::vector<Job*>> same_op;
         for (Job* j : active) {

@@ -679,23 +679,21 @@ struct SplitWork {
     float4* rho;
 };
 
-// right-hand sides of one operator solved in one launch: each thread block
-// stages its block's links once and solves the block for each of them
+// right-hand sides of one operator solved in one launch
 constexpr int SPLIT_MAXR = 12;
 struct SplitRhsList {
     SplitWork r[SPLIT_MAXR];
     int n;
 };
 
-// Same phases as sap_block_body, with the site-pair work split over the
-// two threads of a pair, for the right-hand sides rhs[0 .. nrhs) in turn
-// (the arithmetic of each is the same whatever the others); the residual
-// comes from eta on the first visit of a colour, else from the kept rho and
-// the crossing hops of the kept delta.
+// Same phases as sap_block_body, with the site-pair work split over the two
+// threads of a pair, for one right-hand side; the residual comes from eta on
+// the first visit of a colour, else from the kept rho and the crossing hops of
+// the kept delta.
 template <bool QNZ>
 __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm, int bidx, int colour,
                                                const Fields<float>& f, const SapPlan& plan,
-                                               const SplitWork* rhs, int nrhs, int flags, int nmr, float q) {
+                                               const SplitWork& wk, int flags, int nmr, float q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4* sW4 = reinterpret_cast<float4*>(smem_raw);
     float2* sW2 = reinterpret_cast<float2*>(smem_raw + 16 * SPLIT_LINKS * sizeof(float4));
@@ -724,130 +722,129 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     const float4* Moi = plan.clover + (size_t)blk * PLAN_CLOVER_F4 + t;  // M_oo^-1, M_ee of this pair
     const float4* Mee = Moi + CLOVER_F4 * SAP_HALF;
 
-#pragma unroll 1
-    for (int ir = 0; ir < nrhs; ++ir) {
-        const SplitWork& wk = rhs[ir];
-        {
-            cplx<float> r[12];
-            if (flags & SF_FIRST) {
-                load_spinor(wk.eta, g.V, me.s, r);
-            } else if (sg == 0) {  // even site: the kept rho
-                load_spinor(wk.rho, g.Vh, me.s, r);
-            } else {  // odd site: the block solve left no residual
+    {
+        cplx<float> r[12];
+        if (flags & SF_FIRST) {
+            load_spinor(wk.eta, g.V, me.s, r);
+        } else if (sg == 0) {  // even site: the kept rho
+            load_spinor(wk.rho, g.Vh, me.s, r);
+        } else {  // odd site: the block solve left no residual
 #pragma unroll
-                for (int i = 0; i < 12; ++i) r[i] = mk(0.f, 0.f);
-            }
-            if (flags & SF_CROSS) {  // r -= D_cross delta = r + 1/2 (crossing hops of delta)
-                cplx<float> acc[12];
-                crossing_hops<QNZ>(g, f, wk.delta, q, me, 1 - sg, acc);  // neighbours of the other parity
-#pragma unroll
-                for (int i = 0; i < 12; ++i) r[i] = r[i] + 0.5f * acc[i];
-            }
-            st_full(sg ? s_t : s_rho, t, r);
+            for (int i = 0; i < 12; ++i) r[i] = mk(0.f, 0.f);
         }
-        __syncwarp();
-        copy_async_wait();
-        __syncthreads();
-
-        // r_o (this thread's half) stays in registers until the last step; the
-        // pair overwrites its own halves of s_t with t_o = M_oo^-1 r_o
-        cplx<float> ro[6], v[6], w[6], acc[6], rho[6];
-        ld_half(s_t, sg, t, ro);
-        clover_half(Moi, sg, ro, w);
-        st_half(s_t, sg, t, w);
-        __syncthreads();
-
-        // rho stays in shared memory between steps (fewer live registers)
-        cplx<float> de[6];
+        if (flags & SF_CROSS) {  // r -= D_cross delta = r + 1/2 (crossing hops of delta)
+            cplx<float> acc[12];
+            crossing_hops<QNZ>(g, f, wk.delta, q, me, 1 - sg, acc);  // neighbours of the other parity
 #pragma unroll
-        for (int i = 0; i < 6; ++i) de[i] = mk(0.f, 0.f);
-        const int nsteps = 2 * nmr + 2;
+            for (int i = 0; i < 12; ++i) r[i] = r[i] + 0.5f * acc[i];
+        }
+        st_full(sg ? s_t : s_rho, t, r);
+    }
+    __syncwarp();
+    copy_async_wait();
+    __syncthreads();
+
+    // r_o (this thread's half) stays in registers until the last step; the
+    // pair overwrites its own halves of s_t with t_o = M_oo^-1 r_o
+    cplx<float> ro[6], v[6], w[6], acc[6], rho[6];
+    ld_half(s_t, sg, t, ro);
+    clover_half(Moi, sg, ro, w);
+    st_half(s_t, sg, t, w);
+    __syncthreads();
+
+    // rho stays in shared memory between steps (fewer live registers)
+    cplx<float> de[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) de[i] = mk(0.f, 0.f);
+    const int nsteps = 2 * nmr + 2;
 #pragma unroll 1
-        for (int step = 0; step < nsteps; ++step) {
-            const bool odd = (step & 1) != 0;
-            const bool last = step == nsteps - 1;
-            split_hops<QNZ>(bl, odd ? (last ? s_t : s_rho) : s_t, odd ? so : se, odd ? 1 : 0, sg, sgn, acc);
-            // acc = H psi on the sites of this step's parity (the links carry the -1/2)
-            if (step == 0) {
-                ld_half(s_rho, sg, t, rho);  // r_e
+    for (int step = 0; step < nsteps; ++step) {
+        const bool odd = (step & 1) != 0;
+        const bool last = step == nsteps - 1;
+        split_hops<QNZ>(bl, odd ? (last ? s_t : s_rho) : s_t, odd ? so : se, odd ? 1 : 0, sg, sgn, acc);
+        // acc = H psi on the sites of this step's parity (the links carry the -1/2)
+        if (step == 0) {
+            ld_half(s_rho, sg, t, rho);  // r_e
 #pragma unroll
-                for (int i = 0; i < 6; ++i) rho[i] = rho[i] - acc[i];
-                st_half(s_rho, sg, t, rho);
-            } else if (last) {
+            for (int i = 0; i < 6; ++i) rho[i] = rho[i] - acc[i];
+            st_half(s_rho, sg, t, rho);
+        } else if (last) {
 #pragma unroll
-                for (int i = 0; i < 6; ++i) v[i] = ro[i] - acc[i];
-                clover_half(Moi, sg, v, w);  // delta_o (s_rho is no longer read)
-                st_half(s_rho, sg, t, w);
-            } else if (odd) {
-                clover_half(Moi, sg, acc, w);
-                st_half(s_t, sg, t, w);
-            } else {
-                ld_half(s_rho, sg, t, rho);
-                clover_half(Mee, sg, rho, w);
+            for (int i = 0; i < 6; ++i) v[i] = ro[i] - acc[i];
+            clover_half(Moi, sg, v, w);  // delta_o (s_rho is no longer read)
+            st_half(s_rho, sg, t, w);
+        } else if (odd) {
+            clover_half(Moi, sg, acc, w);
+            st_half(s_t, sg, t, w);
+        } else {
+            ld_half(s_rho, sg, t, rho);
+            clover_half(Mee, sg, rho, w);
 #pragma unroll
-                for (int i = 0; i < 6; ++i) w[i] = w[i] - acc[i];
-                float a_re = 0.f, a_im = 0.f, b = 0.f;
+            for (int i = 0; i < 6; ++i) w[i] = w[i] - acc[i];
+            float a_re = 0.f, a_im = 0.f, b = 0.f;
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                a_re += w[i].re * rho[i].re + w[i].im * rho[i].im;
+                a_im += w[i].re * rho[i].im - w[i].im * rho[i].re;
+                b += w[i].re * w[i].re + w[i].im * w[i].im;
+            }
+            float sums[3];
+            // red is next written two steps later, after the barriers that end each step
+            block_sum3<float, SPLIT_THREADS, false>(a_re, a_im, b, red, sums);
+            if (sums[2] > 0.f) {  // else rho = 0 on the whole block: nothing to add
+                const cplx<float> om = mk(sums[0] / sums[2], sums[1] / sums[2]);
 #pragma unroll
                 for (int i = 0; i < 6; ++i) {
-                    a_re += w[i].re * rho[i].re + w[i].im * rho[i].im;
-                    a_im += w[i].re * rho[i].im - w[i].im * rho[i].re;
-                    b += w[i].re * w[i].re + w[i].im * w[i].im;
-                }
-                float sums[3];
-                // red is next written two steps later, after the barriers that end each step
-                block_sum3<float, SPLIT_THREADS, false>(a_re, a_im, b, red, sums);
-                if (sums[2] > 0.f) {  // else rho = 0 on the whole block: nothing to add
-                    const cplx<float> om = mk(sums[0] / sums[2], sums[1] / sums[2]);
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) {
-                        de[i] = mad(om, rho[i], de[i]);
-                        rho[i] = mad(-om, w[i], rho[i]);
-                    }
-                }
-                if (step == nsteps - 2) {
-                    st_half(s_t, sg, t, de);  // delta_e for the last step
-                    if (flags & SF_KEEP_RHO) {
-                        // this thread's half of rho at the even site: components 3 sg + c and 6 + 3 sg + c
-                        float2* kr = reinterpret_cast<float2*>(wk.rho);
-#pragma unroll
-                        for (int h = 0; h < 2; ++h)
-#pragma unroll
-                            for (int c = 0; c < 3; ++c) {
-                                const int i = 6 * h + 3 * sg + c;
-                                kr[2 * ((size_t)(i >> 1) * g.Vh + se.s) + (i & 1)] = make_float2(rho[3 * h + c].re, rho[3 * h + c].im);
-                            }
-                    }
-                } else {
-                    st_half(s_rho, sg, t, rho);
+                    de[i] = mad(om, rho[i], de[i]);
+                    rho[i] = mad(-om, w[i], rho[i]);
                 }
             }
-            __syncthreads();
-        }
-        // psi_B += delta on this thread's site: delta_e in s_t, delta_o in s_rho
-        cplx<float> d[12];
-        ld_full(sg ? s_rho : s_t, t, d);
-        if (flags & SF_KEEP_DELTA) store_spinor(wk.delta, g.V, me.s, d);
-        if (!(flags & SF_FIRST)) {
-            cplx<float> o[12];
-            load_spinor(wk.psi, g.V, me.s, o);
+            if (step == nsteps - 2) {
+                st_half(s_t, sg, t, de);  // delta_e for the last step
+                if (flags & SF_KEEP_RHO) {
+                    // this thread's half of rho at the even site: components 3 sg + c and 6 + 3 sg + c
+                    float2* kr = reinterpret_cast<float2*>(wk.rho);
 #pragma unroll
-            for (int i = 0; i < 12; ++i) d[i] = d[i] + o[i];
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            const int i = 6 * h + 3 * sg + c;
+                            kr[2 * ((size_t)(i >> 1) * g.Vh + se.s) + (i & 1)] = make_float2(rho[3 * h + c].re, rho[3 * h + c].im);
+                        }
+                }
+            } else {
+                st_half(s_rho, sg, t, rho);
+            }
         }
-        store_spinor(wk.psi, g.V, me.s, d);
-        if (ir + 1 < nrhs) __syncthreads();  // the next right-hand side reuses the block fields
+        __syncthreads();
     }
+    // psi_B += delta on this thread's site: delta_e in s_t, delta_o in s_rho
+    cplx<float> d[12];
+    ld_full(sg ? s_rho : s_t, t, d);
+    if (flags & SF_KEEP_DELTA) store_spinor(wk.delta, g.V, me.s, d);
+    if (!(flags & SF_FIRST)) {
+        cplx<float> o[12];
+        load_spinor(wk.psi, g.V, me.s, o);
+#pragma unroll
+        for (int i = 0; i < 12; ++i) d[i] = d[i] + o[i];
+    }
+    store_spinor(wk.psi, g.V, me.s, d);
 }
 
-// MULTI: several right-hand sides per launch (else exactly one, and the
-// loop over them compiles away)
-template <bool QNZ, bool MULTI>
+// Thread block b: right-hand side b % n of lattice block b / n, so that the
+// right-hand sides of a block run side by side and share its operator data in
+// L2. (One thread block for all right-hand sides of a block, its links staged
+// once, was slower at every size: 6 right-hand sides on 32x32x16x16 946 us each
+// against 818, 12 on 16x16x8x8 269 against 61, where it left SMs idle.)
+template <bool QNZ>
 __global__ void __launch_bounds__(SPLIT_THREADS, 2) k_sap_split(const __grid_constant__ Geom g,
                                                                 const __grid_constant__ SapGeom sgm, int colour,
                                                                 const __grid_constant__ Fields<float> f,
                                                                 const __grid_constant__ SapPlan plan,
                                                                 const __grid_constant__ SplitRhsList rl, int flags,
                                                                 int nmr, float q) {
-    sap_split_body<QNZ>(g, sgm, blockIdx.x, colour, f, plan, rl.r, MULTI ? rl.n : 1, flags, nmr, q);
+    const int b = blockIdx.x / rl.n;
+    sap_split_body<QNZ>(g, sgm, b, colour, f, plan, rl.r[blockIdx.x - b * rl.n], flags, nmr, q);
 }
 
 // The block-by-block copy of the operator for the split kernel: one thread
@@ -906,7 +903,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 2) k_sap_block_batch(const SapJ
     }
     const SapJob& J = jobs[lo];
     const SplitWork wk{J.eta, const_cast<float4*>(J.f.psi), J.delta, J.rho};
-    sap_split_body<true>(J.g, J.sg, b - J.cta_begin, colour, J.f, J.plan, &wk, 1, flags, nmr, J.q);
+    sap_split_body<true>(J.g, J.sg, b - J.cta_begin, colour, J.f, J.plan, wk, flags, nmr, J.q);
 }
 
 template <typename R>
@@ -955,17 +952,17 @@ int launch_sap_block64(qxd_lattice* lat, const SapGeom& sg, int cy, int colour, 
 }
 
 // FP32: the ncy cycles for the right-hand sides of rl (one operator)
-template <bool QNZ, bool MULTI>
+template <bool QNZ>
 int split_cycles(qxd_lattice* lat, const SapGeom& sg, const SplitRhsList& rl, int ncy, int nmr, cudaStream_t st) {
     const size_t smem = sap_smem_bytes<float>();
-    int rc = split_attrs(k_sap_split<QNZ, MULTI>, smem);
+    int rc = split_attrs(k_sap_split<QNZ>, smem);
     if (rc) return rc;
     SapPlan plan;
     if ((rc = sap_plan(lat, st, &plan))) return rc;
     const Fields<float> f{nullptr, nullptr, lat->U32, lat->A32, nullptr};
     for (int cy = 0; cy < ncy; ++cy)
         for (int colour = 0; colour < 2; ++colour) {
-            k_sap_split<QNZ, MULTI><<<sg.nhalf, SPLIT_THREADS, smem, st>>>(lat->g, sg, colour, f, plan, rl,
+            k_sap_split<QNZ><<<sg.nhalf * rl.n, SPLIT_THREADS, smem, st>>>(lat->g, sg, colour, f, plan, rl,
                                                                            split_flags(cy, colour, ncy), nmr,
                                                                            (float)lat->qhat);
             QXD_LAUNCHED("k_sap_split");
@@ -1047,13 +1044,8 @@ int sap_apply_multi(qxd_lattice* lat, int nrhs, void* const* outs, const void* c
         for (int i = 0; i < rl.n; ++i)
             rl.r[i] = SplitWork{(const float4*)ins[i0 + i], (float4*)outs[i0 + i], works[i0 + i],
                                 works[i0 + i] + (size_t)SPINOR_F4 * V};
-        int rc;
-        if (rl.n > 1)
-            rc = lat->qhat != 0 ? split_cycles<true, true>(lat, sg, rl, ncy, nmr, st)
-                                : split_cycles<false, true>(lat, sg, rl, ncy, nmr, st);
-        else
-            rc = lat->qhat != 0 ? split_cycles<true, false>(lat, sg, rl, ncy, nmr, st)
-                                : split_cycles<false, false>(lat, sg, rl, ncy, nmr, st);
+        const int rc = lat->qhat != 0 ? split_cycles<true>(lat, sg, rl, ncy, nmr, st)
+                                      : split_cycles<false>(lat, sg, rl, ncy, nmr, st);
         if (rc) return rc;
     }
     return QXD_OK;

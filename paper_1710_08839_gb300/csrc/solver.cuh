@@ -95,8 +95,8 @@ int sap_check(qxd_lattice* lat);
 template <typename R>
 int sap_apply(qxd_lattice* lat, SapWork& w, void* out, const void* in, int ncy, int nmr, cudaStream_t st);
 // outs[i] = SAP(ins[i]) in FP32 (native layout) for nrhs right-hand sides of
-// the operator lat, solved together (each thread block stages its block's
-// links once for all of them); works[i]: the work fields of right-hand side
+// the operator lat, solved together (one launch per half-cycle for all of
+// them, the operator's data shared in L2); works[i]: the work fields of right-hand side
 // i, (V + Vh) * 6 float4 (delta of every site, then rho of the even sites).
 // Each result is the same as with the right-hand side alone.
 int sap_apply_multi(qxd_lattice* lat, int nrhs, void* const* outs, const void* const* ins, float4* const* works,
