@@ -348,22 +348,27 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) k_sap_block(Geom g, SapGeom sg
 constexpr int SPLIT_THREADS = 256;
 constexpr unsigned FULL_MASK = 0xffffffffu;
 
-// Shared-memory block fields of the split kernel: float2 [12][128], entry
-// (3 spin + colour, pair slot) a complex number, with the slots of spins 1
-// and 3 rotated by 8. The two threads of a pair read the same slot in spins
-// of opposite parity; the rotation puts the eight pairs of a half warp on
-// disjoint halves of the 32 banks.
-__device__ __forceinline__ int spin_slot(int spin, int slot) { return (slot + 8 * (spin & 1)) & (SAP_HALF - 1); }
-__device__ __forceinline__ void ld_spin(const float2* a, int spin, int slot, cplx<float> v[3]) {
-    const float2* p = a + 3 * spin * SAP_HALF + spin_slot(spin, slot);
+// Shared-memory block fields of the split kernel: complex numbers as float2,
+// colour c of spin s of pair slot t at SPIN_STRIDE s + 128 c + t. The stride is
+// 3 x 128 + 8: the two threads of a pair read the same slot in spins of
+// opposite parity, and the 8 puts the eight pairs of a half warp on disjoint
+// halves of the 32 banks. Addresses are linear in the slot, so the hops of a
+// thread are its own base plus constants (a rotation by 8 within rows of 128
+// did the same for the banks at 14 % of all instructions for addresses).
+constexpr int SPIN_STRIDE = 3 * SAP_HALF + 8;
+constexpr int FIELD_F2 = 4 * SPIN_STRIDE;  // float2 of a block field
+__device__ __forceinline__ void ld3(const float2* p, cplx<float> v[3]) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const float2 x = p[c * SAP_HALF];
         v[c] = mk(x.x, x.y);
     }
 }
+__device__ __forceinline__ void ld_spin(const float2* a, int spin, int slot, cplx<float> v[3]) {
+    ld3(a + SPIN_STRIDE * spin + slot, v);
+}
 __device__ __forceinline__ void st_spin(float2* a, int spin, int slot, const cplx<float> v[3]) {
-    float2* p = a + 3 * spin * SAP_HALF + spin_slot(spin, slot);
+    float2* p = a + SPIN_STRIDE * spin + slot;
 #pragma unroll
     for (int c = 0; c < 3; ++c) p[c * SAP_HALF] = make_float2(v[c].re, v[c].im);
 }
@@ -416,12 +421,11 @@ __device__ __forceinline__ int link_entry(int p, int lidx) {
 struct SplitLinks {
     const float4* W4;  // [4][4][192]
     const float2* W2;  // [4][192]
-    __device__ __forceinline__ void link(int mu, int e, cplx<float> u[3][3]) const {
-        const float4 a = W4[(mu * 4 + 0) * SPLIT_LINKS + e];
-        const float4 b = W4[(mu * 4 + 1) * SPLIT_LINKS + e];
-        const float4 c = W4[(mu * 4 + 2) * SPLIT_LINKS + e];
-        const float4 d = W4[(mu * 4 + 3) * SPLIT_LINKS + e];
-        const float2 z = W2[mu * SPLIT_LINKS + e];
+    template <int MU>
+    __device__ __forceinline__ void link(int e, cplx<float> u[3][3]) const {
+        const float4* w = W4 + MU * 4 * SPLIT_LINKS + e;
+        const float4 a = w[0], b = w[SPLIT_LINKS], c = w[2 * SPLIT_LINKS], d = w[3 * SPLIT_LINKS];
+        const float2 z = W2[MU * SPLIT_LINKS + e];
         u[0][0] = mk(a.x, a.y);
         u[0][1] = mk(a.z, a.w);
         u[0][2] = mk(b.x, b.y);
@@ -434,27 +438,52 @@ struct SplitLinks {
     }
 };
 
+// What the hops of a thread need to know of its site pair t: the block
+// coordinates l (l[0..2] are those of both sites), where its spins sit in a
+// block field, and the link entries of its sites without parity
+struct SplitPair {
+    int l0, l1, l2;
+    int par0;       // the even site has local index 2 t + par0
+    int a, b;       // slot t in spin sg, and in spin 3 - sg
+    int e0, e1, e2, e3;
+    __device__ __forceinline__ SplitPair(int t, int sg) {
+        const int base = 2 * t;
+        l0 = base >> 6;
+        l1 = (base >> 4) & 3;
+        l2 = (base >> 2) & 3;
+        par0 = (l0 + l1 + l2 + (base & 3)) & 1;
+        a = SPIN_STRIDE * sg + t;
+        b = SPIN_STRIDE * (3 - sg) + t;
+        e0 = link_entry<0>(0, base);
+        e1 = link_entry<1>(0, base);
+        e2 = link_entry<2>(0, base);
+        e3 = link_entry<3>(0, base);
+    }
+};
+
 constexpr int PLAN_LINK_F4 = 16 * SPLIT_LINKS + 2 * SPLIT_LINKS;  // float4 of one block's links
 constexpr int PLAN_CLOVER_F4 = 2 * CLOVER_F4 * SAP_HALF;          // of its clover blocks
 constexpr size_t split_link_bytes() { return 16 * SPLIT_LINKS * sizeof(float4) + 4 * SPLIT_LINKS * sizeof(float2); }
 
 // Hops of direction MU inside the block for thread sg (sgn = +1 for sg = 0,
-// -1 for sg = 1). With a the neighbour's spin sg and b the lower spin named
-// below, h_sg = a + DIR c_MU b with c_0 = 1, c_1 = i, c_2 = sgn, c_3 = sgn i;
-// g = U h_sg (U^+ backwards) goes to au (upper spin sg) and, times
-// DIR, 1 / -i / sgn / -sgn i for MU = 0..3, to al (lower spin 2 + sg, MU =
-// 0, 3) or ax (lower spin 3 - sg, the partner's, MU = 1, 2).
-template <bool QNZ, int MU>
-__device__ __forceinline__ void split_dir(const SplitLinks& bl, const float2* src, const Site& t, int p, int sg,
-                                          float sgn, cplx<float> au[3], cplx<float> al[3], cplx<float> ax[3]) {
-    constexpr int stride = MU == 0 ? 64 : MU == 1 ? 16 : MU == 2 ? 4 : 1;
-    const int lspin = (MU == 0 || MU == 3) ? 2 + sg : 3 - sg;
+// -1 for sg = 1) at the site of parity p. With a the neighbour's spin sg and b
+// the lower spin named below, h_sg = a + DIR c_MU b with c_0 = 1, c_1 = i, c_2 =
+// sgn, c_3 = sgn i; g = U h_sg (U^+ backwards) goes to au (upper spin sg) and,
+// times DIR, 1 / -i / sgn / -sgn i for MU = 0..3, to al (lower spin 2 + sg, MU =
+// 0, 3) or ax (lower spin 3 - sg, the partner's, MU = 1, 2). l: the site's
+// coordinate; fa, fb: the pair's slot in spins sg and, for MU = 1, 2, 3 - sg of
+// the field; ef, eb: entries of the links at the site and at the site behind it;
+// hop: slots to the next site.
+template <int MU>
+__device__ __forceinline__ void split_dir(const SplitLinks& bl, int l, const float2* fa, const float2* fb, int hopf,
+                                          int hopb, int ef, int eb, float sgn, cplx<float> au[3], cplx<float> al[3],
+                                          cplx<float> ax[3]) {
+    const float2* lower = (MU == 0 || MU == 3) ? fa + 2 * SPIN_STRIDE : fb;
     cplx<float> a[3], b[3], h[3], gv[3], u[3][3];
     __syncwarp();  // one copy of each body per warp
-    if (t.l[MU] < SAP_BS - 1) {
-        const int slot = (t.lidx + stride) >> 1;
-        ld_spin(src, sg, slot, a);
-        ld_spin(src, lspin, slot, b);
+    if (l < SAP_BS - 1) {
+        ld3(fa + hopf, a);
+        ld3(lower + hopf, b);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             if (MU == 0) h[c] = a[c] + b[c];
@@ -462,8 +491,7 @@ __device__ __forceinline__ void split_dir(const SplitLinks& bl, const float2* sr
             else if (MU == 2) h[c] = a[c] + sgn * b[c];
             else h[c] = a[c] + sgn * times_i(b[c]);
         }
-        const int e = link_entry<MU>(p, t.lidx);
-        bl.link(MU, e, u);
+        bl.link<MU>(ef, u);
         su3_mul(u, h, gv);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -475,10 +503,9 @@ __device__ __forceinline__ void split_dir(const SplitLinks& bl, const float2* sr
         }
     }
     __syncwarp();
-    if (t.l[MU] > 0) {
-        const int slot = (t.lidx - stride) >> 1;
-        ld_spin(src, sg, slot, a);
-        ld_spin(src, lspin, slot, b);
+    if (l > 0) {
+        ld3(fa + hopb, a);
+        ld3(lower + hopb, b);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             if (MU == 0) h[c] = a[c] - b[c];
@@ -486,8 +513,7 @@ __device__ __forceinline__ void split_dir(const SplitLinks& bl, const float2* sr
             else if (MU == 2) h[c] = a[c] - sgn * b[c];
             else h[c] = a[c] - sgn * times_i(b[c]);
         }
-        const int e = link_entry<MU>(1 - p, t.lidx - stride);  // link of the neighbour (other parity)
-        bl.link(MU, e, u);
+        bl.link<MU>(eb, u);
         su3_dag_mul(u, h, gv);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -500,19 +526,21 @@ __device__ __forceinline__ void split_dir(const SplitLinks& bl, const float2* sr
     }
 }
 
-// raw block-hop sum at site t, own half (acc[0..2] spin sg, acc[3..5] spin 2 + sg);
-// every thread of the warp must call it (one shuffle at the end)
-// (site t of parity p)
-template <bool QNZ>
-__device__ __forceinline__ void split_hops(const SplitLinks& bl, const float2* src, const Site& t, int p, int sg,
+// raw block-hop sum at the pair's site of parity p (src: field of the other
+// parity), own half (acc[0..2] spin sg, acc[3..5] spin 2 + sg); every thread of
+// the warp must call it (one shuffle at the end)
+__device__ __forceinline__ void split_hops(const SplitLinks& bl, const float2* src, const SplitPair& sp, int t, int p,
                                            float sgn, cplx<float> acc[6]) {
     cplx<float> au[3], al[3], ax[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) au[c] = al[c] = ax[c] = mk(0.f, 0.f);
-    split_dir<QNZ, 0>(bl, src, t, p, sg, sgn, au, al, ax);
-    split_dir<QNZ, 1>(bl, src, t, p, sg, sgn, au, al, ax);
-    split_dir<QNZ, 2>(bl, src, t, p, sg, sgn, au, al, ax);
-    split_dir<QNZ, 3>(bl, src, t, p, sg, sgn, au, al, ax);
+    const float2 *fa = src + sp.a, *fb = src + sp.b;
+    const int d = p ? 1 - sp.par0 : sp.par0;         // the site is 2 t + d
+    const int ef = p * (SPLIT_LINKS / 2), eb = SPLIT_LINKS / 2 - ef;  // entries of this parity and the other
+    split_dir<0>(bl, sp.l0, fa, fb, 32, -32, sp.e0 + ef, sp.e0 + eb - 32, sgn, au, al, ax);
+    split_dir<1>(bl, sp.l1, fa, fb, 8, -8, sp.e1 + ef, sp.e1 + eb - 8, sgn, au, al, ax);
+    split_dir<2>(bl, sp.l2, fa, fb, 2, -2, sp.e2 + ef, sp.e2 + eb - 2, sgn, au, al, ax);
+    split_dir<3>(bl, 2 * (t & 1) + d, fa, fb, d, d - 1, sp.e3 + d, sp.e3 + d - 1, sgn, au, al, ax);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const float xr = __shfl_xor_sync(FULL_MASK, ax[c].re, 1);
@@ -700,19 +728,18 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     const SplitLinks bl{sW4, sW2};
     float2* sm = reinterpret_cast<float2*>(smem_raw + split_link_bytes());
     float2* s_rho = sm;                 // r on the even sites, the MR residual, delta_o at the end
-    float2* s_t = sm + 12 * SAP_HALF;   // r on the odd sites, the odd temporary, delta_e at the end
-    float* red = reinterpret_cast<float*>(sm + 24 * SAP_HALF);  // 3 * warps reduction slots
+    float2* s_t = sm + FIELD_F2;        // r on the odd sites, the odd temporary, delta_e at the end
+    float* red = reinterpret_cast<float*>(sm + 2 * FIELD_F2);  // 3 * warps reduction slots
 
     int org[4];
     const int blk = block_origin(sgm, bidx, colour, org);
     const int t = threadIdx.x >> 1;
     const int sg = threadIdx.x & 1;
     const float sgn = sg ? -1.f : 1.f;
-    const int base = 2 * t;
-    const int par0 = ((base >> 6) + ((base >> 4) & 3) + ((base >> 2) & 3) + (base & 3)) & 1;
-    const Site se = make_site(g, org, base + par0);
-    const Site so = make_site(g, org, base + 1 - par0);
-    const Site& me = sg ? so : se;  // the site this thread stages, and whose residual it computes
+    const SplitPair sp(t, sg);
+    // the site whose residual this thread forms: the even one for sg = 0
+    const Site me = make_site(g, org, 2 * t + (sg ? 1 - sp.par0 : sp.par0));
+    const int even_s = __shfl_sync(FULL_MASK, me.s, threadIdx.x & 30);  // native index of the even site
 
     // the block's links, copied while the residual is formed
     {
@@ -761,7 +788,7 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     for (int step = 0; step < nsteps; ++step) {
         const bool odd = (step & 1) != 0;
         const bool last = step == nsteps - 1;
-        split_hops<QNZ>(bl, odd ? (last ? s_t : s_rho) : s_t, odd ? so : se, odd ? 1 : 0, sg, sgn, acc);
+        split_hops(bl, odd ? (last ? s_t : s_rho) : s_t, sp, t, odd ? 1 : 0, sgn, acc);
         // acc = H psi on the sites of this step's parity (the links carry the -1/2)
         if (step == 0) {
             ld_half(s_rho, sg, t, rho);  // r_e
@@ -809,7 +836,7 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
                             const int i = 6 * h + 3 * sg + c;
-                            kr[2 * ((size_t)(i >> 1) * g.Vh + se.s) + (i & 1)] = make_float2(rho[3 * h + c].re, rho[3 * h + c].im);
+                            kr[2 * ((size_t)(i >> 1) * g.Vh + even_s) + (i & 1)] = make_float2(rho[3 * h + c].re, rho[3 * h + c].im);
                         }
                 }
             } else {
@@ -909,7 +936,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 2) k_sap_block_batch(const SapJ
 template <typename R>
 size_t sap_smem_bytes() {
     if (sizeof(R) == 4)  // split kernel: interior compound links, two block fields, reduction slots of 8 warps
-        return split_link_bytes() + 24 * SAP_HALF * sizeof(float2) + 3 * (SPLIT_THREADS / 32) * sizeof(float);
+        return split_link_bytes() + 2 * FIELD_F2 * sizeof(float2) + 3 * (SPLIT_THREADS / 32) * sizeof(float);
     return (72 * SAP_HALF + 3 * (SAP_THREADS / 32)) * sizeof(R);
 }
 
