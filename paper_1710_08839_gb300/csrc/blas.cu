@@ -31,7 +31,7 @@ __device__ __forceinline__ void st_(double2* p, size_t i, double2 v) { p[i] = v;
 __global__ void __launch_bounds__(RED_FINAL_THREADS) k_reduce_final(const double* __restrict__ partials, int nc,
                                                                      double* __restrict__ res) {
     for (int c = threadIdx.x >> 5; c < nc; c += RED_FINAL_THREADS / 32) {
-        const double x = warp_sum_column(partials, c, RED_BLOCKS);
+        const double x = warp_sum_column(partials, c);
         if ((threadIdx.x & 31) == 0) res[c] = x;
     }
 }
@@ -393,7 +393,6 @@ inline int ew_blocks(size_t n) {
 int reduce_finish(Reducer& red, int nc, cudaStream_t st) {
     k_reduce_final<<<1, RED_FINAL_THREADS, 0, st>>>(red.partials, nc, red.d_res);
     QXD_LAUNCHED("k_reduce_final");
-    QXD_CUDA(cudaMemcpyAsync(red.h_res, red.d_res, nc * sizeof(double), cudaMemcpyDeviceToHost, st));
     QXD_CUDA(cudaStreamSynchronize(st));
     return QXD_OK;
 }
@@ -401,14 +400,13 @@ int reduce_finish(Reducer& red, int nc, cudaStream_t st) {
 int Reducer::init() {
     if (partials) return QXD_OK;
     QXD_CUDA(cudaMalloc(&partials, sizeof(double) * RED_BLOCKS * 2 * BLAS_KMAX));
-    QXD_CUDA(cudaMalloc(&d_res, sizeof(double) * 2 * BLAS_KMAX));
     QXD_CUDA(cudaMallocHost(&h_res, sizeof(double) * 2 * BLAS_KMAX));
+    QXD_CUDA(cudaHostGetDevicePointer((void**)&d_res, h_res, 0));
     return QXD_OK;
 }
 
 void Reducer::release() {
     if (partials) cudaFree(partials);
-    if (d_res) cudaFree(d_res);
     if (h_res) cudaFreeHost(h_res);
     partials = d_res = h_res = nullptr;
 }
@@ -796,7 +794,7 @@ __global__ void __launch_bounds__(RED_FINAL_THREADS) k_reduce_final_batch(const 
                                                                            int nc, double* __restrict__ res) {
     const double* p = partials + (size_t)blockIdx.x * RED_BLOCKS * 2 * BLAS_KMAX;
     for (int c = threadIdx.x >> 5; c < nc; c += RED_FINAL_THREADS / 32) {
-        const double x = warp_sum_column(p, c, RED_BLOCKS);
+        const double x = warp_sum_column(p, c);
         if ((threadIdx.x & 31) == 0) res[(size_t)blockIdx.x * 2 * BLAS_KMAX + c] = x;
     }
 }
@@ -808,8 +806,8 @@ int BatchReducer::ensure(int jobs) {
     release();
     const int c = jobs < 16 ? 16 : jobs;
     QXD_CUDA(cudaMalloc(&partials, sizeof(double) * (size_t)c * RED_BLOCKS * 2 * BLAS_KMAX));
-    QXD_CUDA(cudaMalloc(&d_res, sizeof(double) * (size_t)c * 2 * BLAS_KMAX));
     QXD_CUDA(cudaMallocHost(&h_res, sizeof(double) * (size_t)c * 2 * BLAS_KMAX));
+    QXD_CUDA(cudaHostGetDevicePointer((void**)&d_res, h_res, 0));
     QXD_CUDA(cudaMalloc(&d_jobs, sizeof(BJob) * (size_t)c));
     // pageable on purpose: a copy from pageable memory returns once the data
     // is staged, so the table can be refilled right after a launch
@@ -821,7 +819,6 @@ int BatchReducer::ensure(int jobs) {
 
 void BatchReducer::release() {
     if (partials) cudaFree(partials);
-    if (d_res) cudaFree(d_res);
     if (h_res) cudaFreeHost(h_res);
     if (d_jobs) cudaFree(d_jobs);
     delete[] h_jobs;
@@ -855,8 +852,6 @@ int blas_batch(BatchReducer& red, BOp op, int jobs, int nc, cudaStream_t st) {
     if (!reduce) return QXD_OK;
     k_reduce_final_batch<<<jobs, RED_FINAL_THREADS, 0, st>>>(red.partials, nc, red.d_res);
     QXD_LAUNCHED("k_reduce_final_batch");
-    QXD_CUDA(cudaMemcpyAsync(red.h_res, red.d_res, sizeof(double) * (size_t)jobs * 2 * BLAS_KMAX,
-                             cudaMemcpyDeviceToHost, st));
     QXD_CUDA(cudaStreamSynchronize(st));
     return QXD_OK;
 }

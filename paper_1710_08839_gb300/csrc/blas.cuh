@@ -27,8 +27,8 @@ struct CoefList {
 // device workspace of the reductions
 struct Reducer {
     double* partials = nullptr;  // [RED_BLOCKS][2 * BLAS_KMAX]
-    double* d_res = nullptr;     // [2 * BLAS_KMAX]
-    double* h_res = nullptr;     // pinned host copy
+    double* h_res = nullptr;     // [2 * BLAS_KMAX], page-locked; the last kernel of a reduction writes it
+    double* d_res = nullptr;     // its device address (a copy instead cost 1.4 us and a launch per reduction)
     int init();
     void release();
 };
@@ -69,11 +69,27 @@ __device__ __forceinline__ double warp_sum_column(const double* __restrict__ par
     return x;
 }
 
+// the same for RED_BLOCKS rows, with every load in flight at once
+__device__ __forceinline__ double warp_sum_column(const double* __restrict__ partials, int c) {
+    static_assert(RED_BLOCKS % 32 == 0, "equal rows per lane");
+    const int lane = threadIdx.x & 31;
+    double v[RED_BLOCKS / 32], x = 0.0;
+#pragma unroll
+    for (int i = 0; i < RED_BLOCKS / 32; ++i) v[i] = __ldcg(partials + (size_t)(lane + 32 * i) * 2 * BLAS_KMAX + c);
+#pragma unroll
+    for (int i = 0; i < RED_BLOCKS / 32; ++i) x += v[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
 // threads of the final reduction: one warp per column, columns taken in turn
 constexpr int RED_FINAL_THREADS = 256;
 
 // sums the RED_BLOCKS partials of the first nc values in a fixed order into
-// red.h_res[0..nc) (synchronises the stream)
+// red.h_res[0..nc) (synchronises the stream). A kernel of its own: with the last
+// block of the reducing kernel doing it behind a fence, that kernel took 10 us
+// longer, more than this one takes.
 int reduce_finish(Reducer& red, int nc, cudaStream_t st);
 
 // out[j] = <x_j, y> = sum conj(x_j) y, j < k   (synchronises the stream)
@@ -129,8 +145,8 @@ struct BJob {
 
 struct BatchReducer {
     double* partials = nullptr;  // [jobs][RED_BLOCKS][2 KMAX]
-    double* d_res = nullptr;     // [jobs][2 KMAX]
-    double* h_res = nullptr;     // pinned
+    double* h_res = nullptr;     // [jobs][2 KMAX], page-locked, written by the last kernel of a reduction
+    double* d_res = nullptr;     // its device address
     BJob* d_jobs = nullptr;
     BJob* h_jobs = nullptr;      // host copy of the job table (pageable)
     int cap = 0;
