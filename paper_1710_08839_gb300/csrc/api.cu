@@ -44,15 +44,45 @@ static int dalloc(T** p, size_t n, const char* what) {
     return QXD_OK;
 }
 
+// One allocation for several arrays (a cudaMalloc costs tens of microseconds,
+// more than most kernels of a small lattice), each at a multiple of 256 bytes
+struct Piece {
+    void** p;
+    size_t bytes;
+};
+static int alloc_pieces(void** arena, const Piece* pieces, int n, const char* what) {
+    size_t total = 0;
+    for (int i = 0; i < n; ++i) total += (pieces[i].bytes + 255) / 256 * 256;
+    const int rc = dalloc((char**)arena, total, what);
+    if (rc) return rc;
+    char* at = (char*)*arena;
+    for (int i = 0; i < n; ++i) {
+        *pieces[i].p = at;
+        at += (pieces[i].bytes + 255) / 256 * 256;
+    }
+    return QXD_OK;
+}
+
+// the arrays of the operator (lattices and views) and of the gauge field
+static int alloc_fields(qxd_lattice* L, bool gauge) {
+    const size_t v = (size_t)L->g.V;
+    const Piece op[] = {{(void**)&L->W64, 4 * 9 * v * sizeof(double2)}, {(void**)&L->C64, CLOVER_REALS * v * sizeof(double)},
+                        {(void**)&L->C32, CLOVER_F4 * v * sizeof(float4)}, {(void**)&L->Cinv64, CLOVER_REALS * v * sizeof(double)},
+                        {(void**)&L->Cinv32, CLOVER_F4 * v * sizeof(float4)}, {(void**)&L->d_status, 64 * sizeof(int)}};
+    const Piece ga[] = {{(void**)&L->U64, 4 * 9 * v * sizeof(double2)}, {(void**)&L->U32, 4 * 3 * v * sizeof(float4)},
+                        {(void**)&L->A64, 4 * v * sizeof(double)}, {(void**)&L->Z64, 4 * v * sizeof(double2)},
+                        {(void**)&L->A32, v * sizeof(float4)}, {(void**)&L->ftens, FTENS_REALS * v * sizeof(double)}};
+    int rc = alloc_pieces(&L->op_arena, op, 6, "cudaMalloc(operator)");
+    if (!rc && gauge) rc = alloc_pieces(&L->gauge_arena, ga, 6, "cudaMalloc(gauge field)");
+    return rc;
+}
+
 static void free_all(qxd_lattice* L) {
     release_hostio(L);
-    void* own[] = {L->W64, L->C64, L->C32, L->Cinv64, L->Cinv32, L->d_status, L->scratch_in, L->scratch_out,
-                   L->scratch_lex, L->sap_r, L->sap_multi, L->sap_plan};
+    // gauge_arena is null in a view: the gauge field belongs to the parent
+    void* own[] = {L->op_arena, L->gauge_arena, L->scratch_in, L->scratch_out, L->scratch_lex, L->sap_r, L->sap_multi,
+                   L->sap_plan};
     for (void* p : own)
-        if (p) cudaFree(p);
-    if (L->parent) return;  // the gauge field belongs to the parent
-    void* gauge[] = {L->U64, L->U32, L->A64, L->Z64, L->A32, L->ftens};
-    for (void* p : gauge)
         if (p) cudaFree(p);
 }
 
@@ -114,20 +144,8 @@ int qxd_lattice_create(qxd_lattice** out, int T, int L1, int L2, int L3, unsigne
         delete lat;
         return cuda_fail(e, "cudaGetDevice");
     }
-    size_t v = (size_t)V;
-    int rc = 0;
-    if ((rc = dalloc(&lat->U64, 4 * 9 * v, "cudaMalloc(U64)")) ||
-        (rc = dalloc(&lat->U32, 4 * 3 * v, "cudaMalloc(U32)")) ||
-        (rc = dalloc(&lat->A64, 4 * v, "cudaMalloc(A64)")) ||
-        (rc = dalloc(&lat->Z64, 4 * v, "cudaMalloc(Z64)")) ||
-        (rc = dalloc(&lat->A32, v, "cudaMalloc(A32)")) ||
-        (rc = dalloc(&lat->ftens, FTENS_REALS * v, "cudaMalloc(ftens)")) ||
-        (rc = dalloc(&lat->W64, 4 * 9 * v, "cudaMalloc(W64)")) ||
-        (rc = dalloc(&lat->C64, CLOVER_REALS * v, "cudaMalloc(C64)")) ||
-        (rc = dalloc(&lat->C32, CLOVER_F4 * v, "cudaMalloc(C32)")) ||
-        (rc = dalloc(&lat->Cinv64, CLOVER_REALS * v, "cudaMalloc(Cinv64)")) ||
-        (rc = dalloc(&lat->Cinv32, CLOVER_F4 * v, "cudaMalloc(Cinv32)")) ||
-        (rc = dalloc(&lat->d_status, 64, "cudaMalloc(status)"))) {
+    const int rc = alloc_fields(lat, true);
+    if (rc) {
         free_all(lat);
         delete lat;
         return rc;
@@ -184,14 +202,8 @@ int qxd_lattice_view(qxd_lattice** out, qxd_lattice* parent, void* stream) {
     v->A32 = root->A32;
     v->ftens = root->ftens;
     v->parent = root;
-    size_t n = (size_t)root->g.V;
-    int rc = 0;
-    if ((rc = dalloc(&v->W64, 4 * 9 * n, "cudaMalloc(W64)")) ||
-        (rc = dalloc(&v->C64, CLOVER_REALS * n, "cudaMalloc(C64)")) ||
-        (rc = dalloc(&v->C32, CLOVER_F4 * n, "cudaMalloc(C32)")) ||
-        (rc = dalloc(&v->Cinv64, CLOVER_REALS * n, "cudaMalloc(Cinv64)")) ||
-        (rc = dalloc(&v->Cinv32, CLOVER_F4 * n, "cudaMalloc(Cinv32)")) ||
-        (rc = dalloc(&v->d_status, 64, "cudaMalloc(status)"))) {
+    const int rc = alloc_fields(v, false);
+    if (rc) {
         free_all(v);
         delete v;
         return rc;

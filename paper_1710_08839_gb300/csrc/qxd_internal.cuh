@@ -283,6 +283,10 @@ struct qxd_lattice {
     float4* Cinv32 = nullptr;  // [18][V]
     bool has_clover = false;
 
+    // the allocations that hold the gauge field and the operator's arrays
+    void* gauge_arena = nullptr;
+    void* op_arena = nullptr;
+
     // scratch
     int* d_status = nullptr;   // small device status words
     void* scratch_in = nullptr;   // native spinor FP64-sized

@@ -34,6 +34,7 @@
 #include "eo.cuh"
 #include "herm6.cuh"
 #include "rhmc.cuh"
+#include "su3.cuh"
 
 namespace qxd {
 
@@ -88,14 +89,19 @@ __device__ double ln_abs_det6(const double d[6], const C64 l[15]) {
     return acc;
 }
 
-// sum over the selected sites and both chirality blocks; fixed grid
-__global__ void __launch_bounds__(RED_THREADS) k_sw_logdet(int V, int first, int count,
+// sum over the sites [first, first + count) of the set and both chirality
+// blocks; fixed grid. With an exact mirror half the set is the physical half:
+// the mirror site's blocks are spin-flipped conjugates, with the same |det|.
+__global__ void __launch_bounds__(RED_THREADS) k_sw_logdet(GaugeSet q, int first, int count,
                                                           const double* __restrict__ C,
                                                           double* __restrict__ partials) {
+    const int V = q.g.V;
     double acc[2] = {0.0, 0.0};  // sum, number of non-finite blocks
     const size_t n = (size_t)count * 2;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int s = first + (int)(i >> 1);
+        int x[4];
+        set_coords(q, first + (int)(i >> 1), x);
+        const int s = native_of(q.g, x);
         const int blk = (int)(i & 1);
         double d[6];
         C64 l[15];
@@ -755,17 +761,18 @@ int qxd_sw_logdet(qxd_lattice* lat, int sites, double* out) {
     if (sites != QXD_SITES_EVEN && sites != QXD_SITES_ODD && sites != QXD_SITES_ALL)
         return fail(QXD_ERR_ARG, "qxd_sw_logdet: sites must be QXD_SITES_EVEN, _ODD or _ALL");
     if (!qxd::clover_ready(lat)) return fail(QXD_ERR_STATE, "qxd_sw_logdet: needs qxd_sw_build first");
-    const Geom& g = lat->g;
-    const int first = sites == QXD_SITES_ODD ? g.Vh : 0;
-    const int count = sites == QXD_SITES_ALL ? g.V : g.Vh;
+    const GaugeSet q = gauge_set(lat->g, mirror_exact(gauge_owner(lat)));
+    const int first = sites == QXD_SITES_ODD ? q.n / 2 : 0;
+    const int count = sites == QXD_SITES_ALL ? q.n : q.n / 2;
     if (!lat->mscg) lat->mscg = new MscgWork();
     int rc;
     if ((rc = lat->mscg->red.init())) return rc;
     cudaStream_t st = lat->stream;
-    k_sw_logdet<<<RED_BLOCKS, RED_THREADS, 0, st>>>(g.V, first, count, lat->C64, lat->mscg->red.partials);
+    k_sw_logdet<<<RED_BLOCKS, RED_THREADS, 0, st>>>(q, first, count, lat->C64, lat->mscg->red.partials);
     QXD_LAUNCHED("k_sw_logdet");
     if ((rc = reduce_finish(lat->mscg->red, 2, st))) return rc;
-    const double v = lat->mscg->red.h_res[0], bad = lat->mscg->red.h_res[1];
+    const double both = q.mirror ? 2.0 : 1.0;
+    const double v = both * lat->mscg->red.h_res[0], bad = both * lat->mscg->red.h_res[1];
     if (bad > 0.0 || !std::isfinite(v))
         return fail(QXD_ERR_SW_SINGULAR, "qxd_sw_logdet: " + std::to_string((long long)bad) +
                                              " singular or non-finite site blocks");
