@@ -779,7 +779,8 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     st_half(s_t, sg, t, w);
     __syncthreads();
 
-    // rho stays in shared memory between steps (fewer live registers)
+    // this thread's half of rho stays in registers (read back from shared memory
+    // for every step: 12.56 against 12.52 ms on 64x64x32x32)
     cplx<float> de[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) de[i] = mk(0.f, 0.f);
@@ -804,16 +805,15 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
             clover_half(Moi, sg, acc, w);
             st_half(s_t, sg, t, w);
         } else {
-            ld_half(s_rho, sg, t, rho);
             clover_half(Mee, sg, rho, w);
 #pragma unroll
             for (int i = 0; i < 6; ++i) w[i] = w[i] - acc[i];
             float a_re = 0.f, a_im = 0.f, b = 0.f;
 #pragma unroll
             for (int i = 0; i < 6; ++i) {
-                a_re += w[i].re * rho[i].re + w[i].im * rho[i].im;
-                a_im += w[i].re * rho[i].im - w[i].im * rho[i].re;
-                b += w[i].re * w[i].re + w[i].im * w[i].im;
+                a_re = fmaf(w[i].im, rho[i].im, fmaf(w[i].re, rho[i].re, a_re));
+                a_im = fmaf(-w[i].im, rho[i].re, fmaf(w[i].re, rho[i].im, a_im));
+                b = fmaf(w[i].im, w[i].im, fmaf(w[i].re, w[i].re, b));
             }
             float sums[3];
             // red is next written two steps later, after the barriers that end each step
