@@ -341,9 +341,8 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) k_sap_block(Geom g, SapGeom sg
 // run ahead through the next ones, and warps took them twice (28 % more
 // shared-memory loads; 14.3 -> 13.1 ms). Measured and not kept: M_oo^-1 resident
 // in shared memory (17 of 18 float4 beside the links: 16.8 ms, the loads move to
-// the shared-memory pipe and L1 shrinks), L1 hints on the clover loads (14.5 and
-// 15.0), L2 prefetch of the own or the next block's data (14.5, 14.7), clover
-// loads before the hops (12.9, within the spread elsewhere).
+// the shared-memory pipe), L2 prefetch of the next block's data (14.7 where 14.3
+// without). Tensor memory has neither drawback: see below.
 // ---------------------------------------------------------------------------
 constexpr int SPLIT_THREADS = 256;
 constexpr unsigned FULL_MASK = 0xffffffffu;
@@ -550,18 +549,77 @@ __device__ __forceinline__ void split_hops(const SplitLinks& bl, const float2* s
     }
 }
 
-// Own rows (3 sg + a, a = 0..2) of both packed Hermitian 6x6 blocks of a site
-// times v; v and y are own halves, the partner's half is shuffled in. C: the
-// site's first float4 of its block's SAP_HALF-strided matrices.
-// In block order the rows of thread sg see a Hermitian 3x3 diagonal block
-// (entries d[3 sg + a] and L(3 sg + a, 3 sg + b)) and the off-diagonal
-// 3x3 block B[a][b] = L(3 + a, b) for sg = 1, B^+ for sg = 0. Every thread
-// of the warp must call it.
-__device__ __forceinline__ void clover_half(const float4* __restrict__ C, int sg, const cplx<float> v[6],
-                                            cplx<float> y[6]) {
-    cplx<float> p[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) p[k] = mk(__shfl_xor_sync(FULL_MASK, v[k].re, 1), __shfl_xor_sync(FULL_MASK, v[k].im, 1));
+// Tensor memory of the split kernel. The rows of M_oo^-1 and M_ee that a thread
+// applies, 27 floats for each of the two 6x6 blocks of a matrix, are its own and
+// are used in every MR step: they are put into tensor memory, whose lanes belong
+// to the threads of a warp, once per launch. A warp reaches the 32 lanes from
+// 32 (warp % 4) on, so warps w and w + 4 take different columns: 2 x 4 x 32
+// columns for a thread block, and with two of them all 512 of an SM.
+// Loaded again for every step, 73 KB per block outgrew L1 and, with 304 blocks
+// in flight, L2: DRAM bytes of a launch on 48x48x24x24 sites 929 -> 606 MB, waits
+// for global memory per instruction 2.0 -> 0.8, and with rows chosen and
+// conjugated once 9 % fewer instructions; one application on 64x64x32x32 sites
+// 12.52 -> 11.16 ms, six right-hand sides on 32x32x16x16 4.73 -> 4.29 ms.
+// Measured and not kept: r_o in the spare columns too (11.29), the rows loaded
+// after the residual is formed (11.28), the loads of tm_load28 issued before the
+// shuffles (11.16), the two blocks' rows interleaved and multiplied by packed
+// FP32 pairs (11.60).
+constexpr int TM_BLOCK = 32;             // columns of one 6x6 block's rows (28 used)
+constexpr int TM_COLS = 2 * 4 * TM_BLOCK;
+
+// the whole of warp 0; the address arrives in shared memory
+__device__ __forceinline__ void tm_alloc(uint32_t* s_addr) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(s_addr)),
+                 "n"(TM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+}
+__device__ __forceinline__ void tm_free(uint32_t addr) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "n"(TM_COLS));
+}
+__device__ __forceinline__ void tm_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tm_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tm_store_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// 28 columns of this thread's lane; every thread of the warp takes part
+__device__ __forceinline__ void tm_store28(uint32_t a, const float r[28]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15, %16};" ::"r"(a),
+        "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]), "f"(r[8]), "f"(r[9]),
+        "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15])
+        : "memory");
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(a + 16),
+                 "f"(r[16]), "f"(r[17]), "f"(r[18]), "f"(r[19]), "f"(r[20]), "f"(r[21]), "f"(r[22]), "f"(r[23])
+                 : "memory");
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a + 24), "f"(r[24]),
+                 "f"(r[25]), "f"(r[26]), "f"(r[27])
+                 : "memory");
+}
+__device__ __forceinline__ void tm_load28(uint32_t a, float r[28]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%28];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16, %17, %18, %19, %20, %21, %22, %23}, [%29];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%24, %25, %26, %27}, [%30];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]), "=f"(r[8]),
+          "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]), "=f"(r[16]),
+          "=f"(r[17]), "=f"(r[18]), "=f"(r[19]), "=f"(r[20]), "=f"(r[21]), "=f"(r[22]), "=f"(r[23]), "=f"(r[24]),
+          "=f"(r[25]), "=f"(r[26]), "=f"(r[27])
+        : "r"(a), "r"(a + 16), "r"(a + 24)
+        : "memory");
+}
+
+// This thread's rows (3 sg + a, a = 0..2) of both packed Hermitian 6x6 blocks
+// of a site, to tensor memory at a: per block E[a][b] (18 floats), L(3 sg + 1,
+// 3 sg), L(3 sg + 2, 3 sg), L(3 sg + 2, 3 sg + 1) (6) and the diagonal (3). In
+// block order the rows of thread sg see a Hermitian 3x3 diagonal block (entries
+// d[3 sg + a] and L(3 sg + a, 3 sg + b)) and the off-diagonal 3x3 block E =
+// B[a][b] = L(3 + a, b) for sg = 1, B^+ for sg = 0. C: the site's first float4
+// of its block's SAP_HALF-strided matrices.
+__device__ __forceinline__ void clover_rows(const float4* __restrict__ C, int sg, uint32_t a) {
 #pragma unroll
     for (int blk = 0; blk < 2; ++blk) {
         const float4* Cb = C + 9 * blk * SAP_HALF;
@@ -569,16 +627,39 @@ __device__ __forceinline__ void clover_half(const float4* __restrict__ C, int sg
         const float4 q5 = Cb[5 * SAP_HALF], q6 = Cb[6 * SAP_HALF], q7 = Cb[7 * SAP_HALF];
         const float4 X = Cb[(sg ? 8 : 2) * SAP_HALF];
         // packed floats: d_i at i, L_k at (6 + 2k, 7 + 2k); float4 n holds 4n..4n+3
-        const float d0 = sg ? q0.w : q0.x, d1 = sg ? q1.x : q0.y, d2 = sg ? q1.y : q0.z;
-        const cplx<float> l10 = sg ? mk(q6.x, q6.y) : mk(q1.z, q1.w);  // L(4,3) : L(1,0)
-        const cplx<float> l20 = mk(X.x, X.y);                          // L(5,3) : L(2,0)
-        const cplx<float> l21 = mk(X.z, X.w);                          // L(5,4) : L(2,1)
         const cplx<float> B[3][3] = {{mk(q3.x, q3.y), mk(q3.z, q3.w), mk(q4.x, q4.y)},
                                      {mk(q4.z, q4.w), mk(q5.x, q5.y), mk(q5.z, q5.w)},
                                      {mk(q6.z, q6.w), mk(q7.x, q7.y), mk(q7.z, q7.w)}};
+        float r[28];
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+#pragma unroll
+            for (int y = 0; y < 3; ++y) {
+                r[6 * x + 2 * y] = sg ? B[x][y].re : B[y][x].re;
+                r[6 * x + 2 * y + 1] = sg ? B[x][y].im : -B[y][x].im;
+            }
+        r[18] = sg ? q6.x : q1.z, r[19] = sg ? q6.y : q1.w;  // L(4,3) : L(1,0)
+        r[20] = X.x, r[21] = X.y;                            // L(5,3) : L(2,0)
+        r[22] = X.z, r[23] = X.w;                            // L(5,4) : L(2,1)
+        r[24] = sg ? q0.w : q0.x, r[25] = sg ? q1.x : q0.y, r[26] = sg ? q1.y : q0.z;
+        r[27] = 0.f;
+        tm_store28(a + blk * TM_BLOCK, r);
+    }
+}
+
+// Own rows of the matrix at a times v; v and y are own halves, the partner's
+// half is shuffled in. Every thread of the warp must call it.
+__device__ __forceinline__ void clover_half(uint32_t tm, const cplx<float> v[6], cplx<float> y[6]) {
+#pragma unroll
+    for (int blk = 0; blk < 2; ++blk) {
         const cplx<float>* w = v + 3 * blk;
-        const cplx<float>* pp = p + 3 * blk;
-        cplx<float> z[3];
+        cplx<float> pp[3], z[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            pp[k] = mk(__shfl_xor_sync(FULL_MASK, w[k].re, 1), __shfl_xor_sync(FULL_MASK, w[k].im, 1));
+        float r[28];
+        tm_load28(tm + blk * TM_BLOCK, r);
+        const cplx<float> l10 = mk(r[18], r[19]), l20 = mk(r[20], r[21]), l21 = mk(r[22], r[23]);
         // the diagonal, the largest term, comes last
         z[0] = cmad(l20, w[2], cmul(l10, w[1]));
         z[1] = cmad(l21, w[2], l10 * w[0]);
@@ -586,14 +667,9 @@ __device__ __forceinline__ void clover_half(const float4* __restrict__ C, int sg
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                // E[a][b] = sg ? B[a][b] : conj(B[b][a])
-                const cplx<float> e = mk(sg ? B[a][b].re : B[b][a].re, sg ? B[a][b].im : -B[b][a].im);
-                z[a] = mad(e, pp[b], z[a]);
-            }
-        y[3 * blk] = rmad(d0, w[0], z[0]);
-        y[3 * blk + 1] = rmad(d1, w[1], z[1]);
-        y[3 * blk + 2] = rmad(d2, w[2], z[2]);
+            for (int b = 0; b < 3; ++b) z[a] = mad(mk(r[6 * a + 2 * b], r[6 * a + 2 * b + 1]), pp[b], z[a]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) y[3 * blk + a] = rmad(r[24 + a], w[a], z[a]);
     }
 }
 
@@ -730,7 +806,9 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     float2* s_rho = sm;                 // r on the even sites, the MR residual, delta_o at the end
     float2* s_t = sm + FIELD_F2;        // r on the odd sites, the odd temporary, delta_e at the end
     float* red = reinterpret_cast<float*>(sm + 2 * FIELD_F2);  // 3 * warps reduction slots
+    uint32_t* s_tm = reinterpret_cast<uint32_t*>(red + 3 * (SPLIT_THREADS / 32));
 
+    if (threadIdx.x < 32) tm_alloc(s_tm);
     int org[4];
     const int blk = block_origin(sgm, bidx, colour, org);
     const int t = threadIdx.x >> 1;
@@ -746,8 +824,19 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
         const float4* src = plan.links + (size_t)blk * PLAN_LINK_F4;
         for (int k = threadIdx.x; k < PLAN_LINK_F4; k += SPLIT_THREADS) copy_async16(sW4 + k, src + k);
     }
-    const float4* Moi = plan.clover + (size_t)blk * PLAN_CLOVER_F4 + t;  // M_oo^-1, M_ee of this pair
-    const float4* Mee = Moi + CLOVER_F4 * SAP_HALF;
+    tm_fence_before();
+    __syncthreads();
+    tm_fence_after();
+    const uint32_t tm = *s_tm;
+    // M_oo^-1 and M_ee of this pair, this thread's rows
+    const uint32_t Moi = tm + ((threadIdx.x & 96u) << 16) + (threadIdx.x >> 7) * (TM_COLS / 2);
+    const uint32_t Mee = Moi + 2 * TM_BLOCK;
+    {
+        const float4* src = plan.clover + (size_t)blk * PLAN_CLOVER_F4 + t;
+        clover_rows(src, sg, Moi);
+        clover_rows(src + CLOVER_F4 * SAP_HALF, sg, Mee);
+        tm_store_wait();
+    }
 
     {
         cplx<float> r[12];
@@ -775,7 +864,7 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     // pair overwrites its own halves of s_t with t_o = M_oo^-1 r_o
     cplx<float> ro[6], v[6], w[6], acc[6], rho[6];
     ld_half(s_t, sg, t, ro);
-    clover_half(Moi, sg, ro, w);
+    clover_half(Moi, ro, w);
     st_half(s_t, sg, t, w);
     __syncthreads();
 
@@ -799,13 +888,13 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
         } else if (last) {
 #pragma unroll
             for (int i = 0; i < 6; ++i) v[i] = ro[i] - acc[i];
-            clover_half(Moi, sg, v, w);  // delta_o (s_rho is no longer read)
+            clover_half(Moi, v, w);  // delta_o (s_rho is no longer read)
             st_half(s_rho, sg, t, w);
         } else if (odd) {
-            clover_half(Moi, sg, acc, w);
+            clover_half(Moi, acc, w);
             st_half(s_t, sg, t, w);
         } else {
-            clover_half(Mee, sg, rho, w);
+            clover_half(Mee, rho, w);
 #pragma unroll
             for (int i = 0; i < 6; ++i) w[i] = w[i] - acc[i];
             float a_re = 0.f, a_im = 0.f, b = 0.f;
@@ -843,8 +932,11 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
                 st_half(s_rho, sg, t, rho);
             }
         }
+        tm_fence_before();
         __syncthreads();
     }
+    tm_fence_after();
+    if (threadIdx.x < 32) tm_free(tm);
     // psi_B += delta on this thread's site: delta_e in s_t, delta_o in s_rho
     cplx<float> d[12];
     ld_full(sg ? s_rho : s_t, t, d);
@@ -936,13 +1028,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 2) k_sap_block_batch(const SapJ
 template <typename R>
 size_t sap_smem_bytes() {
     if (sizeof(R) == 4)  // split kernel: interior compound links, two block fields, reduction slots of 8 warps
-        return split_link_bytes() + 2 * FIELD_F2 * sizeof(float2) + 3 * (SPLIT_THREADS / 32) * sizeof(float);
+        return split_link_bytes() + 2 * FIELD_F2 * sizeof(float2) + 3 * (SPLIT_THREADS / 32) * sizeof(float) +
+               sizeof(uint32_t);
     return (72 * SAP_HALF + 3 * (SAP_THREADS / 32)) * sizeof(R);
 }
 
 // Dynamic shared memory of the split kernel, and an L1/shared carveout just
-// large enough for two blocks per SM: the rest of the SM's L1 caches the
-// clover blocks that every MR step re-reads.
+// large enough for two blocks per SM.
 template <typename K>
 int split_attrs(K kernel, size_t smem) {
     int dev = 0, per_sm = 0;
