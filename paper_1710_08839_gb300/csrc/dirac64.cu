@@ -11,8 +11,8 @@
 // is left over, up to 4864 sites, is split further, over 6 threads (spin and
 // colour, 232 instructions; 8 lanes with two idle). Measured: 262144 sites 515
 // us (0.90 of the FP64 issue rate; one thread per site 800 before the compound
-// links and multiply-add chains), 41472 sites of D_hat's first half 98 us (5
-// rounds of 552 where 4.26 would do; one thread per site 120 us), D on 1024
+// links and multiply-add chains), 41472 sites of D_hat's first half 91 us (four
+// rounds of 552 and two of 232; one thread per site 120 us), D on 1024
 // lexicographic sites 12.3 us for the call (one thread per site, with the two
 // layout conversions, 55 us). 128 registers (4 blocks of 128 threads): 96 with
 // spills took 3-5 % longer on 41472 sites.
