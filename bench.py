@@ -770,14 +770,14 @@ def rational_benchmark(qxd, torch):
 
 
 # Wilson flow of the solver workload's gauge field: FP64 work per RK3 stage
-# and integrated link: the staple sum (12 complex 3x3 products of 198 flops),
-# W = U S and exp(X) U (2 more), the exponential by Cayley-Hamilton (X^2: one
-# product; det X ~ 60; 24 terms of the scalar recurrence ~ 26 each; the
-# combination A + B X + C X^2 ~ 144), plus the U(1) angle update (~ 60); the
-# links integrated are the physical ones (half the simulated lattice with C*
-# boundaries)
+# and integrated link: 1.5 plaquettes, each 3 complex 3x3 products (198 flops)
+# and the anti-Hermitian parts of 3 more (171); the sum of six leaves (~ 108) and
+# the accumulator (~ 27); the exponential by Cayley-Hamilton (H^2 and det H ~ 80,
+# 15 terms of the real recurrence ~ 8 each, the combination ~ 90) and its product
+# with the link; the links integrated are the physical ones (half the simulated
+# lattice with C* boundaries)
 FLOW_WORKLOAD = dict(eps=0.02, steps=(5, 5, 10), q_el=1.0 / 6.0)
-FLOW_FLOPS_PER_LINK_STAGE = 15 * 198 + 60 + 24 * 26 + 144 + 60
+FLOW_FLOPS_PER_LINK_STAGE = 1.5 * (3 * 198 + 3 * 171) + 108 + 27 + 80 + 15 * 8 + 90 + 198
 
 
 def flow_benchmark(qxd, torch):
@@ -970,7 +970,7 @@ def sap_benchmark(qxd, torch, steps, w):
     return {"sap_ms": single, "sites": V, "ncy": 5, "nmr": 5,
             "lattice": f"{w['T']}x{2 * w['L1']}x{w['L2']}x{w['L3']}",
             "multi_rhs": {"rhs": R, "ms_per_rhs": multi, "speedup_vs_single": single / multi,
-                          "note": "qxd_sap_multi: links staged once per block for all right-hand sides"}}
+                          "note": "qxd_sap_multi: the right-hand sides of a block side by side in one launch"}}
 
 
 # --- the oracle on all host cores ------------------------------------------
