@@ -559,7 +559,7 @@ __device__ __forceinline__ void split_hops(const SplitLinks& bl, const float2* s
 // in flight, L2: DRAM bytes of a launch on 48x48x24x24 sites 929 -> 606 MB, waits
 // for global memory per instruction 2.0 -> 0.8, and with rows chosen and
 // conjugated once 9 % fewer instructions; one application on 64x64x32x32 sites
-// 12.52 -> 11.16 ms, six right-hand sides on 32x32x16x16 4.73 -> 4.29 ms.
+// 12.52 -> 11.08 ms, six right-hand sides on 32x32x16x16 4.73 -> 4.24 ms.
 // Measured and not kept: r_o in the spare columns too (11.29), the rows loaded
 // after the residual is formed (11.28), the loads of tm_load28 issued before the
 // shuffles (11.16), the two blocks' rows interleaved and multiplied by packed
@@ -588,14 +588,11 @@ __device__ __forceinline__ void tm_store28(uint32_t a, const float r[28]) {
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
         "%15, %16};" ::"r"(a),
         "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]), "f"(r[8]), "f"(r[9]),
-        "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15])
-        : "memory");
+        "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15]));
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(a + 16),
-                 "f"(r[16]), "f"(r[17]), "f"(r[18]), "f"(r[19]), "f"(r[20]), "f"(r[21]), "f"(r[22]), "f"(r[23])
-                 : "memory");
+                 "f"(r[16]), "f"(r[17]), "f"(r[18]), "f"(r[19]), "f"(r[20]), "f"(r[21]), "f"(r[22]), "f"(r[23]));
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a + 24), "f"(r[24]),
-                 "f"(r[25]), "f"(r[26]), "f"(r[27])
-                 : "memory");
+                 "f"(r[25]), "f"(r[26]), "f"(r[27]));
 }
 __device__ __forceinline__ void tm_load28(uint32_t a, float r[28]) {
     asm volatile(
@@ -608,24 +605,36 @@ __device__ __forceinline__ void tm_load28(uint32_t a, float r[28]) {
           "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15]), "=f"(r[16]),
           "=f"(r[17]), "=f"(r[18]), "=f"(r[19]), "=f"(r[20]), "=f"(r[21]), "=f"(r[22]), "=f"(r[23]), "=f"(r[24]),
           "=f"(r[25]), "=f"(r[26]), "=f"(r[27])
-        : "r"(a), "r"(a + 16), "r"(a + 24)
-        : "memory");
+        : "r"(a), "r"(a + 16), "r"(a + 24));
 }
 
-// This thread's rows (3 sg + a, a = 0..2) of both packed Hermitian 6x6 blocks
-// of a site, to tensor memory at a: per block E[a][b] (18 floats), L(3 sg + 1,
-// 3 sg), L(3 sg + 2, 3 sg), L(3 sg + 2, 3 sg + 1) (6) and the diagonal (3). In
-// block order the rows of thread sg see a Hermitian 3x3 diagonal block (entries
-// d[3 sg + a] and L(3 sg + a, 3 sg + b)) and the off-diagonal 3x3 block E =
-// B[a][b] = L(3 + a, b) for sg = 1, B^+ for sg = 0. C: the site's first float4
-// of its block's SAP_HALF-strided matrices.
-__device__ __forceinline__ void clover_rows(const float4* __restrict__ C, int sg, uint32_t a) {
+// What the rows of thread sg of both packed Hermitian 6x6 blocks of a site need,
+// eight of the nine float4 of each; C: the site's first float4 of its block's
+// SAP_HALF-strided matrices. All loads of a matrix are under way before the first
+// is used (block by block, with the stores between: 11.16 against 11.08 ms on
+// 64x64x32x32 sites, 8.28 against 7.91 with 2 MR steps).
+__device__ __forceinline__ void clover_load(const float4* __restrict__ C, int sg, float4 q[16]) {
 #pragma unroll
     for (int blk = 0; blk < 2; ++blk) {
         const float4* Cb = C + 9 * blk * SAP_HALF;
-        const float4 q0 = Cb[0], q1 = Cb[SAP_HALF], q3 = Cb[3 * SAP_HALF], q4 = Cb[4 * SAP_HALF];
-        const float4 q5 = Cb[5 * SAP_HALF], q6 = Cb[6 * SAP_HALF], q7 = Cb[7 * SAP_HALF];
-        const float4 X = Cb[(sg ? 8 : 2) * SAP_HALF];
+        q[8 * blk] = Cb[0], q[8 * blk + 1] = Cb[SAP_HALF];
+        q[8 * blk + 2] = Cb[(sg ? 8 : 2) * SAP_HALF];
+#pragma unroll
+        for (int n = 3; n < 8; ++n) q[8 * blk + n] = Cb[n * SAP_HALF];
+    }
+}
+
+// This thread's rows (3 sg + a, a = 0..2), from clover_load, to tensor memory at
+// a: per block E[a][b] (18 floats), L(3 sg + 1, 3 sg), L(3 sg + 2, 3 sg), L(3 sg +
+// 2, 3 sg + 1) (6) and the diagonal (3). In block order the rows of thread sg see
+// a Hermitian 3x3 diagonal block (entries d[3 sg + a] and L(3 sg + a, 3 sg + b))
+// and the off-diagonal 3x3 block E = B[a][b] = L(3 + a, b) for sg = 1, B^+ for
+// sg = 0.
+__device__ __forceinline__ void clover_rows(const float4 q[16], int sg, uint32_t a) {
+#pragma unroll
+    for (int blk = 0; blk < 2; ++blk) {
+        const float4 q0 = q[8 * blk], q1 = q[8 * blk + 1], X = q[8 * blk + 2], q3 = q[8 * blk + 3];
+        const float4 q4 = q[8 * blk + 4], q5 = q[8 * blk + 5], q6 = q[8 * blk + 6], q7 = q[8 * blk + 7];
         // packed floats: d_i at i, L_k at (6 + 2k, 7 + 2k); float4 n holds 4n..4n+3
         const cplx<float> B[3][3] = {{mk(q3.x, q3.y), mk(q3.z, q3.w), mk(q4.x, q4.y)},
                                      {mk(q4.z, q4.w), mk(q5.x, q5.y), mk(q5.z, q5.w)},
@@ -833,8 +842,11 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     const uint32_t Mee = Moi + 2 * TM_BLOCK;
     {
         const float4* src = plan.clover + (size_t)blk * PLAN_CLOVER_F4 + t;
-        clover_rows(src, sg, Moi);
-        clover_rows(src + CLOVER_F4 * SAP_HALF, sg, Mee);
+        float4 q[16];
+        clover_load(src, sg, q);
+        clover_rows(q, sg, Moi);
+        clover_load(src + CLOVER_F4 * SAP_HALF, sg, q);
+        clover_rows(q, sg, Mee);
         tm_store_wait();
     }
 
