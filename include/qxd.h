@@ -121,6 +121,9 @@ int qxd_lattice_dims(const qxd_lattice* lat, int* N4, long long* volume);
  * the third): otherwise QXD_ERR_ARG. CHECKED rejects fields that violate
  * Eq. (4a) beyond 1e-12 with QXD_ERR_NOT_ADMISSIBLE. The field tensors of
  * the clover term are computed here (FP64). Invalidates the clover term.
+ * Links that are refused have overwritten the old field all the same: the
+ * lattice then has none (QXD_ERR_STATE until a field is accepted), and its
+ * clover term and those of its views are stale.
  * Synchronises the lattice stream.
  */
 int qxd_set_gauge(qxd_lattice* lat, const double* su3, const double* u1_angle, int flags);

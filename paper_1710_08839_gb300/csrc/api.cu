@@ -242,6 +242,9 @@ int qxd_set_gauge(qxd_lattice* lat, const double* su3, const double* u1_angle, i
         d_su3 = tmp;
         d_ang = tmp + nsites * 4 * 18;
     }
+    // the field is written from here on: the clover terms of this lattice and its
+    // views are stale even if the new links are refused
+    ++lat->gauge_version;
     int rc = launch_gauge_ingest(lat, d_su3, d_ang, kind, lat->d_status);
     if (rc == QXD_OK) rc = launch_field_tensor(lat);
     int st[4] = {0, 0, 0, 0};
@@ -257,7 +260,6 @@ int qxd_set_gauge(qxd_lattice* lat, const double* su3, const double* u1_angle, i
     if (st[1]) return fail(QXD_ERR_NOT_ADMISSIBLE, "qxd_set_gauge: " + std::to_string(st[1]) +
                                                        " mirror links violate the orbifold constraint");
     lat->has_gauge = true;
-    ++lat->gauge_version;
     return QXD_OK;
 }
 

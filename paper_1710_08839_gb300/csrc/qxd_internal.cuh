@@ -308,7 +308,8 @@ struct qxd_lattice {
     // parameters, clover term, scratch and solver work
     qxd_lattice* parent = nullptr;
     int nviews = 0;                    // live views of this lattice
-    unsigned gauge_version = 0;        // bumped by every successful set_gauge
+    unsigned gauge_version = 0;        // bumped whenever the field is written: set_gauge (also when it refuses
+                                       // the links it has read) and the flow
     unsigned built_gauge_version = 0;  // gauge version the clover was built from
 };
 
