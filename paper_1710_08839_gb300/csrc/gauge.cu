@@ -30,20 +30,21 @@ __global__ void __launch_bounds__(256) k_gauge_ingest(GaugeSet q, const double* 
 #pragma unroll
         for (int j = 0; j < 3; ++j) u[i][j] = mk(p[(i * 3 + j) * 2], p[(i * 3 + j) * 2 + 1]);
     const double a = ang[src * 4 + mu];
-    // SU(3) check: |U U^+ - 1| (Hermitian: the entries on and above the diagonal) and |det U - 1|
-    double dev = 0.0;
+    // SU(3) check: |U U^+ - 1| (Hermitian: the entries on and above the diagonal) and |det U - 1|, each entry compared
+    // by itself (a maximum of them would drop a NaN)
+    bool ok = isfinite(a);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = i; j < 3; ++j) {
             const C64 s2 = cmad(u[j][2], u[i][2], cmad(u[j][1], u[i][1], mulc(u[i][0], u[j][0])));
-            dev = fmax(dev, fmax(fabs(s2.re - (i == j ? 1.0 : 0.0)), fabs(s2.im)));
+            ok = ok && fabs(s2.re - (i == j ? 1.0 : 0.0)) <= 1e-10 && fabs(s2.im) <= 1e-10;
         }
     const C64 m0 = u[1][1] * u[2][2] - u[1][2] * u[2][1], m1 = u[1][2] * u[2][0] - u[1][0] * u[2][2],
               m2 = u[1][0] * u[2][1] - u[1][1] * u[2][0];
     const C64 det = mad(u[0][2], m2, mad(u[0][1], m1, u[0][0] * m0));
-    dev = fmax(dev, fmax(fabs(det.re - 1.0), fabs(det.im)));
-    if (!(dev <= 1e-10) || !isfinite(a)) atomicAdd(&bad[0], q.mirror ? 2 : 1);
+    ok = ok && fabs(det.re - 1.0) <= 1e-10 && fabs(det.im) <= 1e-10;
+    if (!ok) atomicAdd(&bad[0], q.mirror ? 2 : 1);
     double sa, ca;
     sincos(a, &sa, &ca);
     for (int m = 0; m <= q.mirror; ++m) {
@@ -77,18 +78,18 @@ __global__ void k_check_admissible(Geom g, const double* __restrict__ su3, const
     size_t m = (size_t)i, p = (size_t)lex_index(g, x0, x1 - g.L1, x2, x3);
     int nbad = 0;
     for (int mu = 0; mu < 4; ++mu) {
-        double dev = 0.0;
+        bool ok = true;
         for (int e = 0; e < 9; ++e) {
             double mre = su3[(m * 4 + mu) * 18 + 2 * e], mim = su3[(m * 4 + mu) * 18 + 2 * e + 1];
             double pre = su3[(p * 4 + mu) * 18 + 2 * e], pim = su3[(p * 4 + mu) * 18 + 2 * e + 1];
-            dev = fmax(dev, fmax(fabs(mre - pre), fabs(mim + pim)));
+            ok = ok && fabs(mre - pre) <= 1e-12 && fabs(mim + pim) <= 1e-12;
         }
         double am = ang[m * 4 + mu], ap = ang[p * 4 + mu];
         double sm, cm, sp, cp;
         sincos(am, &sm, &cm);
         sincos(ap, &sp, &cp);
-        dev = fmax(dev, fmax(fabs(cm - cp), fabs(sm + sp)));
-        if (!(dev <= 1e-12)) ++nbad;
+        ok = ok && fabs(cm - cp) <= 1e-12 && fabs(sm + sp) <= 1e-12;
+        if (!ok) ++nbad;
     }
     if (nbad) atomicAdd(&bad[1], nbad);
 }
