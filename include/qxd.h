@@ -145,11 +145,16 @@ int qxd_set_params(qxd_lattice* lat, double m0, double csw, double cswqed, int q
  * singular to working precision or non-finite (inverse pivots below
  * 1e-12 of the block norm). On lattices that admit the Schwarz blocks of
  * qxd_sap it also lays the FP32 operator out block by block for it (504 bytes
- * per site, allocated by the first build and kept with the lattice; if there
- * is no memory for it, the first FP32 Schwarz application tries again).
- * Synchronises the lattice stream.
+ * per site, allocated by the first build and kept with the lattice; without
+ * memory for it the FP32 Schwarz method reads the lattice's other fields, with
+ * the same results, slower). Synchronises the lattice stream.
  */
 int qxd_sw_build(qxd_lattice* lat);
+
+/* enable = 0: qxd_sw_build does not make that copy (a program that has better
+ * use for the memory); 1 (the default): it does. QXD_ERR_STATE once the
+ * lattice has one. Views have their own. */
+int qxd_set_sap_copy(qxd_lattice* lat, int enable);
 
 /*
  * out = D in (Sec. 2.3): (D psi)(x) = M(x) psi(x)

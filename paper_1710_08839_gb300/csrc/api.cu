@@ -283,12 +283,7 @@ int qxd_sw_build(qxd_lattice* lat) {
     lat->has_clover = false;
     int rc = launch_clover_build(lat, lat->d_status);
     if (rc) return rc;
-    bool plan = sap_admissible(lat);
-    if (plan && (rc = launch_sap_plan(lat, lat->stream))) {
-        if (rc != QXD_ERR_OOM) return rc;
-        cudaGetLastError();  // the first SAP application tries again
-        plan = false;
-    }
+    if (sap_admissible(lat) && (rc = launch_sap_plan(lat, lat->stream))) return rc;
     int st[4];
     cudaError_t e = cudaMemcpyAsync(st, lat->d_status, sizeof(st), cudaMemcpyDeviceToHost, lat->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(lat->stream);
@@ -298,7 +293,6 @@ int qxd_sw_build(qxd_lattice* lat) {
     lat->has_clover = true;
     lat->built_gauge_version = gauge_owner(lat)->gauge_version;
     ++lat->op_version;
-    if (plan) lat->sap_plan_version = lat->op_version;
     return QXD_OK;
 }
 

@@ -187,8 +187,6 @@ struct Engine {
         if (j->P.precond == QXD_PRECOND_SAP) {
             j->sapw_bytes = sap_work_bytes(j->op);
             if ((rc = pool.alloc(j->sapw_bytes, &j->sapw))) return rc;
-            SapPlan plan;  // built with the operator, or now if there was no memory for it then
-            if ((rc = sap_plan(j->op, st, &plan))) return rc;
         }
         // Krylov vectors are allocated when first used (SAP-preconditioned
         // GCR rarely needs all nkv of them)
@@ -337,7 +335,7 @@ struct Engine {
                 J.g = j->op->g;
                 J.sg = sap_geom(j->op->g);
                 J.f = Fields<float>{(const float4*)j->phi[j->k], nullptr, j->op->U32, j->op->A32, j->op->C32};
-                if ((rc = sap_plan(j->op, st, &J.plan))) return rc;
+                J.plan = sap_plan(j->op);
                 J.eta = (const float4*)j->rin;
                 J.delta = (float4*)j->sapw;
                 J.rho = J.delta + (size_t)SPINOR_F4 * j->op->g.V;

@@ -293,8 +293,9 @@ struct qxd_lattice {
     void* scratch_out = nullptr;  // native spinor FP64-sized
     void* scratch_lex = nullptr;  // lexicographic FP64 spinor
     float4* sap_r = nullptr;      // FP32 work fields of the Schwarz method (delta, rho; first FP32 SAP application)
-    float4* sap_plan = nullptr;   // the operator block by block for the Schwarz method (lattices that admit it)
-    unsigned sap_plan_version = 0;  // op_version it was built for
+    float4* sap_plan = nullptr;   // the operator block by block for the Schwarz method: of lattices that admit it,
+                                  // made with the operator by sw_build (null: no memory for it, or not wanted)
+    bool sap_copy_wanted = true;
     float4* sap_multi = nullptr;  // work fields of qxd_sap_multi, sap_multi_n right-hand sides
     int sap_multi_n = 0;
     qxd::HostPipe* hostpipe = nullptr;  // streams and events of the pipelined host-buffer D
@@ -320,7 +321,7 @@ int launch_gauge_ingest(qxd_lattice* lat, const double* su3, const double* ang, 
 int launch_field_tensor(qxd_lattice* lat);
 int launch_clover_build(qxd_lattice* lat, int* d_bad);
 // the operator block by block for the Schwarz method, from the FP32 fields;
-// allocates it on first use (504 bytes per site)
+// allocates it on first use (504 bytes per site), does without if it cannot
 bool sap_admissible(const qxd_lattice* lat);
 int launch_sap_plan(qxd_lattice* lat, cudaStream_t st);
 int launch_dirac(qxd_lattice* lat, void* out, const void* in, int prec, cudaStream_t st);

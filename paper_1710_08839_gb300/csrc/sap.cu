@@ -460,6 +460,34 @@ struct SplitPair {
     }
 };
 
+// The compound links of site me (parity sg) that stay inside its block, to
+// their entries of the block's links at W4, W2 (SplitLinks)
+template <bool QNZ>
+__device__ __forceinline__ void block_links(const Geom& g, const Fields<float>& f, const Site& me, int sg, float q,
+                                            float4* __restrict__ W4, float2* __restrict__ W2) {
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        if (me.l[mu] == SAP_BS - 1) continue;
+        const int e = mu == 0   ? link_entry<0>(sg, me.lidx)
+                      : mu == 1 ? link_entry<1>(sg, me.lidx)
+                      : mu == 2 ? link_entry<2>(sg, me.lidx)
+                                : link_entry<3>(sg, me.lidx);
+        cplx<float> u[3][3];
+        load_link(f.U, g.V, mu, me.s, u);
+        cplx<float> z = QNZ ? link_phase(f.A, g.V, mu, me.s, q) : mk(1.f, 0.f);
+        z = -0.5f * z;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) u[a][b] = z * u[a][b];
+        W4[(mu * 4 + 0) * SPLIT_LINKS + e] = make_float4(u[0][0].re, u[0][0].im, u[0][1].re, u[0][1].im);
+        W4[(mu * 4 + 1) * SPLIT_LINKS + e] = make_float4(u[0][2].re, u[0][2].im, u[1][0].re, u[1][0].im);
+        W4[(mu * 4 + 2) * SPLIT_LINKS + e] = make_float4(u[1][1].re, u[1][1].im, u[1][2].re, u[1][2].im);
+        W4[(mu * 4 + 3) * SPLIT_LINKS + e] = make_float4(u[2][0].re, u[2][0].im, u[2][1].re, u[2][1].im);
+        W2[mu * SPLIT_LINKS + e] = make_float2(u[2][2].re, u[2][2].im);
+    }
+}
+
 constexpr int PLAN_LINK_F4 = 16 * SPLIT_LINKS + 2 * SPLIT_LINKS;  // float4 of one block's links
 constexpr int PLAN_CLOVER_F4 = 2 * CLOVER_F4 * SAP_HALF;          // of its clover blocks
 constexpr size_t split_link_bytes() { return 16 * SPLIT_LINKS * sizeof(float4) + 4 * SPLIT_LINKS * sizeof(float2); }
@@ -609,18 +637,18 @@ __device__ __forceinline__ void tm_load28(uint32_t a, float r[28]) {
 }
 
 // What the rows of thread sg of both packed Hermitian 6x6 blocks of a site need,
-// eight of the nine float4 of each; C: the site's first float4 of its block's
-// SAP_HALF-strided matrices. All loads of a matrix are under way before the first
+// eight of the nine float4 of each; C: the site's first float4, the others
+// `stride` apart. All loads of a matrix are under way before the first
 // is used (block by block, with the stores between: 11.16 against 11.08 ms on
 // 64x64x32x32 sites, 8.28 against 7.91 with 2 MR steps).
-__device__ __forceinline__ void clover_load(const float4* __restrict__ C, int sg, float4 q[16]) {
+__device__ __forceinline__ void clover_load(const float4* __restrict__ C, size_t stride, int sg, float4 q[16]) {
 #pragma unroll
     for (int blk = 0; blk < 2; ++blk) {
-        const float4* Cb = C + 9 * blk * SAP_HALF;
-        q[8 * blk] = Cb[0], q[8 * blk + 1] = Cb[SAP_HALF];
-        q[8 * blk + 2] = Cb[(sg ? 8 : 2) * SAP_HALF];
+        const float4* Cb = C + 9 * blk * stride;
+        q[8 * blk] = Cb[0], q[8 * blk + 1] = Cb[stride];
+        q[8 * blk + 2] = Cb[(sg ? 8 : 2) * stride];
 #pragma unroll
-        for (int n = 3; n < 8; ++n) q[8 * blk + n] = Cb[n * SAP_HALF];
+        for (int n = 3; n < 8; ++n) q[8 * blk + n] = Cb[n * stride];
     }
 }
 
@@ -803,7 +831,10 @@ struct SplitRhsList {
 // threads of a pair, for one right-hand side; the residual comes from eta on
 // the first visit of a colour, else from the kept rho and the crossing hops of
 // the kept delta.
-template <bool QNZ>
+// COPY: operator data from the block-by-block copy; else from the native fields
+// (f.U, f.A, f.C, plan.Cinv), the block's links made here from the same
+// expressions as in the copy. The results are the same bits.
+template <bool QNZ, bool COPY>
 __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm, int bidx, int colour,
                                                const Fields<float>& f, const SapPlan& plan,
                                                const SplitWork& wk, int flags, int nmr, float q) {
@@ -828,8 +859,9 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     const Site me = make_site(g, org, 2 * t + (sg ? 1 - sp.par0 : sp.par0));
     const int even_s = __shfl_sync(FULL_MASK, me.s, threadIdx.x & 30);  // native index of the even site
 
-    // the block's links, copied while the residual is formed
-    {
+    if constexpr (!COPY) {
+        block_links<QNZ>(g, f, me, sg, q, sW4, sW2);
+    } else {  // the block's links, copied while the residual is formed
         const float4* src = plan.links + (size_t)blk * PLAN_LINK_F4;
         for (int k = threadIdx.x; k < PLAN_LINK_F4; k += SPLIT_THREADS) copy_async16(sW4 + k, src + k);
     }
@@ -841,12 +873,15 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     const uint32_t Moi = tm + ((threadIdx.x & 96u) << 16) + (threadIdx.x >> 7) * (TM_COLS / 2);
     const uint32_t Mee = Moi + 2 * TM_BLOCK;
     {
-        const float4* src = plan.clover + (size_t)blk * PLAN_CLOVER_F4 + t;
-        float4 q[16];
-        clover_load(src, sg, q);
-        clover_rows(q, sg, Moi);
-        clover_load(src + CLOVER_F4 * SAP_HALF, sg, q);
-        clover_rows(q, sg, Mee);
+        const int odd_s = COPY ? 0 : __shfl_sync(FULL_MASK, me.s, (threadIdx.x & 30) | 1);
+        const float4* oi = COPY ? plan.clover + (size_t)blk * PLAN_CLOVER_F4 + t : plan.Cinv + odd_s;
+        const float4* ee = COPY ? oi + CLOVER_F4 * SAP_HALF : f.C + even_s;
+        const size_t stride = COPY ? SAP_HALF : g.V;
+        float4 c[16];
+        clover_load(oi, stride, sg, c);
+        clover_rows(c, sg, Moi);
+        clover_load(ee, stride, sg, c);
+        clover_rows(c, sg, Mee);
         tm_store_wait();
     }
 
@@ -967,7 +1002,7 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
 // L2. (One thread block for all right-hand sides of a block, its links staged
 // once, was slower at every size: 6 right-hand sides on 32x32x16x16 946 us each
 // against 818, 12 on 16x16x8x8 269 against 61, where it left SMs idle.)
-template <bool QNZ>
+template <bool QNZ, bool COPY>
 __global__ void __launch_bounds__(SPLIT_THREADS, 2) k_sap_split(const __grid_constant__ Geom g,
                                                                 const __grid_constant__ SapGeom sgm, int colour,
                                                                 const __grid_constant__ Fields<float> f,
@@ -975,7 +1010,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 2) k_sap_split(const __grid_con
                                                                 const __grid_constant__ SplitRhsList rl, int flags,
                                                                 int nmr, float q) {
     const int b = blockIdx.x / rl.n;
-    sap_split_body<QNZ>(g, sgm, b, colour, f, plan, rl.r[blockIdx.x - b * rl.n], flags, nmr, q);
+    sap_split_body<QNZ, COPY>(g, sgm, b, colour, f, plan, rl.r[blockIdx.x - b * rl.n], flags, nmr, q);
 }
 
 // The block-by-block copy of the operator for the split kernel: one thread
@@ -994,27 +1029,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_sap_plan(Geom g, SapGeom sgm,
     const int base = 2 * t;
     const int par0 = ((base >> 6) + ((base >> 4) & 3) + ((base >> 2) & 3) + (base & 3)) & 1;
     const Site me = make_site(g, org, base + (sg ? 1 - par0 : par0));
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-        if (me.l[mu] == SAP_BS - 1) continue;
-        const int e = mu == 0   ? link_entry<0>(sg, me.lidx)
-                      : mu == 1 ? link_entry<1>(sg, me.lidx)
-                      : mu == 2 ? link_entry<2>(sg, me.lidx)
-                                : link_entry<3>(sg, me.lidx);
-        cplx<float> u[3][3];
-        load_link(f.U, g.V, mu, me.s, u);
-        cplx<float> z = QNZ ? link_phase(f.A, g.V, mu, me.s, q) : mk(1.f, 0.f);
-        z = -0.5f * z;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) u[a][b] = z * u[a][b];
-        W4[(mu * 4 + 0) * SPLIT_LINKS + e] = make_float4(u[0][0].re, u[0][0].im, u[0][1].re, u[0][1].im);
-        W4[(mu * 4 + 1) * SPLIT_LINKS + e] = make_float4(u[0][2].re, u[0][2].im, u[1][0].re, u[1][0].im);
-        W4[(mu * 4 + 2) * SPLIT_LINKS + e] = make_float4(u[1][1].re, u[1][1].im, u[1][2].re, u[1][2].im);
-        W4[(mu * 4 + 3) * SPLIT_LINKS + e] = make_float4(u[2][0].re, u[2][0].im, u[2][1].re, u[2][1].im);
-        W2[mu * SPLIT_LINKS + e] = make_float2(u[2][2].re, u[2][2].im);
-    }
+    block_links<QNZ>(g, f, me, sg, q, W4, W2);
     float4* C = clover + (size_t)blk * PLAN_CLOVER_F4 + (sg ? 0 : CLOVER_F4 * SAP_HALF) + t;
     const float4* src = sg ? Cinv : f.C;
 #pragma unroll
@@ -1022,7 +1037,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_sap_plan(Geom g, SapGeom sgm,
 }
 
 // batched form: thread block b works on block (b - cta_begin) of the job
-// whose range holds b (one launch serves every job of a batch)
+// whose range holds b (one launch serves every job of a batch; without COPY all
+// of them read the native fields)
+template <bool COPY>
 __global__ void __launch_bounds__(SPLIT_THREADS, 2) k_sap_block_batch(const SapJob* __restrict__ jobs, int njobs,
                                                                       int colour, int flags, int nmr) {
     int lo = 0, hi = njobs - 1;
@@ -1034,7 +1051,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 2) k_sap_block_batch(const SapJ
     }
     const SapJob& J = jobs[lo];
     const SplitWork wk{J.eta, const_cast<float4*>(J.f.psi), J.delta, J.rho};
-    sap_split_body<true>(J.g, J.sg, b - J.cta_begin, colour, J.f, J.plan, wk, flags, nmr, J.q);
+    sap_split_body<true, COPY>(J.g, J.sg, b - J.cta_begin, colour, J.f, J.plan, wk, flags, nmr, J.q);
 }
 
 template <typename R>
@@ -1083,17 +1100,16 @@ int launch_sap_block64(qxd_lattice* lat, const SapGeom& sg, int cy, int colour, 
 }
 
 // FP32: the ncy cycles for the right-hand sides of rl (one operator)
-template <bool QNZ>
+template <bool QNZ, bool COPY>
 int split_cycles(qxd_lattice* lat, const SapGeom& sg, const SplitRhsList& rl, int ncy, int nmr, cudaStream_t st) {
     const size_t smem = sap_smem_bytes<float>();
-    int rc = split_attrs(k_sap_split<QNZ>, smem);
+    const int rc = split_attrs(k_sap_split<QNZ, COPY>, smem);
     if (rc) return rc;
-    SapPlan plan;
-    if ((rc = sap_plan(lat, st, &plan))) return rc;
-    const Fields<float> f{nullptr, nullptr, lat->U32, lat->A32, nullptr};
+    const SapPlan plan = sap_plan(lat);
+    const Fields<float> f{nullptr, nullptr, lat->U32, lat->A32, lat->C32};
     for (int cy = 0; cy < ncy; ++cy)
         for (int colour = 0; colour < 2; ++colour) {
-            k_sap_split<QNZ><<<sg.nhalf * rl.n, SPLIT_THREADS, smem, st>>>(lat->g, sg, colour, f, plan, rl,
+            k_sap_split<QNZ, COPY><<<sg.nhalf * rl.n, SPLIT_THREADS, smem, st>>>(lat->g, sg, colour, f, plan, rl,
                                                                            split_flags(cy, colour, ncy), nmr,
                                                                            (float)lat->qhat);
             QXD_LAUNCHED("k_sap_split");
@@ -1129,16 +1145,24 @@ int sap_check(qxd_lattice* lat) {
     return why ? fail(QXD_ERR_ARG, why) : QXD_OK;
 }
 
+bool sap_admissible(const qxd_lattice* lat) { return !sap_refusal(lat->g); }
+
+// Part of qxd_sw_build, which waits for it: the copy is complete before any
+// application, on whatever stream, can follow, and no application allocates.
+// Without memory for it the block solve reads the native fields (sap_split_body
+// without COPY: one application on 64x64x32x32 sites 12.78 ms instead of 11.08).
 int launch_sap_plan(qxd_lattice* lat, cudaStream_t st) {
     const SapGeom sg = sap_geom(lat->g);
-    if (!lat->sap_plan) {
-        const cudaError_t e =
-            cudaMalloc(&lat->sap_plan, (size_t)sg.nblk * (PLAN_LINK_F4 + PLAN_CLOVER_F4) * sizeof(float4));
+    if (!lat->sap_plan && lat->sap_copy_wanted) {
+        const size_t bytes = (size_t)sg.nblk * (PLAN_LINK_F4 + PLAN_CLOVER_F4) * sizeof(float4);
+        const cudaError_t e = cudaMalloc(&lat->sap_plan, bytes);
         if (e != cudaSuccess) {
             lat->sap_plan = nullptr;
-            return cuda_fail(e, "SAP: cudaMalloc(operator by blocks)");
+            if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "SAP: cudaMalloc(operator by blocks)");
+            cudaGetLastError();
         }
     }
+    if (!lat->sap_plan) return QXD_OK;
     const Fields<float> f{nullptr, nullptr, lat->U32, lat->A32, lat->C32};
     float4* clover = lat->sap_plan + (size_t)sg.nblk * PLAN_LINK_F4;
     if (lat->qhat != 0)
@@ -1150,19 +1174,9 @@ int launch_sap_plan(qxd_lattice* lat, cudaStream_t st) {
     return QXD_OK;
 }
 
-// Built with the operator (qxd_sw_build), so that requests on several streams
-// may share it; if there was no memory for it then, by the first application.
-bool sap_admissible(const qxd_lattice* lat) { return !sap_refusal(lat->g); }
-
-int sap_plan(qxd_lattice* lat, cudaStream_t st, SapPlan* plan) {
-    if (!lat->sap_plan || lat->sap_plan_version != lat->op_version) {
-        const int rc = launch_sap_plan(lat, st);
-        if (rc) return rc;
-        lat->sap_plan_version = lat->op_version;
-    }
-    const SapGeom sg = sap_geom(lat->g);
-    *plan = SapPlan{lat->sap_plan, lat->sap_plan + (size_t)sg.nblk * PLAN_LINK_F4};
-    return QXD_OK;
+SapPlan sap_plan(const qxd_lattice* lat) {
+    if (!lat->sap_plan) return SapPlan{nullptr, nullptr, lat->Cinv32};
+    return SapPlan{lat->sap_plan, lat->sap_plan + (size_t)sap_geom(lat->g).nblk * PLAN_LINK_F4, lat->Cinv32};
 }
 
 int sap_apply_multi(qxd_lattice* lat, int nrhs, void* const* outs, const void* const* ins, float4* const* works,
@@ -1175,8 +1189,11 @@ int sap_apply_multi(qxd_lattice* lat, int nrhs, void* const* outs, const void* c
         for (int i = 0; i < rl.n; ++i)
             rl.r[i] = SplitWork{(const float4*)ins[i0 + i], (float4*)outs[i0 + i], works[i0 + i],
                                 works[i0 + i] + (size_t)SPINOR_F4 * V};
-        const int rc = lat->qhat != 0 ? split_cycles<true>(lat, sg, rl, ncy, nmr, st)
-                                      : split_cycles<false>(lat, sg, rl, ncy, nmr, st);
+        const bool copy = lat->sap_plan != nullptr;
+        const int rc = lat->qhat != 0 ? (copy ? split_cycles<true, true>(lat, sg, rl, ncy, nmr, st)
+                                              : split_cycles<true, false>(lat, sg, rl, ncy, nmr, st))
+                                      : (copy ? split_cycles<false, true>(lat, sg, rl, ncy, nmr, st)
+                                              : split_cycles<false, false>(lat, sg, rl, ncy, nmr, st));
         if (rc) return rc;
     }
     return QXD_OK;
@@ -1238,19 +1255,22 @@ void SapGraphCache::release() {
 
 namespace {
 
-void launch_batch_set(const SapJob* d_jobs, int njobs, int ctas, int ncy, int nmr, size_t smem, cudaStream_t st) {
+void launch_batch_set(const SapJob* d_jobs, int njobs, int ctas, bool copy, int ncy, int nmr, size_t smem,
+                      cudaStream_t st) {
     for (int cy = 0; cy < ncy; ++cy)
-        for (int colour = 0; colour < 2; ++colour)
-            k_sap_block_batch<<<ctas, SPLIT_THREADS, smem, st>>>(d_jobs, njobs, colour, split_flags(cy, colour, ncy),
-                                                                 nmr);
+        for (int colour = 0; colour < 2; ++colour) {
+            const int fl = split_flags(cy, colour, ncy);
+            if (copy) k_sap_block_batch<true><<<ctas, SPLIT_THREADS, smem, st>>>(d_jobs, njobs, colour, fl, nmr);
+            else k_sap_block_batch<false><<<ctas, SPLIT_THREADS, smem, st>>>(d_jobs, njobs, colour, fl, nmr);
+        }
 }
 
 // the executable graph of this launch set, captured on first use
-int batch_graph(SapGraphCache& gc, const SapJob* d_jobs, int njobs, int ctas, int ncy, int nmr, size_t smem,
+int batch_graph(SapGraphCache& gc, const SapJob* d_jobs, int njobs, int ctas, bool copy, int ncy, int nmr, size_t smem,
                 cudaGraphExec_t* out) {
     ++gc.tick;
     for (auto& e : gc.entries)
-        if (e.table == d_jobs && e.njobs == njobs && e.ctas == ctas && e.ncy == ncy && e.nmr == nmr) {
+        if (e.table == d_jobs && e.njobs == njobs && e.ctas == ctas && e.copy == copy && e.ncy == ncy && e.nmr == nmr) {
             e.last = gc.tick;
             ++gc.replays;
             *out = e.exec;
@@ -1258,7 +1278,7 @@ int batch_graph(SapGraphCache& gc, const SapJob* d_jobs, int njobs, int ctas, in
         }
     if (!gc.cap) QXD_CUDA(cudaStreamCreateWithFlags(&gc.cap, cudaStreamNonBlocking));
     QXD_CUDA(cudaStreamBeginCapture(gc.cap, cudaStreamCaptureModeThreadLocal));
-    launch_batch_set(d_jobs, njobs, ctas, ncy, nmr, smem, gc.cap);
+    launch_batch_set(d_jobs, njobs, ctas, copy, ncy, nmr, smem, gc.cap);
     const cudaError_t le = cudaGetLastError();
     cudaGraph_t graph = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(gc.cap, &graph);  // always ends the capture
@@ -1276,7 +1296,7 @@ int batch_graph(SapGraphCache& gc, const SapJob* d_jobs, int njobs, int ctas, in
         cudaGraphExecDestroy(lru->exec);
         gc.entries.erase(lru);
     }
-    gc.entries.push_back(SapGraphCache::Entry{d_jobs, njobs, ctas, ncy, nmr, exec, gc.tick});
+    gc.entries.push_back(SapGraphCache::Entry{d_jobs, njobs, ctas, ncy, nmr, copy, exec, gc.tick});
     ++gc.captures;
     *out = exec;
     return QXD_OK;
@@ -1288,22 +1308,24 @@ int sap_apply_batch(std::vector<SapJob>& jobs, SapJob* d_jobs, int ncy, int nmr,
                     SapGraphCache* graphs) {
     if (jobs.empty()) return QXD_OK;
     int ctas = 0;
+    bool copy = true;  // every operator has its block-by-block copy
     for (auto& J : jobs) {  // the first visit of each colour writes psi without reading it
         J.cta_begin = ctas;
         ctas += J.sg.nhalf;
+        copy = copy && J.plan.links;
     }
     QXD_CUDA(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(SapJob), cudaMemcpyHostToDevice, st));
     const size_t smem = sap_smem_bytes<float>();
-    int rc = split_attrs(k_sap_block_batch, smem);
+    int rc = copy ? split_attrs(k_sap_block_batch<true>, smem) : split_attrs(k_sap_block_batch<false>, smem);
     if (rc) return rc;
     const int njobs = (int)jobs.size();
     if (graphs) {
         cudaGraphExec_t exec = nullptr;
-        if ((rc = batch_graph(*graphs, d_jobs, njobs, ctas, ncy, nmr, smem, &exec))) return rc;
+        if ((rc = batch_graph(*graphs, d_jobs, njobs, ctas, copy, ncy, nmr, smem, &exec))) return rc;
         QXD_CUDA(cudaGraphLaunch(exec, st));
         return QXD_OK;
     }
-    launch_batch_set(d_jobs, njobs, ctas, ncy, nmr, smem, st);
+    launch_batch_set(d_jobs, njobs, ctas, copy, ncy, nmr, smem, st);
     QXD_LAUNCHED("k_sap_block_batch");
     return QXD_OK;
 }
@@ -1364,4 +1386,11 @@ extern "C" int qxd_sap_multi(qxd_lattice* lat, int nrhs, void* const* out, const
     for (int i = 0; i < nrhs; ++i) works[i] = lat->sap_multi + per * i;
     cudaStream_t st = stream ? (cudaStream_t)stream : lat->stream;
     return sap_apply_multi(lat, nrhs, out, in, works.data(), ncy, nmr, st);
+}
+
+extern "C" int qxd_set_sap_copy(qxd_lattice* lat, int enable) {
+    if (!lat) return fail(QXD_ERR_ARG, "qxd_set_sap_copy: lat is NULL");
+    if (lat->sap_plan) return fail(QXD_ERR_STATE, "qxd_set_sap_copy: the lattice has its copy already");
+    lat->sap_copy_wanted = enable != 0;
+    return QXD_OK;
 }

@@ -21,14 +21,15 @@ struct SapWork {
     SapGeom sg{};
 };
 
-// the operator block by block, for the FP32 block solve (sap.cu): the compound
-// interior links and the clover blocks M_oo^-1, M_ee of every block
+// The operator block by block, for the FP32 block solve (sap.cu): the compound
+// interior links and the clover blocks M_oo^-1, M_ee of every block. links null:
+// no copy (no memory for it), M_oo^-1 in Cinv and the rest in the native fields.
 struct SapPlan {
     const float4* links;
     const float4* clover;
+    const float4* Cinv;
 };
-// lat's plan, built on st if sw_build had no memory for it
-int sap_plan(qxd_lattice* lat, cudaStream_t st, SapPlan* plan);
+SapPlan sap_plan(const qxd_lattice* lat);
 
 // one job of a batched SAP application (FP32): out = SAP(eta) on the job's
 // operator; f.psi is the output field
@@ -55,6 +56,7 @@ struct SapGraphCache {
     struct Entry {
         const void* table;
         int njobs, ctas, ncy, nmr;
+        bool copy;  // which form of the kernel
         cudaGraphExec_t exec;
         unsigned long long last;
     };

@@ -99,6 +99,7 @@ SIGNATURES = {
     "qxd_set_gauge": (_i, [_vp, _vp, _vp, _i]),
     "qxd_set_params": (_i, [_vp, _d, _d, _d, _i]),
     "qxd_sw_build": (_i, [_vp]),
+    "qxd_set_sap_copy": (_i, [_vp, _i]),
     "qxd_Dw": (_i, [_vp, _vp, _vp, _i, _vp]),
     "qxd_Dw_noalloc": (_i, [_vp, _vp, _vp, _i, _vp]),
     "qxd_Dw_batch": (_i, [_i, ctypes.POINTER(_vp), ctypes.POINTER(_vp), ctypes.POINTER(_vp), _i, _i, _vp]),
@@ -428,6 +429,10 @@ class Lattice:
 
     def sw_build(self):
         qxd_sw_build(self.handle)
+
+    def set_sap_copy(self, enable):
+        """qxd_set_sap_copy: whether sw_build lays the operator out for the FP32 Schwarz method."""
+        check(_call("qxd_set_sap_copy", self.handle, int(enable)))
 
     def spinor_bytes(self, prec):
         return qxd_spinor_bytes(self.handle, prec)
