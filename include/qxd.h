@@ -145,9 +145,10 @@ int qxd_set_params(qxd_lattice* lat, double m0, double csw, double cswqed, int q
  * singular to working precision or non-finite (inverse pivots below
  * 1e-12 of the block norm). On lattices that admit the Schwarz blocks of
  * qxd_sap it also lays the FP32 operator out block by block for it (504 bytes
- * per site, allocated by the first build and kept with the lattice; without
- * memory for it the FP32 Schwarz method reads the lattice's other fields, with
- * the same results, slower). Synchronises the lattice stream.
+ * per site, allocated by the first build that leaves half of the device memory
+ * and 16 times the copy free, and kept with the lattice; until then the FP32
+ * Schwarz method reads the lattice's other fields, with the same results,
+ * slower). Synchronises the lattice stream.
  */
 int qxd_sw_build(qxd_lattice* lat);
 

@@ -1147,6 +1147,23 @@ int sap_check(qxd_lattice* lat) {
 
 bool sap_admissible(const qxd_lattice* lat) { return !sap_refusal(lat->g); }
 
+namespace {
+
+// Whether the copy, which the Schwarz method can do without, may have its
+// memory: half of the device stays free, for the program's other lattices,
+// views and fields, and 16 times the copy (8 KB per site; a mixed GCR solve
+// with 16 Krylov pairs takes 4), for the work on this operator itself.
+bool copy_has_room(size_t bytes) {
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return free_bytes > bytes && free_bytes - bytes >= std::max(total / 2, 16 * bytes);
+}
+
+}  // namespace
+
 // Part of qxd_sw_build, which waits for it: the copy is complete before any
 // application, on whatever stream, can follow, and no application allocates.
 // Without memory for it the block solve reads the native fields (sap_split_body
@@ -1155,7 +1172,7 @@ int launch_sap_plan(qxd_lattice* lat, cudaStream_t st) {
     const SapGeom sg = sap_geom(lat->g);
     if (!lat->sap_plan && lat->sap_copy_wanted) {
         const size_t bytes = (size_t)sg.nblk * (PLAN_LINK_F4 + PLAN_CLOVER_F4) * sizeof(float4);
-        const cudaError_t e = cudaMalloc(&lat->sap_plan, bytes);
+        const cudaError_t e = copy_has_room(bytes) ? cudaMalloc(&lat->sap_plan, bytes) : cudaErrorMemoryAllocation;
         if (e != cudaSuccess) {
             lat->sap_plan = nullptr;
             if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "SAP: cudaMalloc(operator by blocks)");

@@ -147,3 +147,27 @@ def test_the_switch_is_for_before_the_copy():
     assert e.value.code == qxd.QXD_ERR_STATE
     a.close()
     b.close()
+
+
+def test_the_copy_leaves_half_of_the_memory():
+    """With less than half of the device memory free qxd_sw_build makes no copy
+    (the switch still answers then); once there is room the next build makes it."""
+    from paper_1710_08839_gb300 import qxd
+    c = Case(**SIZES[0], qhat=2)
+    x = c.psi.to(torch.complex64).cuda()
+    torch.cuda.empty_cache()
+    free, total = torch.cuda.mem_get_info()
+    taken = torch.empty(max(0, free - total // 2 + (64 << 20)), dtype=torch.uint8, device="cuda")
+    lat = c.lattice()
+    lat.set_sap_copy(1)
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    lat.sap(y, x, ncy=2, nmr=2)
+    torch.cuda.synchronize()
+    del taken
+    torch.cuda.empty_cache()
+    lat.sw_build()
+    with pytest.raises(qxd.QxdError):
+        lat.set_sap_copy(1)
+    lat.sap(z, x, ncy=2, nmr=2)
+    assert torch.equal(y, z)
+    lat.close()
