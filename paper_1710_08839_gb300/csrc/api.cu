@@ -65,10 +65,12 @@ static int alloc_pieces(void** arena, const Piece* pieces, int n, const char* wh
 
 // the arrays of the operator (lattices and views) and of the gauge field
 static int alloc_fields(qxd_lattice* L, bool gauge) {
-    const size_t v = (size_t)L->g.V;
+    const size_t v = (size_t)L->g.V, vh = (size_t)L->g.Vh;
+    // W64 to Cinv32 lie side by side (V is a multiple of 16, so each is one of
+    // 256 bytes): together they are the work space of leaf_buf
     const Piece op[] = {{(void**)&L->W64, 4 * 9 * v * sizeof(double2)}, {(void**)&L->C64, CLOVER_REALS * v * sizeof(double)},
-                        {(void**)&L->C32, CLOVER_F4 * v * sizeof(float4)}, {(void**)&L->Cinv64, CLOVER_REALS * v * sizeof(double)},
-                        {(void**)&L->Cinv32, CLOVER_F4 * v * sizeof(float4)}, {(void**)&L->d_status, 64 * sizeof(int)}};
+                        {(void**)&L->C32, CLOVER_F4 * v * sizeof(float4)}, {(void**)&L->Cinv64, CLOVER_REALS * vh * sizeof(double)},
+                        {(void**)&L->Cinv32, CLOVER_F4 * vh * sizeof(float4)}, {(void**)&L->d_status, 64 * sizeof(int)}};
     const Piece ga[] = {{(void**)&L->U64, 4 * 9 * v * sizeof(double2)}, {(void**)&L->U32, 4 * 3 * v * sizeof(float4)},
                         {(void**)&L->A64, 4 * v * sizeof(double)}, {(void**)&L->Z64, 4 * v * sizeof(double2)},
                         {(void**)&L->A32, v * sizeof(float4)}, {(void**)&L->ftens, FTENS_REALS * v * sizeof(double)}};

@@ -169,6 +169,7 @@ __device__ __forceinline__ void spin_flip_conj(double d[6], C64 l[15]) {
         }
 }
 
+// V: entries of the array per real, s: the site's
 __device__ __forceinline__ void store_packed(const double d[6], const C64 l[15], int blk, double* __restrict__ C64p,
                                              float4* __restrict__ C32p, size_t V, int s) {
     double v[36];
@@ -188,8 +189,9 @@ __device__ __forceinline__ void store_packed(const double d[6], const C64 l[15],
 }
 
 // One thread per (site, block): assemble the block from the field tensors,
-// store it, invert it (LDL^H, Gauss-Jordan with pivoting as the fallback); with
-// an exact mirror half both blocks of the mirror site follow. Bound by the FP64
+// store it, invert it (LDL^H, Gauss-Jordan with pivoting as the fallback; on the
+// even sites this only tells whether it is singular); with an exact mirror half
+// both blocks of the mirror site follow. Bound by the FP64
 // units. 48x48x24x24 sites: 1.96 ms; 5.24 ms for every site by itself, with 20
 // square roots and 40 divisions a block.
 __global__ void __launch_bounds__(128) k_clover_build(GaugeSet q, const double* __restrict__ F, double m0,
@@ -267,14 +269,17 @@ __global__ void __launch_bounds__(128) k_clover_build(GaugeSet q, const double* 
         }
         if (!ok) atomicAdd(&bad[0], q.mirror ? 2 : 1);
     }
-    store_packed(id, il, blk, Ci64, Ci32, V, s);
+    const bool odd = s >= g.Vh;  // and the mirror site with it: L1 is even
+    if (odd) store_packed(id, il, blk, Ci64, Ci32, g.Vh, s - g.Vh);
     if (q.mirror) {
         x[1] += g.L1;
         const int sm = native_of(g, x);
         spin_flip_conj(d, l);
         store_packed(d, l, blk, C64p, C32p, V, sm);
-        spin_flip_conj(id, il);
-        store_packed(id, il, blk, Ci64, Ci32, V, sm);
+        if (odd) {
+            spin_flip_conj(id, il);
+            store_packed(id, il, blk, Ci64, Ci32, g.Vh, sm - g.Vh);
+        }
     }
 }
 

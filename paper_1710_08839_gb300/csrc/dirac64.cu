@@ -274,7 +274,8 @@ __global__ void __launch_bounds__(DW_THREADS, 4)
     else dirac64_site<3>(g, f, in, out, x0b, nx0, d);
 }
 
-// the even-odd parts (modes of eo.cuh) on the sites of parity p
+// the even-odd parts (modes of eo.cuh) on the sites of parity p (the inverse
+// clover blocks of the odd sites, V/2 of each real)
 template <int NC, int MODE>
 __device__ __forceinline__ void dslash64_site(const Geom& g, int p, const Fields<double>& f, const SpRef<double>& in,
                                               const SpRef<double>& aux, const SpRefOut<double>& out,
@@ -290,7 +291,7 @@ __device__ __forceinline__ void dslash64_site(const Geom& g, int p, const Fields
     C64 hu[NC], hl[NC], u[NC], l[NC];
     hops64<NC>(g, f.U, in, sp, x0, x1, x2, x3, s, 1 - p, hu, hl);
     if (MODE == EO_INV_HOP) {
-        clover64_reg<NC>(Cl, g.V, s, sp, hu, hl, u, l);
+        clover64_reg<NC>(Cl, g.Vh, s - g.Vh, sp, hu, hl, u, l);
     } else if (MODE == EO_CLOVER_AUX_MHOP || MODE == EO_G5_CLOVER_AUX_MHOP) {
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
@@ -310,7 +311,7 @@ __device__ __forceinline__ void dslash64_site(const Geom& g, int p, const Fields
             l[k] = l[k] - hl[k];
         }
         if (MODE == EO_INV_AUX_MHOP) {
-            clover64_reg<NC>(Cl, g.V, s, sp, u, l, hu, hl);
+            clover64_reg<NC>(Cl, g.Vh, s - g.Vh, sp, u, l, hu, hl);
 #pragma unroll
             for (int k = 0; k < NC; ++k) {
                 u[k] = hu[k];
@@ -344,9 +345,9 @@ int launch_dirac64(qxd_lattice* lat, const SpRefOut<double>& out, const SpRef<do
 }
 
 int launch_eo64(qxd_lattice* lat, int mode, int p, const SpRef<double>& in, const SpRef<double>& aux,
-                const SpRefOut<double>& out, bool inverse, cudaStream_t st) {
+                const SpRefOut<double>& out, cudaStream_t st) {
     const Geom& g = lat->g;
-    const double* Cl = inverse ? lat->Cinv64 : lat->C64;
+    const double* Cl = eo_inverse(mode) ? lat->Cinv64 : lat->C64;
     const Fields<double> f{nullptr, nullptr, lat->W64, nullptr};
     const Deal d = deal(g.Vh, DW_THREADS);
     const int grid = d.full + d.rest;

@@ -12,6 +12,6 @@ int launch_dirac64(qxd_lattice* lat, const SpRefOut<double>& out, const SpRef<do
                    int x0b, int nx0, cudaStream_t st);
 // an even-odd part (mode as in eo.cuh) on the sites of parity p
 int launch_eo64(qxd_lattice* lat, int mode, int p, const SpRef<double>& in, const SpRef<double>& aux,
-                const SpRefOut<double>& out, bool inverse, cudaStream_t st);
+                const SpRefOut<double>& out, cudaStream_t st);
 
 }  // namespace qxd

@@ -13,7 +13,8 @@
 // FP64 in dirac64.cu. Each field is addressed as
 // (pointer, stride, offset): element k of the site with native index s is at
 // p[k * stride + s - offset], so full-lattice arrays (stride V, offset 0)
-// and half-lattice arrays (stride V/2, offset parity * V/2) both work.
+// and half-lattice arrays (stride V/2, offset parity * V/2) both work. M^-1 is
+// kept and applied on the odd sites only.
 #include <string>
 
 #include "dirac_common.cuh"
@@ -43,7 +44,7 @@ __global__ void __launch_bounds__(DW_THREADS, DW_PP_MIN_BLOCKS)
         cplx<float> t[12];
 #pragma unroll
         for (int i = 0; i < 12; ++i) t[i] = HS * acc[i];
-        clover_mul<true>(Cl, g.V, s, t, w);
+        clover_mul<true>(Cl, g.Vh, s - g.Vh, t, w);
     } else if (MODE == EO_CLOVER_AUX_MHOP || MODE == EO_G5_CLOVER_AUX_MHOP) {
         cplx<float> a[12];
         load_spinor(aux.p + aux.at(lex, s), aux.stride, 0, a);
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(DW_THREADS, DW_PP_MIN_BLOCKS)
         load_spinor(aux.p + aux.at(lex, s), aux.stride, 0, a);
 #pragma unroll
         for (int i = 0; i < 12; ++i) a[i] = rmad(-HS, acc[i], a[i]);
-        clover_mul<true>(Cl, g.V, s, a, w);
+        clover_mul<true>(Cl, g.Vh, s - g.Vh, a, w);
     }
     store_spinor(out.p + out.at(lex, s), out.stride, 0, w);
     if (out.zero_other) {
@@ -74,13 +75,12 @@ __global__ void __launch_bounds__(DW_THREADS, DW_PP_MIN_BLOCKS)
     }
 }
 
-// out = M in (or M^-1 in) on the sites of parity p
+// out = M_oo^-1 in on the odd sites
 template <typename R>
-__global__ void k_clover_half(Geom g, int p, SpRef<R> in, SpRefOut<R> out,
-                              const typename Fields<R>::cvec* __restrict__ Cl) {
+__global__ void k_minv_odd(Geom g, SpRef<R> in, SpRefOut<R> out, const typename Fields<R>::cvec* __restrict__ Cinv) {
     const int h = blockIdx.x * blockDim.x + threadIdx.x;
     if (h >= g.Vh) return;
-    const int s = p * g.Vh + h;
+    const int s = g.Vh + h;
     int lex = 0;
     if (in.lex || out.lex) {
         int x0, x1, x2, x3;
@@ -89,7 +89,7 @@ __global__ void k_clover_half(Geom g, int p, SpRef<R> in, SpRefOut<R> out,
     }
     cplx<R> a[12], w[12];
     load_spinor(in.p + in.at(lex, s), in.stride, 0, a);
-    clover_mul<true>(Cl, g.V, s, a, w);
+    clover_mul<true>(Cinv, g.Vh, h, a, w);
     store_spinor(out.p + out.at(lex, s), out.stride, 0, w);
 }
 
@@ -114,45 +114,47 @@ int launch_mode(qxd_lattice* lat, int mode, int p, const Fields<float>& f, SpRef
 
 template <>
 int launch_eo<float>(qxd_lattice* lat, int mode, int p, SpRef<float> in, SpRef<float> aux, SpRefOut<float> out,
-                     bool inverse, cudaStream_t st) {
+                     cudaStream_t st) {
+    if (eo_inverse(mode) && p != 1) return fail(QXD_ERR_ARG, "launch_eo: M^-1 is kept on the odd sites");
     const Fields<float> f = fields_of<float>(lat);
-    const float4* Cl = clover_of<float>(lat, inverse);
+    const float4* Cl = clover_of<float>(lat, eo_inverse(mode));
     if (lat->qhat != 0) return launch_mode<true>(lat, mode, p, f, in, aux, out, Cl, st);
     return launch_mode<false>(lat, mode, p, f, in, aux, out, Cl, st);
 }
 template <>
 int launch_eo<double>(qxd_lattice* lat, int mode, int p, SpRef<double> in, SpRef<double> aux, SpRefOut<double> out,
-                      bool inverse, cudaStream_t st) {
-    return launch_eo64(lat, mode, p, in, aux, out, inverse, st);
+                      cudaStream_t st) {
+    if (eo_inverse(mode) && p != 1) return fail(QXD_ERR_ARG, "launch_eo: M^-1 is kept on the odd sites");
+    return launch_eo64(lat, mode, p, in, aux, out, st);
 }
 
 template <typename R>
-int launch_clover_half(qxd_lattice* lat, int p, SpRef<R> in, SpRefOut<R> out, bool inverse, cudaStream_t st) {
+int launch_minv_odd(qxd_lattice* lat, SpRef<R> in, SpRefOut<R> out, cudaStream_t st) {
     const Geom& g = lat->g;
     const int blocks = (g.Vh + 255) / 256;
-    k_clover_half<R><<<blocks, 256, 0, st>>>(g, p, in, out, clover_of<R>(lat, inverse));
-    QXD_LAUNCHED("k_clover_half");
+    k_minv_odd<R><<<blocks, 256, 0, st>>>(g, in, out, clover_of<R>(lat, true));
+    QXD_LAUNCHED("k_minv_odd");
     return QXD_OK;
 }
 
-template int launch_clover_half<float>(qxd_lattice*, int, SpRef<float>, SpRefOut<float>, bool, cudaStream_t);
-template int launch_clover_half<double>(qxd_lattice*, int, SpRef<double>, SpRefOut<double>, bool, cudaStream_t);
+template int launch_minv_odd<float>(qxd_lattice*, SpRef<float>, SpRefOut<float>, cudaStream_t);
+template int launch_minv_odd<double>(qxd_lattice*, SpRef<double>, SpRefOut<double>, cudaStream_t);
 
 // D_hat psi_e = M_ee psi_e - H_eo M_oo^-1 H_oe psi_e; tmp is an odd-parity field
 template <typename R>
 int apply_dhat(qxd_lattice* lat, SpRefOut<R> out_e, SpRef<R> in_e, SpRefOut<R> tmp_o, cudaStream_t st) {
-    int rc = launch_eo<R>(lat, EO_INV_HOP, 1, in_e, SpRef<R>{}, tmp_o, true, st);
+    int rc = launch_eo<R>(lat, EO_INV_HOP, 1, in_e, SpRef<R>{}, tmp_o, st);
     if (rc) return rc;
-    return launch_eo<R>(lat, EO_CLOVER_AUX_MHOP, 0, as_in(tmp_o), in_e, out_e, false, st);
+    return launch_eo<R>(lat, EO_CLOVER_AUX_MHOP, 0, as_in(tmp_o), in_e, out_e, st);
 }
 template int apply_dhat<float>(qxd_lattice*, SpRefOut<float>, SpRef<float>, SpRefOut<float>, cudaStream_t);
 template int apply_dhat<double>(qxd_lattice*, SpRefOut<double>, SpRef<double>, SpRefOut<double>, cudaStream_t);
 
 template <typename R>
 int apply_g5dhat(qxd_lattice* lat, SpRefOut<R> out_e, SpRef<R> in_e, SpRefOut<R> tmp_o, cudaStream_t st) {
-    int rc = launch_eo<R>(lat, EO_INV_HOP, 1, in_e, SpRef<R>{}, tmp_o, true, st);
+    int rc = launch_eo<R>(lat, EO_INV_HOP, 1, in_e, SpRef<R>{}, tmp_o, st);
     if (rc) return rc;
-    return launch_eo<R>(lat, EO_G5_CLOVER_AUX_MHOP, 0, as_in(tmp_o), in_e, out_e, false, st);
+    return launch_eo<R>(lat, EO_G5_CLOVER_AUX_MHOP, 0, as_in(tmp_o), in_e, out_e, st);
 }
 template int apply_g5dhat<float>(qxd_lattice*, SpRefOut<float>, SpRef<float>, SpRefOut<float>, cudaStream_t);
 template int apply_g5dhat<double>(qxd_lattice*, SpRefOut<double>, SpRef<double>, SpRefOut<double>, cudaStream_t);
@@ -168,15 +170,15 @@ int eo_parts(qxd_lattice* lat, int what, SpRefOut<R> out, SpRef<R> in, SpRef<R> 
     const int V = lat->g.V;
     int rc;
     if (what == EOAPI_RECONSTRUCT)  // out holds x (even part read); in holds b
-        return launch_eo<R>(lat, EO_INV_AUX_MHOP, 1, gin, in, out, true, st);
+        return launch_eo<R>(lat, EO_INV_AUX_MHOP, 1, gin, in, out, st);
     out.zero_other = 1;  // the odd sites of out
     if (what == EOAPI_DHAT) {  // tmp (odd half of a full array) holds M_oo^-1 H_oe in_e
         const SpRefOut<R> t = full_out<R>(tmp, V);
-        if ((rc = launch_eo<R>(lat, EO_INV_HOP, 1, gin, SpRef<R>{}, t, true, st))) return rc;
-        return launch_eo<R>(lat, EO_CLOVER_AUX_MHOP, 0, as_in(t), in, out, false, st);
+        if ((rc = launch_eo<R>(lat, EO_INV_HOP, 1, gin, SpRef<R>{}, t, st))) return rc;
+        return launch_eo<R>(lat, EO_CLOVER_AUX_MHOP, 0, as_in(t), in, out, st);
     }
-    if ((rc = launch_clover_half<R>(lat, 1, in, full_out<R>(tmp, V), true, st))) return rc;
-    return launch_eo<R>(lat, EO_AUX_MHOP, 0, full_ref<R>(tmp, V), in, out, false, st);
+    if ((rc = launch_minv_odd<R>(lat, in, full_out<R>(tmp, V), st))) return rc;
+    return launch_eo<R>(lat, EO_AUX_MHOP, 0, full_ref<R>(tmp, V), in, out, st);
 }
 
 template <typename R>

@@ -85,11 +85,12 @@ inline const double* clover_of<double>(qxd_lattice* lat, bool inverse) {
     return inverse ? lat->Cinv64 : lat->C64;
 }
 
+// the modes with M^-1 are for the odd sites, p = 1 (QXD_ERR_ARG otherwise)
+inline bool eo_inverse(int mode) { return mode == EO_INV_HOP || mode == EO_INV_AUX_MHOP; }
 template <typename R>
-int launch_eo(qxd_lattice* lat, int mode, int p, SpRef<R> in, SpRef<R> aux, SpRefOut<R> out, bool inverse,
-              cudaStream_t st);
+int launch_eo(qxd_lattice* lat, int mode, int p, SpRef<R> in, SpRef<R> aux, SpRefOut<R> out, cudaStream_t st);
 template <typename R>
-int launch_clover_half(qxd_lattice* lat, int p, SpRef<R> in, SpRefOut<R> out, bool inverse, cudaStream_t st);
+int launch_minv_odd(qxd_lattice* lat, SpRef<R> in, SpRefOut<R> out, cudaStream_t st);
 template <typename R>
 int apply_dhat(qxd_lattice* lat, SpRefOut<R> out_e, SpRef<R> in_e, SpRefOut<R> tmp_o, cudaStream_t st);
 // gamma5 D_hat psi_e (Hermitian: D_hat^dag = gamma5 D_hat gamma5)

@@ -337,12 +337,13 @@ int qxd_wflow(qxd_lattice* lat, double eps, int nsteps) {
     const Geom& g = lat->g;
     const size_t V = (size_t)g.V;
     const bool cstar1 = lat->cstar_mask & 2u;
-    // Work space: the clover arrays, stale after the flow. Leaves and sines in
-    // leaf_buf; the accumulators in the FP32 inverse clover (36 V doubles) and
-    // behind the sines in the FP32 clover (6 + 4 of its 36 V).
+    // Work space: the operator's arrays, stale after the flow. The three leaves
+    // of the six planes take 162 V doubles of leaf_buf's 216 V; the accumulators
+    // (36 V and 4 V) lie behind them.
     const GaugeSet q = gauge_set(g, cstar1);
-    double* X = (double*)lat->Cinv32;
-    double* Xa = (double*)lat->C32 + 6 * V;
+    double* X = leaf_buf(lat, q.n).b + (size_t)6 * 3 * 9 * V;
+    double* Xa = X + 4 * 9 * V;
+    static_assert(6 * 3 * 9 + 4 * 9 + 4 <= LEAF_REALS, "accumulators before the sines");
     const double coef[3][2] = {{0.25, 0.0}, {8.0 / 9.0, -17.0 / 9.0}, {0.75, -1.0}};
     bool exact = mirror_exact(lat);
     lat->has_clover = false;

@@ -176,6 +176,8 @@ __host__ __device__ __forceinline__ int neighbour_lex(const Geom& g, int x0, int
 //                                   below the diagonal, row major
 //                                   ((1,0),(2,0),(2,1),(3,0),...,(5,4))
 // clover FP64 : double  C[72][V]    same 72 reals
+// their inverses             [Vh]   on the odd sites only (site s at s - Vh):
+//                                   M_oo^-1 is the one that is applied
 // field tensor: double  F[60][V]    per plane (01,02,03,12,13,23): the SU(3)
 //                                   anti-Hermitian 3x3 F_hat as 9 reals
 //                                   (Im d0, Im d1, Im d2, re/im of the upper
@@ -279,8 +281,8 @@ struct qxd_lattice {
     double2* W64 = nullptr;    // [4][9][V] -1/2 z^qhat U for this operator's qhat (FP64 kernels)
     double* C64 = nullptr;     // [72][V]
     float4* C32 = nullptr;     // [18][V]
-    double* Cinv64 = nullptr;  // [72][V]
-    float4* Cinv32 = nullptr;  // [18][V]
+    double* Cinv64 = nullptr;  // [72][Vh]
+    float4* Cinv32 = nullptr;  // [18][Vh]
     bool has_clover = false;
 
     // the allocations that hold the gauge field and the operator's arrays

@@ -234,7 +234,7 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
         residual_at<R>(g, f, eta, k ? so : se, psi_zero, k ? v : re);
     }
     s_ro.store(t, v);
-    clover_mul(Cinv, g.V, so.s, v, w);  // t_o = M_oo^-1 r_o
+    clover_mul(Cinv, g.Vh, so.s - g.Vh, v, w);  // t_o = M_oo^-1 r_o
     s_t.store(t, w);
     __syncthreads();
 
@@ -257,9 +257,9 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
             s_ro.load(t, v);
 #pragma unroll
             for (int i = 0; i < 12; ++i) v[i] = v[i] - acc[i];
-            clover_mul(Cinv, g.V, so.s, v, w);  // delta_o
+            clover_mul(Cinv, g.Vh, so.s - g.Vh, v, w);  // delta_o
         } else if (odd) {
-            clover_mul(Cinv, g.V, so.s, acc, w);
+            clover_mul(Cinv, g.Vh, so.s - g.Vh, acc, w);
             s_t.store(t, w);
         } else {
 #pragma unroll
@@ -874,13 +874,12 @@ __device__ __forceinline__ void sap_split_body(const Geom& g, const SapGeom& sgm
     const uint32_t Mee = Moi + 2 * TM_BLOCK;
     {
         const int odd_s = COPY ? 0 : __shfl_sync(FULL_MASK, me.s, (threadIdx.x & 30) | 1);
-        const float4* oi = COPY ? plan.clover + (size_t)blk * PLAN_CLOVER_F4 + t : plan.Cinv + odd_s;
+        const float4* oi = COPY ? plan.clover + (size_t)blk * PLAN_CLOVER_F4 + t : plan.Cinv + (odd_s - g.Vh);
         const float4* ee = COPY ? oi + CLOVER_F4 * SAP_HALF : f.C + even_s;
-        const size_t stride = COPY ? SAP_HALF : g.V;
         float4 c[16];
-        clover_load(oi, stride, sg, c);
+        clover_load(oi, COPY ? SAP_HALF : g.Vh, sg, c);
         clover_rows(c, sg, Moi);
-        clover_load(ee, stride, sg, c);
+        clover_load(ee, COPY ? SAP_HALF : g.V, sg, c);
         clover_rows(c, sg, Mee);
         tm_store_wait();
     }
@@ -1031,9 +1030,10 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_sap_plan(Geom g, SapGeom sgm,
     const Site me = make_site(g, org, base + (sg ? 1 - par0 : par0));
     block_links<QNZ>(g, f, me, sg, q, W4, W2);
     float4* C = clover + (size_t)blk * PLAN_CLOVER_F4 + (sg ? 0 : CLOVER_F4 * SAP_HALF) + t;
-    const float4* src = sg ? Cinv : f.C;
+    const float4* src = sg ? Cinv + (me.s - g.Vh) : f.C + me.s;
+    const size_t stride = sg ? g.Vh : g.V;
 #pragma unroll
-    for (int n = 0; n < CLOVER_F4; ++n) C[n * SAP_HALF] = src[(size_t)n * g.V + me.s];
+    for (int n = 0; n < CLOVER_F4; ++n) C[n * SAP_HALF] = src[n * stride];
 }
 
 // batched form: thread block b works on block (b - cta_begin) of the job

@@ -263,11 +263,10 @@ int run_solve(qxd_lattice* lat, const qxd_solver_params& P, qxd_solve_info& info
     if (eo) {
         // b_hat_e = b_e - H_eo M_oo^-1 b_o
         const int Vh = g.Vh;
-        if ((rc = launch_clover_half<double>(lat, 1, full_ref<double>(w.b64, g.V), half_out<double>(w.tmp64, Vh, 1),
-                                             true, st)))
+        if ((rc = launch_minv_odd<double>(lat, full_ref<double>(w.b64, g.V), half_out<double>(w.tmp64, Vh, 1), st)))
             return rc;
         if ((rc = launch_eo<double>(lat, EO_AUX_MHOP, 0, half_ref<double>(w.tmp64, Vh, 1),
-                                    full_ref<double>(w.b64, g.V), half_out<double>(w.bs, Vh, 0), false, st)))
+                                    full_ref<double>(w.b64, g.V), half_out<double>(w.bs, Vh, 0), st)))
             return rc;
     } else {
         QXD_CUDA(cudaMemcpyAsync(w.bs, w.b64, nfull * sizeof(double2), cudaMemcpyDeviceToDevice, st));
@@ -280,7 +279,7 @@ int run_solve(qxd_lattice* lat, const qxd_solver_params& P, qxd_solve_info& info
         const int Vh = g.Vh;
         if ((rc = copy_parity(lat, 0, half_ref<double>(w.xs, Vh, 0), full_out<double>(w.x64, g.V), st))) return rc;
         if ((rc = launch_eo<double>(lat, EO_INV_AUX_MHOP, 1, half_ref<double>(w.xs, Vh, 0),
-                                    full_ref<double>(w.b64, g.V), full_out<double>(w.x64, g.V), true, st)))
+                                    full_ref<double>(w.b64, g.V), full_out<double>(w.x64, g.V), st)))
             return rc;
     } else {
         QXD_CUDA(cudaMemcpyAsync(w.x64, w.xs, nfull * sizeof(double2), cudaMemcpyDeviceToDevice, st));

@@ -179,17 +179,17 @@ __host__ __device__ __forceinline__ void plane_dirs(int plane, int& mu, int& nu)
 __host__ __device__ __forceinline__ int plane_of(int mu, int nu) { return mu == 0 ? nu - 1 : mu == 1 ? nu + 1 : 5; }
 
 // Leaf buffers, in arrays of the lattice that a new gauge field makes stale: the
-// clover, its inverse and the hop links (72 V doubles each) hold the leaves of
-// two planes each, per plane one after the other, nine reals each (at most 4 x
-// 9 x 2 = 72); the FP32 clover (36 V doubles) holds the sines of the U(1)
-// plaquette angles, one per plane.
+// hop links, the clover terms and their inverses, 234 V doubles side by side.
+// First the leaves of the six planes, nine reals each (at most 6 x 4 x 9 = 216),
+// then the sines of the U(1) plaquette angles, one per plane.
+constexpr int LEAF_REALS = 216;
 struct LeafBuf {
-    double* b[3];
+    double* b;
     double* sine;
     size_t n;  // sites of the set, at most V
     template <int LEAVES>
     __device__ __forceinline__ double* leaf(int plane, int l) const {
-        return b[plane >> 1] + (size_t)((plane & 1) * LEAVES + l) * 9 * n;
+        return b + (size_t)(plane * LEAVES + l) * 9 * n;
     }
     __device__ __forceinline__ double* sines(int plane) const { return sine + (size_t)plane * n; }
 };
@@ -243,7 +243,8 @@ __device__ __forceinline__ void plaquette_leaves(const GaugeSet& q, const double
 // physical half (built or flowed as such), so that x1 < L1 carries everything
 inline bool mirror_exact(const qxd_lattice* lat) { return (lat->cstar_mask & 2u) && lat->mirror_built; }
 inline LeafBuf leaf_buf(const qxd_lattice* lat, int n) {
-    return LeafBuf{{lat->C64, lat->Cinv64, (double*)lat->W64}, (double*)lat->C32, (size_t)n};
+    double* b = (double*)lat->W64;
+    return LeafBuf{b, b + (size_t)LEAF_REALS * lat->g.V, (size_t)n};
 }
 
 }  // namespace qxd
