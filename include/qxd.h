@@ -605,7 +605,8 @@ int qxd_spinor_unpack(qxd_lattice* lat, void* lex_out, const void* native_in, in
  * output of every call comes from the chosen shape; all shapes compute the
  * same per-site sums in the same order. A first call inside a stream
  * capture must not tune: pin the shape (qxd_dw_set_shape) or make a first
- * call before the capture.
+ * call before the capture. A shape timed on lexicographic fields holds until
+ * the first call on native ones, which is timed in its place.
  * ------------------------------------------------------------------------- */
 /* enable = 0 or 1; returns the previous setting */
 int qxd_set_autotune(int enable);

@@ -160,17 +160,26 @@ int tune_dirac(qxd_lattice* lat, void* out, const void* in, int prec, bool lex, 
 
 namespace {
 
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
+}
+
 int dirac_full(qxd_lattice* lat, void* out, const void* in, int prec, bool lex, cudaStream_t st) {
     const DwKey key = dw_key(lat, prec);
+    const bool tune = autotune_enabled();
     DwShape sh;
-    if (!dw_shape_get(key, &sh)) {
-        if (autotune_enabled()) {
+    bool timed_lex = false;
+    // a shape timed on lexicographic fields is not kept for native ones, which
+    // the solvers apply D to, unless the call cannot be timed
+    if (!dw_shape_get(key, &sh, &timed_lex) || (timed_lex && !lex && tune && !capturing(st))) {
+        if (tune) {
             int rc = tune_dirac(lat, out, in, prec, lex, st, &sh);
             if (rc) return rc;
         } else {
             sh = dw_default_shape(lat, prec);
         }
-        dw_shape_put(key, sh, autotune_enabled() ? "tuned" : "default");
+        dw_shape_put(key, sh, tune ? "tuned" : "default", tune && lex);
     }
     return launch_dirac_shape(lat, out, in, prec, sh, st, 0, -1, lex);
 }

@@ -16,6 +16,7 @@ namespace {
 struct Entry {
     DwShape sh;
     std::string how;  // "tuned", "default" or "set"
+    bool lex;         // timed on lexicographic fields
 };
 
 std::mutex g_mu;
@@ -33,17 +34,18 @@ DwShape dw_default_shape(const qxd_lattice* lat, int prec) {
     return DwShape{prec == QXD_FP32 ? 1 : 0, DW_THREADS, lat->g.R, 0.f};
 }
 
-bool dw_shape_get(const DwKey& key, DwShape* out) {
+bool dw_shape_get(const DwKey& key, DwShape* out, bool* lex) {
     std::lock_guard<std::mutex> lock(g_mu);
     auto it = g_table.find(key);
     if (it == g_table.end()) return false;
     *out = it->second.sh;
+    if (lex) *lex = it->second.lex;
     return true;
 }
 
-void dw_shape_put(const DwKey& key, const DwShape& sh, const char* how) {
+void dw_shape_put(const DwKey& key, const DwShape& sh, const char* how, bool lex) {
     std::lock_guard<std::mutex> lock(g_mu);
-    g_table[key] = Entry{sh, how};
+    g_table[key] = Entry{sh, how, lex};
 }
 
 bool autotune_enabled() { return g_autotune.load() != 0; }
@@ -89,11 +91,12 @@ int qxd_tune_report(char* buf, size_t len, size_t* needed) {
             const DwKey& k = kv.first;
             const DwShape& sh = kv.second.sh;
             std::snprintf(line, sizeof line,
-                          "Dw %s qhat%s %dx%dx%dx%d cstar=%u: %s threads=%d rows=%d window=%lld sites ms=%.4f (%s)\n",
+                          "Dw %s qhat%s %dx%dx%dx%d cstar=%u: %s threads=%d rows=%d window=%lld sites ms=%.4f (%s)%s\n",
                           std::get<0>(k) == QXD_FP32 ? "fp32" : "fp64", std::get<1>(k) ? "!=0" : "=0", std::get<2>(k),
                           std::get<3>(k), std::get<4>(k), std::get<5>(k), std::get<6>(k),
                           sh.pipelined ? "pipelined" : "plain", sh.threads, sh.rows,
-                          (long long)std::get<3>(k) * sh.rows * std::get<5>(k), sh.ms, kv.second.how.c_str());
+                          (long long)std::get<3>(k) * sh.rows * std::get<5>(k), sh.ms, kv.second.how.c_str(),
+                          kv.second.lex ? " on lexicographic fields" : "");
             out += line;
         }
     }

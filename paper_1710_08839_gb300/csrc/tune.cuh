@@ -1,5 +1,7 @@
 // Launch-shape autotuning of the D kernels: the process-wide table of chosen
-// shapes, keyed by lattice shape and precision.
+// shapes, keyed by lattice shape and precision. A shape timed on lexicographic
+// fields stands only until D is first applied to native ones (the solvers'),
+// which then time their own.
 #pragma once
 
 #include <string>
@@ -24,8 +26,9 @@ using DwKey = std::tuple<int, int, int, int, int, int, unsigned>;
 
 DwKey dw_key(const qxd_lattice* lat, int prec);
 DwShape dw_default_shape(const qxd_lattice* lat, int prec);
-bool dw_shape_get(const DwKey& key, DwShape* out);
-void dw_shape_put(const DwKey& key, const DwShape& sh, const char* how);
+// lex: whether the shape was timed on lexicographic fields
+bool dw_shape_get(const DwKey& key, DwShape* out, bool* lex = nullptr);
+void dw_shape_put(const DwKey& key, const DwShape& sh, const char* how, bool lex = false);
 bool autotune_enabled();
 // the rhs-per-site choices of the batched D, as text lines (batch.cu)
 void dw_batch_report(std::string& out);
