@@ -38,8 +38,18 @@ struct DwGroup {
     int cta_begin;
 };
 
+// Several right-hand sides per site in FP32: 128 registers (4 blocks per SM, 8
+// bytes spilled). With 80 registers for 6 blocks 112 bytes are spilled, which
+// costs more than the occupancy gives: two per site, 6 right-hand sides on
+// 32x32x16x16 sites 267 us, with 5 blocks 255, with 4 250; over 1024 to 262144
+// sites and 1 to 8 right-hand sides 4 blocks take 0.80 to 1.02 of the time of 6.
+// One per site: 6 blocks (205 us; 5: 204, and slower where 5 make one more round,
+// 49.0 -> 51.7 us for 4 right-hand sides on 24x24x12x12).
 template <typename R, int NR>
-__global__ void __launch_bounds__(DW_THREADS, DwMinBlocks<R>::value)
+constexpr int batch_min_blocks() { return sizeof(R) == 4 && NR > 1 ? 4 : DwMinBlocks<R>::value; }
+
+template <typename R, int NR>
+__global__ void __launch_bounds__(DW_THREADS, (batch_min_blocks<R, NR>()))
     k_dirac_batch(const DwGroup<R>* __restrict__ groups, int ngroups) {
     // group of this thread block
     int lo = 0, hi = ngroups - 1;
