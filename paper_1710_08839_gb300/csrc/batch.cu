@@ -30,7 +30,7 @@ namespace {
 template <typename R>
 struct DwGroup {
     Geom g;
-    Fields<R> f;  // psi/out unused; U, A, C of the group's operator
+    Fields<R> f;  // psi unused; U, A, C of the group's operator
     R q;
     int nr;                                     // right-hand sides in this group (<= NR)
     const typename Fields<R>::vec* in[BATCH_MAXR];
@@ -87,11 +87,11 @@ template <typename R>
 Fields<R> op_fields(qxd_lattice* lat);
 template <>
 Fields<float> op_fields<float>(qxd_lattice* lat) {
-    return Fields<float>{nullptr, nullptr, lat->U32, lat->A32, lat->C32};
+    return Fields<float>{nullptr, lat->U32, lat->A32, lat->C32};
 }
 template <>
 Fields<double> op_fields<double>(qxd_lattice* lat) {
-    return Fields<double>{nullptr, nullptr, lat->W64, lat->C64};
+    return Fields<double>{nullptr, lat->W64, lat->C64};
 }
 
 // device buffer for group tables, grown on demand, one per (device, stream)

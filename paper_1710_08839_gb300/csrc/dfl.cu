@@ -493,7 +493,7 @@ void launch_invert(DflWork& W, cudaStream_t st);  // A_oo^-1 of the odd blocks (
 
 int build_little(qxd_lattice* lat, DflWork& W, cudaStream_t st) {
     const Geom& g = lat->g;
-    Fields<float> f{nullptr, nullptr, lat->U32, lat->A32, lat->C32};
+    Fields<float> f{nullptr, lat->U32, lat->A32, lat->C32};
     const float q = (float)lat->qhat;
     int rc;
     for (int l = 0; l < W.ns; ++l) {

@@ -84,7 +84,7 @@ int launch_dirac_shape(qxd_lattice* lat, void* out, const void* in, int prec, co
     const int blocks = (n + sh.threads - 1) / sh.threads;
     const bool qnz = lat->qhat != 0;
     if (prec == QXD_FP32) {
-        const Fields<float> f{(const float4*)in, nullptr, lat->U32, lat->A32, lat->C32};
+        const Fields<float> f{(const float4*)in, lat->U32, lat->A32, lat->C32};
         const SpRefOut<float> o = lex ? lex_out<float>(out) : full_out<float>(out, g.V);
         if (sh.pipelined) {
             if (qnz) k_dirac32<true><<<blocks, sh.threads, 0, st>>>(g, f, o, (float)lat->qhat, x0b, nx0, n);

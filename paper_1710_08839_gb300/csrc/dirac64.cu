@@ -9,13 +9,14 @@
 // site is split over 2 threads (by spin, 552 instructions each) and the warps
 // are dealt out so that each of the 608 schedulers gets the same number; what
 // is left over, up to 4864 sites, is split further, over 6 threads (spin and
-// colour, 232 instructions; 8 lanes with two idle). Measured: 262144 sites 515
-// us (0.90 of the FP64 issue rate; one thread per site 800 before the compound
-// links and multiply-add chains), 41472 sites of D_hat's first half 91 us (four
-// rounds of 552 and two of 232; one thread per site 120 us), D on 1024
-// lexicographic sites 12.3 us for the call (one thread per site, with the two
-// layout conversions, 55 us). 128 registers (4 blocks of 128 threads): 96 with
-// spills took 3-5 % longer on 41472 sites.
+// colour, 216 instructions: 8 hops x 18, 7 accumulations x 4, 44 for the clover
+// rows; 8 lanes with two idle). Measured: 262144 sites 515 us (0.90 of the FP64
+// issue rate; one thread per site 800 before the compound links and multiply-add
+// chains), 41472 sites of D_hat's first half 91 us (four rounds of 552 and two of
+// 216; one thread per site 120 us), D on 1024 lexicographic sites 12.3 us for the
+// call (one thread per site, with the two layout conversions, 55 us). 128
+// registers (4 blocks of 128 threads): 96 with spills took 3-5 % longer on 41472
+// sites.
 // In the chiral basis (1 -+ g_mu) psi is fixed by the half spinor (h_0, h_1):
 // the thread of spin s forms h_s from two spin components of the neighbour
 // (spin s, and spin 2 + s for mu = 0, 3 or 3 - s for mu = 1, 2), takes W h_s,
@@ -60,7 +61,7 @@ Deal deal(int n, int threads) {
     const int warps = threads / 32;
     d.full = (n / 16) / SCHEDULERS * SCHEDULERS / warps;
     const int left = n - d.full * warps * 16;
-    // 6 threads per site: two rounds of 232 instructions at most, against one of
+    // 6 threads per site: two rounds of 216 instructions at most, against one of
     // 552 (next to full blocks too: 41472 sites 97 -> 91 us)
     d.fine = left <= SCHEDULERS * 8;
     const int chunks = d.fine ? (left + 3) / 4 : (left + 15) / 16;
@@ -337,7 +338,7 @@ int launch_dirac64(qxd_lattice* lat, const SpRefOut<double>& out, const SpRef<do
                    int x0b, int nx0, cudaStream_t st) {
     Geom g = lat->g;
     g.R = rows;
-    const Fields<double> f{nullptr, nullptr, lat->W64, lat->C64};
+    const Fields<double> f{nullptr, lat->W64, lat->C64};
     const Deal d = deal(nx0 * g.N1 * g.N2 * g.N3, threads);
     k_dirac64<<<d.full + d.rest, threads, 0, st>>>(g, f, in, out, x0b, nx0, d);
     QXD_LAUNCHED("k_dirac64");
@@ -348,7 +349,7 @@ int launch_eo64(qxd_lattice* lat, int mode, int p, const SpRef<double>& in, cons
                 const SpRefOut<double>& out, cudaStream_t st) {
     const Geom& g = lat->g;
     const double* Cl = eo_inverse(mode) ? lat->Cinv64 : lat->C64;
-    const Fields<double> f{nullptr, nullptr, lat->W64, nullptr};
+    const Fields<double> f{nullptr, lat->W64, nullptr};
     const Deal d = deal(g.Vh, DW_THREADS);
     const int grid = d.full + d.rest;
     switch (mode) {

@@ -334,7 +334,7 @@ struct Engine {
                 SapJob J{};
                 J.g = j->op->g;
                 J.sg = sap_geom(j->op->g);
-                J.f = Fields<float>{(const float4*)j->phi[j->k], nullptr, j->op->U32, j->op->A32, j->op->C32};
+                J.f = Fields<float>{(const float4*)j->phi[j->k], j->op->U32, j->op->A32, j->op->C32};
                 J.plan = sap_plan(j->op);
                 J.eta = (const float4*)j->rin;
                 J.delta = (float4*)j->sapw;

@@ -68,11 +68,11 @@ template <typename R>
 Fields<R> fields_of(qxd_lattice* lat);
 template <>
 inline Fields<float> fields_of<float>(qxd_lattice* lat) {
-    return Fields<float>{nullptr, nullptr, lat->U32, lat->A32, lat->C32};
+    return Fields<float>{nullptr, lat->U32, lat->A32, lat->C32};
 }
 template <>
 inline Fields<double> fields_of<double>(qxd_lattice* lat) {
-    return Fields<double>{nullptr, nullptr, lat->W64, lat->C64};
+    return Fields<double>{nullptr, lat->W64, lat->C64};
 }
 template <typename R>
 const typename Fields<R>::cvec* clover_of(qxd_lattice* lat, bool inverse);

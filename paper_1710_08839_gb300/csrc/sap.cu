@@ -14,9 +14,9 @@
 // Starting from psi = 0, ncy cycles give psi = SAP(eta).
 // FP32, single lattice (k_sap_split): two threads per site pair, the block's
 // interior compound links W' = -1/2 z^qhat U (all three rows) and two block
-// fields in shared memory, the clover blocks read through L1, both from a
-// block-by-block copy of the operator. The residual
-// of a block is not recomputed from eta - D psi: the even-odd block solve
+// fields in shared memory, the clover rows of each thread in tensor memory,
+// both from a block-by-block copy of the operator (or from the native fields
+// where there is none). The residual of a block is not recomputed from eta - D psi: the even-odd block solve
 // leaves the block residual r_B - D_B delta equal to the MR residual rho on
 // the even sites and to zero on the odd sites (delta_o = M_oo^-1 (r_o - H_oe
 // delta_e) solves the odd rows exactly), and between two visits of a block
@@ -40,19 +40,20 @@ namespace qxd {
 
 namespace {
 
+using C64 = cplx<double>;
+
 constexpr int SAP_BS = 4;          // block extent in every direction
 constexpr int SAP_HALF = 128;      // sites of one parity per block
 constexpr int SAP_THREADS = 128;   // one thread per (even, odd) site pair
 
-// shared-memory half-spinor field of one block: R[24][128], conflict-free
-template <typename R>
+// shared-memory half-spinor field of one block: double[24][128], conflict-free
 struct SmemField {
-    R* a;
-    __device__ __forceinline__ void load(int slot, cplx<R> v[12]) const {
+    double* a;
+    __device__ __forceinline__ void load(int slot, C64 v[12]) const {
 #pragma unroll
         for (int i = 0; i < 12; ++i) v[i] = mk(a[(2 * i) * SAP_HALF + slot], a[(2 * i + 1) * SAP_HALF + slot]);
     }
-    __device__ __forceinline__ void store(int slot, const cplx<R> v[12]) const {
+    __device__ __forceinline__ void store(int slot, const C64 v[12]) const {
 #pragma unroll
         for (int i = 0; i < 12; ++i) {
             a[(2 * i) * SAP_HALF + slot] = v[i].re;
@@ -119,51 +120,49 @@ __device__ __forceinline__ int back_native(const Geom& g, const Site& t) {
 
 // hops of direction MU that stay inside the block (Dirichlet block boundary);
 // the neighbour spinor comes from shared memory (field of the other parity).
-// FP64 only: the links are compound (the charge and the factor -1/2 are in).
-template <typename R, int MU>
-__device__ __forceinline__ void block_dir(const Geom& g, const Fields<R>& f, const SmemField<R>& src, const Site& t,
-                                          cplx<R> acc[12]) {
+// The links are compound (the charge and the factor -1/2 are in).
+template <int MU>
+__device__ __forceinline__ void block_dir(const Geom& g, const Fields<double>& f, const SmemField& src, const Site& t,
+                                          C64 acc[12]) {
     constexpr int stride = MU == 0 ? 64 : MU == 1 ? 16 : MU == 2 ? 4 : 1;
-    cplx<R> v[12], h0[3], h1[3], g0[3], g1[3], u[3][3];
+    C64 v[12], h0[3], h1[3], g0[3], g1[3], u[3][3];
     if (t.l[MU] < SAP_BS - 1) {
         src.load((t.lidx + stride) >> 1, v);
-        project<R, MU, +1>(v, h0, h1);
+        project<double, MU, +1>(v, h0, h1);
         load_link(f.U, g.V, MU, t.s, u);
         su3_mul(u, h0, g0);
         su3_mul(u, h1, g1);
-        accumulate<R, MU, +1>(acc, g0, g1);
+        accumulate<double, MU, +1>(acc, g0, g1);
     }
     if (t.l[MU] > 0) {
         src.load((t.lidx - stride) >> 1, v);
-        project<R, MU, -1>(v, h0, h1);
+        project<double, MU, -1>(v, h0, h1);
         load_link(f.U, g.V, MU, back_native<MU>(g, t), u);
         su3_dag_mul(u, h0, g0);
         su3_dag_mul(u, h1, g1);
-        accumulate<R, MU, -1>(acc, g0, g1);
+        accumulate<double, MU, -1>(acc, g0, g1);
     }
 }
 
-template <typename R>
-__device__ __forceinline__ void block_hops(const Geom& g, const Fields<R>& f, const SmemField<R> src, const Site& t,
-                                           cplx<R> acc[12]) {
+__device__ __forceinline__ void block_hops(const Geom& g, const Fields<double>& f, const SmemField src, const Site& t,
+                                           C64 acc[12]) {
 #pragma unroll
-    for (int i = 0; i < 12; ++i) acc[i] = mk<R>(0, 0);
-    block_dir<R, 0>(g, f, src, t, acc);
-    block_dir<R, 1>(g, f, src, t, acc);
-    block_dir<R, 2>(g, f, src, t, acc);
-    block_dir<R, 3>(g, f, src, t, acc);
+    for (int i = 0; i < 12; ++i) acc[i] = mk(0.0, 0.0);
+    block_dir<0>(g, f, src, t, acc);
+    block_dir<1>(g, f, src, t, acc);
+    block_dir<2>(g, f, src, t, acc);
+    block_dir<3>(g, f, src, t, acc);
 }
 
 // r = eta - (D psi)(x), D over the whole lattice, at one site; out of line,
 // for the one-thread-per-pair kernel, which calls it twice
-template <typename R>
-__device__ __noinline__ void residual_at(const Geom& g, const Fields<R>& f, const typename Fields<R>::vec* eta,
-                                         const Site& t, bool psi_zero, cplx<R> r[12]) {
+__device__ __noinline__ void residual_at(const Geom& g, const Fields<double>& f, const double2* eta,
+                                         const Site& t, bool psi_zero, C64 r[12]) {
     load_spinor(eta, g.V, t.s, r);
     if (psi_zero) return;
     const int po = 1 - ((t.x[0] + t.x[1] + t.x[2] + t.x[3]) & 1);
-    cplx<R> acc[12], v[12];
-    dirac_hops<R, false>(g, f, f.psi, g.V, 0, R(0), t.x[0], t.x[1], t.x[2], t.x[3], t.s, po, acc);
+    C64 acc[12], v[12];
+    dirac_hops<double, false>(g, f, f.psi, g.V, 0, 0.0, t.x[0], t.x[1], t.x[2], t.x[3], t.s, po, acc);
     load_spinor(f.psi, g.V, t.s, v);
     clover_mul<false, true>(f.C, g.V, t.s, v, acc);
 #pragma unroll
@@ -207,17 +206,15 @@ __device__ __forceinline__ void block_sum3(R a, R b, R c, R* red, R out[3]) {
 //                      omega = <w,rho>/<w,w>, delta_e += omega rho,
 //                      rho -= omega w (even)             for k < nmr
 //   last step:         delta_o = M_oo^-1 (r_o - H_oe delta_e)     (odd)
-template <typename R>
 __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg, int bidx, int colour, int psi_zero,
-                                               const Fields<R>& f, const typename Fields<R>::cvec* __restrict__ Cinv,
-                                               const typename Fields<R>::vec* __restrict__ eta, int nmr) {
-    static_assert(sizeof(R) == 8, "FP64 block solve (compound links)");
+                                               const Fields<double>& f, const double* __restrict__ Cinv,
+                                               const double2* __restrict__ eta, int nmr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    R* sm = reinterpret_cast<R*>(smem_raw);
-    const SmemField<R> s_ro{sm};                    // r on the odd sites
-    const SmemField<R> s_rho{sm + 24 * SAP_HALF};   // MR residual (even)
-    const SmemField<R> s_t{sm + 48 * SAP_HALF};     // odd temporary / delta_e at the end
-    R* red = sm + 72 * SAP_HALF;                    // 3 * warps reduction slots
+    double* sm = reinterpret_cast<double*>(smem_raw);
+    const SmemField s_ro{sm};                   // r on the odd sites
+    const SmemField s_rho{sm + 24 * SAP_HALF};  // MR residual (even)
+    const SmemField s_t{sm + 48 * SAP_HALF};    // odd temporary / delta_e at the end
+    double* red = sm + 72 * SAP_HALF;           // 3 * warps reduction slots
 
     int org[4];
     block_origin(sg, bidx, colour, org);
@@ -228,26 +225,26 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
     const Site so = make_site(g, org, base + 1 - par0);
 
     // residual r = eta - D psi on both sites (one call site)
-    cplx<R> re[12], v[12], w[12], acc[12];
+    C64 re[12], v[12], w[12], acc[12];
 #pragma unroll 1
     for (int k = 0; k < 2; ++k) {
-        residual_at<R>(g, f, eta, k ? so : se, psi_zero, k ? v : re);
+        residual_at(g, f, eta, k ? so : se, psi_zero, k ? v : re);
     }
     s_ro.store(t, v);
     clover_mul(Cinv, g.Vh, so.s - g.Vh, v, w);  // t_o = M_oo^-1 r_o
     s_t.store(t, w);
     __syncthreads();
 
-    cplx<R> rho[12], de[12];
+    C64 rho[12], de[12];
 #pragma unroll
-    for (int i = 0; i < 12; ++i) de[i] = mk<R>(0, 0);
+    for (int i = 0; i < 12; ++i) de[i] = mk(0.0, 0.0);
     const int nsteps = 2 * nmr + 2;
 #pragma unroll 1
     for (int step = 0; step < nsteps; ++step) {
         const bool odd = (step & 1) != 0;   // steps 1, 3, ..., 2 nmr + 1 work on the odd sites
         const bool last = step == nsteps - 1;
         // odd steps read rho (or delta_e on the last step), even steps read t_o
-        block_hops<R>(g, f, odd ? (last ? s_t : s_rho) : s_t, odd ? so : se, acc);
+        block_hops(g, f, odd ? (last ? s_t : s_rho) : s_t, odd ? so : se, acc);
         // acc = H psi on the sites of this step's parity
         if (step == 0) {
 #pragma unroll
@@ -265,17 +262,17 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
 #pragma unroll
             for (int i = 0; i < 12; ++i) w[i] = -acc[i];
             clover_mul<false, true>(f.C, g.V, se.s, rho, w);
-            R a_re = 0, a_im = 0, b = 0;
+            double a_re = 0, a_im = 0, b = 0;
 #pragma unroll
             for (int i = 0; i < 12; ++i) {
                 a_re += w[i].re * rho[i].re + w[i].im * rho[i].im;
                 a_im += w[i].re * rho[i].im - w[i].im * rho[i].re;
                 b += w[i].re * w[i].re + w[i].im * w[i].im;
             }
-            R sums[3];
+            double sums[3];
             block_sum3(a_re, a_im, b, red, sums);
-            if (sums[2] > R(0)) {  // else rho = 0 on the whole block: nothing to add
-                const cplx<R> om = mk(sums[0] / sums[2], sums[1] / sums[2]);
+            if (sums[2] > 0.0) {  // else rho = 0 on the whole block: nothing to add
+                const C64 om = mk(sums[0] / sums[2], sums[1] / sums[2]);
 #pragma unroll
                 for (int i = 0; i < 12; ++i) {
                     de[i] = mad(om, rho[i], de[i]);
@@ -288,7 +285,7 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
         __syncthreads();
     }
     // psi_B += delta (w holds delta_o)
-    typename Fields<R>::vec* psi = const_cast<typename Fields<R>::vec*>(f.psi);
+    double2* psi = const_cast<double2*>(f.psi);
     if (psi_zero) {
         store_spinor(psi, g.V, se.s, de);
         store_spinor(psi, g.V, so.s, w);
@@ -304,11 +301,10 @@ __device__ __forceinline__ void sap_block_body(const Geom& g, const SapGeom& sg,
     }
 }
 
-template <typename R>
 __global__ void __launch_bounds__(SAP_THREADS, 2) k_sap_block(Geom g, SapGeom sg, int colour, int psi_zero,
-                                                              Fields<R> f, const typename Fields<R>::cvec* __restrict__ Cinv,
-                                                              const typename Fields<R>::vec* __restrict__ eta, int nmr) {
-    sap_block_body<R>(g, sg, blockIdx.x, colour, psi_zero, f, Cinv, eta, nmr);
+                                                              Fields<double> f, const double* __restrict__ Cinv,
+                                                              const double2* __restrict__ eta, int nmr) {
+    sap_block_body(g, sg, blockIdx.x, colour, psi_zero, f, Cinv, eta, nmr);
 }
 
 // ---------------------------------------------------------------------------
@@ -339,10 +335,7 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) k_sap_block(Geom g, SapGeom sg
 // The bodies of the block hops and of the crossing hops start with
 // __syncwarp(): left to itself the compiler lets the lanes that skipped a body
 // run ahead through the next ones, and warps took them twice (28 % more
-// shared-memory loads; 14.3 -> 13.1 ms). Measured and not kept: M_oo^-1 resident
-// in shared memory (17 of 18 float4 beside the links: 16.8 ms, the loads move to
-// the shared-memory pipe), L2 prefetch of the next block's data (14.7 where 14.3
-// without). Tensor memory has neither drawback: see below.
+// shared-memory loads; 14.3 -> 13.1 ms).
 // ---------------------------------------------------------------------------
 constexpr int SPLIT_THREADS = 256;
 constexpr unsigned FULL_MASK = 0xffffffffu;
@@ -587,11 +580,11 @@ __device__ __forceinline__ void split_hops(const SplitLinks& bl, const float2* s
 // in flight, L2: DRAM bytes of a launch on 48x48x24x24 sites 929 -> 606 MB, waits
 // for global memory per instruction 2.0 -> 0.8, and with rows chosen and
 // conjugated once 9 % fewer instructions; one application on 64x64x32x32 sites
-// 12.52 -> 11.08 ms, six right-hand sides on 32x32x16x16 4.73 -> 4.24 ms.
-// Measured and not kept: r_o in the spare columns too (11.29), the rows loaded
-// after the residual is formed (11.28), the loads of tm_load28 issued before the
-// shuffles (11.16), the two blocks' rows interleaved and multiplied by packed
-// FP32 pairs (11.60).
+// 12.52 -> 11.08 ms, six right-hand sides on 32x32x16x16 4.73 -> 4.24 ms. Filling
+// the rows costs one pass and pays from the second MR step on: with nmr = 1, 2,
+// 3, 5, 8 an application takes 7.80, 7.91, 8.71, 11.08, 14.84 ms, and 6.82, 8.31,
+// 9.66, 12.58, 17.08 with the blocks read from memory in every step. There is no
+// second form for nmr = 1: the solvers take 5 steps (the deflation's smoothing 4).
 constexpr int TM_BLOCK = 32;             // columns of one 6x6 block's rows (28 used)
 constexpr int TM_COLS = 2 * 4 * TM_BLOCK;
 
@@ -1093,8 +1086,8 @@ int launch_sap_block64(qxd_lattice* lat, const SapGeom& sg, int cy, int colour, 
                        const double* Cinv, const double2* eta, int nmr, cudaStream_t st) {
     const size_t smem = sap_smem_bytes<double>();
     const int psi_zero = (cy == 0 && colour == 0) ? 1 : 0;
-    QXD_CUDA(cudaFuncSetAttribute(k_sap_block<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_sap_block<double><<<sg.nhalf, SAP_THREADS, smem, st>>>(lat->g, sg, colour, psi_zero, f, Cinv, eta, nmr);
+    QXD_CUDA(cudaFuncSetAttribute(k_sap_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_sap_block<<<sg.nhalf, SAP_THREADS, smem, st>>>(lat->g, sg, colour, psi_zero, f, Cinv, eta, nmr);
     QXD_LAUNCHED("k_sap_block");
     return QXD_OK;
 }
@@ -1106,7 +1099,7 @@ int split_cycles(qxd_lattice* lat, const SapGeom& sg, const SplitRhsList& rl, in
     const int rc = split_attrs(k_sap_split<QNZ, COPY>, smem);
     if (rc) return rc;
     const SapPlan plan = sap_plan(lat);
-    const Fields<float> f{nullptr, nullptr, lat->U32, lat->A32, lat->C32};
+    const Fields<float> f{nullptr, lat->U32, lat->A32, lat->C32};
     for (int cy = 0; cy < ncy; ++cy)
         for (int colour = 0; colour < 2; ++colour) {
             k_sap_split<QNZ, COPY><<<sg.nhalf * rl.n, SPLIT_THREADS, smem, st>>>(lat->g, sg, colour, f, plan, rl,
@@ -1180,7 +1173,7 @@ int launch_sap_plan(qxd_lattice* lat, cudaStream_t st) {
         }
     }
     if (!lat->sap_plan) return QXD_OK;
-    const Fields<float> f{nullptr, nullptr, lat->U32, lat->A32, lat->C32};
+    const Fields<float> f{nullptr, lat->U32, lat->A32, lat->C32};
     float4* clover = lat->sap_plan + (size_t)sg.nblk * PLAN_LINK_F4;
     if (lat->qhat != 0)
         k_sap_plan<true><<<sg.nblk, SPLIT_THREADS, 0, st>>>(lat->g, sg, f, lat->Cinv32, lat->sap_plan, clover,
@@ -1236,7 +1229,7 @@ int sap_apply(qxd_lattice* lat, SapWork& w, void* out, const void* in, int ncy, 
         // psi starts at zero; the first half-cycle writes the blocks of colour 0
         // without reading psi, and the blocks of colour 1 must read zeros there
         QXD_CUDA(cudaMemsetAsync(out, 0, (size_t)g.V * 24 * sizeof(R), st));
-        const Fields<double> f{(const double2*)out, nullptr, lat->W64, lat->C64};
+        const Fields<double> f{(const double2*)out, lat->W64, lat->C64};
         for (int cy = 0; cy < ncy; ++cy)
             for (int colour = 0; colour < 2; ++colour) {
                 const int rc = launch_sap_block64(lat, w.sg, cy, colour, f, lat->Cinv64, (const double2*)in, nmr, st);
