@@ -19,6 +19,7 @@ int fail(int code, const std::string& msg) {
 }
 
 int cuda_fail(cudaError_t e, const char* what) {
+    cudaGetLastError();  // reported here: the check after the next launch must not find it (a refused allocation) again
     g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? QXD_ERR_OOM : QXD_ERR_CUDA;
 }
