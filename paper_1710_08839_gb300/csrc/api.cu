@@ -91,11 +91,18 @@ static void free_all(qxd_lattice* L) {
 
 int ensure_scratch(qxd_lattice* L) {
     if (L->scratch_in) return QXD_OK;
-    size_t nat = (size_t)L->g.V * SPINOR_D2 * sizeof(double2);
-    int rc;
-    if ((rc = dalloc((char**)&L->scratch_in, nat, "cudaMalloc(scratch)"))) return rc;
-    if ((rc = dalloc((char**)&L->scratch_out, nat, "cudaMalloc(scratch)"))) return rc;
-    if ((rc = dalloc((char**)&L->scratch_lex, nat, "cudaMalloc(scratch)"))) return rc;
+    const size_t nat = (size_t)L->g.V * SPINOR_D2 * sizeof(double2);
+    void* p[3] = {};
+    for (int i = 0; i < 3; ++i) {
+        const int rc = dalloc((char**)&p[i], nat, "cudaMalloc(scratch)");
+        if (rc) {  // all three or none: a later call must not find the first alone
+            while (i--) cudaFree(p[i]);
+            return rc;
+        }
+    }
+    L->scratch_in = p[0];
+    L->scratch_out = p[1];
+    L->scratch_lex = p[2];
     return QXD_OK;
 }
 
