@@ -51,6 +51,7 @@ struct DevicePool {
         if (held + bytes > cap) reclaim(bytes);
         cudaError_t e = cudaMalloc(p, bytes);
         if (e != cudaSuccess) {
+            cudaGetLastError();  // not an error of the next launch if the second attempt succeeds
             trim();
             e = cudaMalloc(p, bytes);
         }

@@ -1,0 +1,53 @@
+"""On a full device the engine frees the cached blocks of finished requests and
+goes on: the allocation it tried first is no error of the request."""
+import pytest
+import torch
+
+from qxd_cases import Case
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__ as ge
+    ge.build()
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+
+
+def test_request_after_trimming_the_cache():
+    from paper_1710_08839_gb300 import qxd
+    small, large = Case(16, 16, 16, 16, qhat=2, device="cuda"), Case(24, 16, 16, 16, qhat=2, device="cuda")
+    ops = {}
+    for c in (small, large):
+        lat = c.lattice()
+        b = c.psi.to(torch.complex128)
+        ops[c.T] = (lat, b, torch.empty_like(b), torch.empty_like(b))
+    e = qxd.Engine(64 << 30)
+
+    def solve(T, k):
+        lat, b = ops[T][:2]
+        rid = e.submit(lat, ops[T][k], b, tol=1e-10, nkv=6)
+        e.run()
+        assert e.poll(rid)[1]["status"] == qxd.QXD_OK
+        e.forget(rid)
+    solve(small.T, 2)  # kernels loaded, launch shapes timed; its blocks cached
+    solve(large.T, 2)  # other block sizes, cached as well
+    e.close()
+    e = qxd.Engine(64 << 30)
+    solve(large.T, 3)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    # less than one field of the small lattice is left beside the cached blocks
+    taken = torch.empty(torch.cuda.mem_get_info()[0] - (8 << 20), dtype=torch.uint8, device="cuda")
+    held = e.stats()["bytes_held"]
+    solve(small.T, 3)
+    assert e.stats()["bytes_held"] < held
+    del taken
+    torch.cuda.synchronize()
+    for T in ops:
+        lat, b, x, y = ops[T]
+        assert torch.equal(x, y)
+        lat.close()
+    e.close()
