@@ -399,10 +399,12 @@ int reduce_finish(Reducer& red, int nc, cudaStream_t st) {
 
 int Reducer::init() {
     if (partials) return QXD_OK;
-    QXD_CUDA(cudaMalloc(&partials, sizeof(double) * RED_BLOCKS * 2 * BLAS_KMAX));
-    QXD_CUDA(cudaMallocHost(&h_res, sizeof(double) * 2 * BLAS_KMAX));
-    QXD_CUDA(cudaHostGetDevicePointer((void**)&d_res, h_res, 0));
-    return QXD_OK;
+    cudaError_t e = cudaMalloc(&partials, sizeof(double) * RED_BLOCKS * 2 * BLAS_KMAX);
+    if (e == cudaSuccess) e = cudaMallocHost(&h_res, sizeof(double) * 2 * BLAS_KMAX);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&d_res, h_res, 0);
+    if (e == cudaSuccess) return QXD_OK;
+    release();  // all or none: a later call must not take a part for the whole
+    return cuda_fail(e, "reduction work space");
 }
 
 void Reducer::release() {

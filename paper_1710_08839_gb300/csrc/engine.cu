@@ -365,9 +365,12 @@ struct Engine {
                     cudaStreamSynchronize(st);
                     sap_graphs.clear();  // they hold the old table address
                     cudaFree(d_sap);
+                    d_sap = nullptr;  // and stays so, with its size, if there is no memory for the new one
+                    d_sap_cap = 0;
                 }
-                d_sap_cap = (int)sj.size() * 2;
-                QXD_CUDA(cudaMalloc(&d_sap, sizeof(SapJob) * d_sap_cap));
+                const int cap = (int)sj.size() * 2;
+                QXD_CUDA(cudaMalloc(&d_sap, sizeof(SapJob) * cap));
+                d_sap_cap = cap;
             }
             // all SAP jobs of a step share ncy and nmr of their own params:
             // group by (ncy, nmr)
