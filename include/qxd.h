@@ -340,8 +340,10 @@ int qxd_Dw_batch(int n, qxd_lattice* const* lats, void* const* out, const void* 
  * active requests stays within hbm_budget_bytes (a request larger than the
  * budget runs alone) and their number within max_active. Each request is
  * charged its largest footprint at admission: four FP64 fields, one FP32
- * residual and params->nkv FP32 Krylov pairs, 24 V (4 * 8 + (1 + 2 nkv) * 4)
- * bytes on a lattice of V sites. Work vectors come from the engine's caching
+ * residual, params->nkv FP32 Krylov pairs and the Schwarz work fields, 24 V (4 *
+ * 8 + (1 + 2 nkv) * 4 + 6) bytes on a lattice of V sites. The operators' own
+ * memory (fields, clover term, the copy of qxd_sw_build) is the lattices', not
+ * charged here: the engine allocates none of it. Work vectors come from the engine's caching
  * device allocator, which keeps the bytes it holds (in use plus cached)
  * within the budget by releasing cached blocks before it allocates more. A
  * request whose work vectors cannot be allocated fails alone (its status is

@@ -162,7 +162,9 @@ namespace {
 
 bool capturing(cudaStream_t st) {
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(st, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    cudaGetLastError();  // the legacy stream beside a capture elsewhere: nothing can be timed there either
+    return true;
 }
 
 int dirac_full(qxd_lattice* lat, void* out, const void* in, int prec, bool lex, cudaStream_t st) {
