@@ -41,10 +41,13 @@ def test_request_after_trimming_the_cache():
     torch.cuda.empty_cache()
     # less than one field of the small lattice is left beside the cached blocks
     taken = torch.empty(torch.cuda.mem_get_info()[0] - (8 << 20), dtype=torch.uint8, device="cuda")
-    held = e.stats()["bytes_held"]
-    solve(small.T, 3)
-    assert e.stats()["bytes_held"] < held
-    del taken
+    try:
+        held = e.stats()["bytes_held"]
+        solve(small.T, 3)
+        assert e.stats()["bytes_held"] < held
+    finally:
+        del taken
+        torch.cuda.empty_cache()
     torch.cuda.synchronize()
     for T in ops:
         lat, b, x, y = ops[T]

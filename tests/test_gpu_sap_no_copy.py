@@ -158,13 +158,15 @@ def test_the_copy_leaves_half_of_the_memory():
     torch.cuda.empty_cache()
     free, total = torch.cuda.mem_get_info()
     taken = torch.empty(max(0, free - total // 2 + (64 << 20)), dtype=torch.uint8, device="cuda")
-    lat = c.lattice()
-    lat.set_sap_copy(1)
-    y, z = torch.empty_like(x), torch.empty_like(x)
-    lat.sap(y, x, ncy=2, nmr=2)
-    torch.cuda.synchronize()
-    del taken
-    torch.cuda.empty_cache()
+    try:
+        lat = c.lattice()
+        lat.set_sap_copy(1)
+        y, z = torch.empty_like(x), torch.empty_like(x)
+        lat.sap(y, x, ncy=2, nmr=2)
+        torch.cuda.synchronize()
+    finally:
+        del taken
+        torch.cuda.empty_cache()
     lat.sw_build()
     with pytest.raises(qxd.QxdError):
         lat.set_sap_copy(1)

@@ -30,13 +30,15 @@ def test_scratch_is_all_or_nothing():
     torch.cuda.empty_cache()
     field = lat.V * 24 * 8
     taken = torch.empty(torch.cuda.mem_get_info()[0] - 2 * field - field // 2, dtype=torch.uint8, device="cuda")
-    for _ in range(3):
-        for call in (lat.Dw, lat.Dhat, lat.eo_prepare):
-            with pytest.raises(qxd.QxdError) as e:
-                call(y, x)
-            assert e.value.code == qxd.QXD_ERR_OOM
-    del taken
-    torch.cuda.empty_cache()
+    try:
+        for _ in range(3):
+            for call in (lat.Dw, lat.Dhat, lat.eo_prepare):
+                with pytest.raises(qxd.QxdError) as e:
+                    call(y, x)
+                assert e.value.code == qxd.QXD_ERR_OOM
+    finally:
+        del taken
+        torch.cuda.empty_cache()
     lat.Dw(y, x)
     assert torch.equal(y, want)
     lat.close()
